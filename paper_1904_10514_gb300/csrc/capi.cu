@@ -312,7 +312,7 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
         // per-order operators; without room for them the plan keeps the sweeps
         std::vector<int64_t> off((size_t)(L + 1) * 2 + 1, 0);
         std::vector<int> tiles;
-        const int rows = hpx::fused_tile_rows(g.B);
+        const int rows = hpx::fused_tile_rows(fp64);
         for (int m = 0; m <= L; ++m)
             for (int c = 0; c < 2; ++c) {
                 const int n = hpx::chain_len(m, c, L);
@@ -356,8 +356,9 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
             double* D64 = (double*)t.D;
             hpx::cplx<double>* sk64 = (hpx::cplx<double>*)t.skew;
             if (!fp64) { D64 = up.vec(tb.D); sk64 = (hpx::cplx<double>*)up.vec(tb.skew); }
-            int rc = up.ok ? (fp64 ? hpx::build_fused<double>(P, D64, sk64, nullptr, P->fusedM, P->use_tc)
-                                   : hpx::build_fused<float>(P, D64, sk64, nullptr, P->fusedM, P->use_tc))
+            const int form = P->use_tc ? 1 : !fp64 && g.B <= 8 ? 2 : 0;
+            int rc = up.ok ? (fp64 ? hpx::build_fused<double>(P, D64, sk64, nullptr, P->fusedM, form)
+                                   : hpx::build_fused<float>(P, D64, sk64, nullptr, P->fusedM, form))
                            : -1;
             if (rc == 0 && P->use_tc) rc = hpx::prepare_fused_tc(P);
             // synthesis operators R_{m,c} Es (row-major), when asked for and room allows
@@ -368,8 +369,8 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
                 P->bytes += (int64_t)sBytes;
                 cudaMemset(P->synM, 0, sBytes);
                 double* Es64 = fp64 ? (double*)t.Es : up.vec(EsHost);
-                rc = up.ok ? (fp64 ? hpx::build_fused<double>(P, Es64, sk64, nullptr, P->synM, false)
-                                   : hpx::build_fused<float>(P, Es64, sk64, nullptr, P->synM, false))
+                rc = up.ok ? (fp64 ? hpx::build_fused<double>(P, Es64, sk64, nullptr, P->synM, 0)
+                                   : hpx::build_fused<float>(P, Es64, sk64, nullptr, P->synM, 0))
                            : -1;
                 if (!fp64 && Es64) { cudaFree(Es64); P->bytes -= (int64_t)(EsHost.size() * 8); }
                 // FP32 plans on the tensor cores apply them there too

@@ -18,6 +18,12 @@
 
 namespace hpx {
 
+// Element (row i, column k) of a chain of n rows in the layout of fused_quad_kernel.
+__host__ __device__ inline int64_t quad_elem(int n, int ldm, int i, int k) {
+    const int g0 = i & ~31, cnt = n - g0 < 32 ? n - g0 : 32;
+    return (int64_t)g0 * ldm + (int64_t)(k >> 2) * 4 * cnt + 4 * (i - g0) + (k & 3);
+}
+
 // ---------------------------------------------------------------- build (FP64)
 // One warp per (m, chain c, group of 32 complex columns); complex column j holds
 // the real columns 2j and 2j+1 of D.  The chain of each lane lives in `scratch`.
@@ -29,7 +35,7 @@ __global__ void __launch_bounds__(64) build_fused_kernel(const double* __restric
                                                          int ldm, int L, int m_lo, int m_cnt, int ngroups,
                                                          cplx<double>* __restrict__ scratch,
                                                          const int64_t* __restrict__ tcOff,
-                                                         const int* __restrict__ tcFirst) {
+                                                         const int* __restrict__ tcFirst, bool quad) {
     constexpr int KMAX = 16;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -85,6 +91,14 @@ __global__ void __launch_bounds__(64) build_fused_kernel(const double* __restric
         return;
     }
     T* out = Mout + moff[(size_t)m * 2 + c] * ldm;
+    if (quad) {   // groups of 32 rows, four k side by side (fused_quad_kernel)
+        for (int i = 0; i < n; ++i) {
+            const cplx<double> v = chain[(int64_t)i * ldc];
+            out[quad_elem(n, ldm, i, 2 * j)] = (T)v.r;
+            if (2 * j + 1 < P2) out[quad_elem(n, ldm, i, 2 * j + 1)] = (T)v.i;
+        }
+        return;
+    }
     for (int i = 0; i < n; ++i) {
         const cplx<double> v = chain[(int64_t)i * ldc];
         out[(size_t)i * ldm + 2 * j] = (T)v.r;
@@ -93,6 +107,9 @@ __global__ void __launch_bounds__(64) build_fused_kernel(const double* __restric
 }
 
 // ---------------------------------------------------------------- apply
+namespace {
+constexpr int kFusedRows = 64;   // rows per block of fused_rows_kernel
+}  // namespace
 
 // Block = one (m, c, tile of 8*TR rows) x 2*TC maps; TR*TC threads, each 8 rows x 2 maps.
 // M rows are padded to ldm (a multiple of 4, zero filled) so that they load as
@@ -177,6 +194,194 @@ __global__ void __launch_bounds__(TR* TC) fused_apply_kernel(const T* __restrict
         for (int r = 0; r < 8; ++r) {
             const int i = i0 + tr * 8 + r;
             if (i < nrows) out[2 * i] = mk<T>(accr[r][q], acci[r][q]);
+        }
+    }
+}
+
+// FP32 batches of at most 8 maps.  The operator is stored for it at plan time in
+// groups of 32 rows of one chain (the last group of a chain has fewer, cnt), four k
+// of all rows of a group side by side (quad_elem), so that lane = row reads 16 bytes
+// of 512 contiguous ones per four k and every coefficient is one thread's sum over k
+// in ascending order (the order of the 32-map form below, so a map's coefficients
+// do not depend on the batch).  b sits in shared memory, read as broadcasts.  The
+// bound is the operator's stream, 4 (nside + 1) n_alm bytes per call: blocks of four
+// warps (128 rows) with eight loads in flight per lane.  Before, row-major M went
+// through shared memory in tiles of 512 rows x 2 maps with 64 threads: analysis and
+// C_l of one map at Nside 256 took 297 us, now 98; five at Nside 128 79.9, now 64.9.
+template <int NB>
+__global__ void __launch_bounds__(128) fused_quad_kernel(const float* __restrict__ M, const int64_t* __restrict__ moff,
+                                                         const int* __restrict__ tiles,
+                                                         const cplx<float>* __restrict__ bvec,
+                                                         cplx<float>* __restrict__ alm, int P2, int ldm, int p, int L,
+                                                         int B, int64_t nalm) {
+    constexpr int NC = 2 * NB;
+    extern __shared__ __align__(16) float bq[];   // [ldm][NC]: k, then (map, part)
+    const int m = tiles[3 * blockIdx.x], c = tiles[3 * blockIdx.x + 1], i0 = tiles[3 * blockIdx.x + 2];
+    const int par = ((m & 1) + c) & 1;
+    const int nrows = chain_len(m, c, L);
+    const int b0 = blockIdx.y * NB;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        const cplx<float>* col = bvec + (((int64_t)min(b0 + q, B - 1) * (p + 1) + m) * 2 + par) * P2;
+        for (int k = threadIdx.x; k < ldm; k += 128)
+            reinterpret_cast<cplx<float>*>(bq)[k * NB + q] =
+                b0 + q < B && k < P2 ? col[k] : mk<float>(0.f, 0.f);
+    }
+    __syncthreads();
+    const int g0 = i0 + 32 * warp;   // this warp's group of rows
+    const int cnt = min(32, nrows - g0);
+    if (lane >= cnt) return;
+    const float4* A = reinterpret_cast<const float4*>(M + (moff[(size_t)m * 2 + c] + g0) * ldm) + lane;
+    float acc[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) acc[q] = 0.f;
+    auto step = [&](const float4& a4, int k4) {
+        const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+        const float4* x4 = reinterpret_cast<const float4*>(bq + k4 * 4 * NC);
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {   // 4 NC values: k = h / (NC / 4) when NC >= 4
+            const float4 v = x4[h];
+            const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int id = 4 * h + e;
+                acc[id % NC] = fmaf(a[id / NC], x[e], acc[id % NC]);
+            }
+        }
+    };
+    const int n4 = ldm >> 2;
+    int k4 = 0;
+    for (; k4 + 8 <= n4; k4 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldg(A + (int64_t)(k4 + u) * cnt);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) step(v[u], k4 + u);
+    }
+    for (; k4 < n4; ++k4) step(__ldg(A + (int64_t)k4 * cnt), k4);
+    const int64_t at = (int64_t)m * (2 * L + 1 - m) / 2 + m + c + 2 * (int64_t)(g0 + lane);
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+        if (b0 + q < B) alm[(int64_t)(b0 + q) * nalm + at] = mk<float>(acc[2 * q], acc[2 * q + 1]);
+}
+
+// FP64 batches (and the FP32 equal-weight analysis of at most 8 maps, on row-major
+// operators): a matrix-vector form.  A block takes 64 rows of one (m, c) and NB
+// maps; a warp takes R rows at a time, its lanes split the k of a row (one 16-byte
+// load per lane and row: 512 contiguous bytes of the operator per warp load, R loads
+// in flight per lane), b sits in shared memory as 2 NB real columns, and the R x 2 NB
+// partial sums of the lanes are combined by a butterfly that leaves each lane with
+// one result.  Every sum has the same order whatever NB, R and the map's position
+// are: lane l adds k = VA l + CH j + a for j, a ascending, the lanes combine over
+// lane distance 16, 8, 4, 2, 1, then the last term k = nside.
+// The bound is the FP64 pipe (2 FMA per SM and clock on this GPU), so no lane
+// computes for a map or row that is not there beyond the tail of a group.  One map,
+// Nside 512: analysis and C_l 5.11 -> 1.87 ms (this kernel about 4.2 -> 1.0, FMA floor
+// 0.87); Nside 16: 107 -> 80 us.
+// Tiles of 512 rows x 2 maps, always computed in full, before.
+template <class T, int NB, int R>
+__global__ void __launch_bounds__(256) fused_rows_kernel(const T* __restrict__ M, const int64_t* __restrict__ moff,
+                                                         const int* __restrict__ tiles,
+                                                         const cplx<T>* __restrict__ bvec, T* __restrict__ alm,
+                                                         int P2, int ldm, int p, int L, int B, int64_t nalm) {
+    constexpr int VA = 16 / sizeof(T), CH = 32 * VA;   // k per lane and load, k per warp load
+    constexpr int NC = 2 * NB;
+    constexpr int V = R * NC <= 16 ? 16 : R * NC <= 32 ? 32 : 64;   // sums per lane, rounded up
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* bs = reinterpret_cast<T*>(smem_raw);   // [NC][KP], then the NC values at k = K
+    const int K = P2 - 1;                     // = nside; the term k = K is added last
+    const int KP = (K + CH - 1) / CH * CH;
+    T* bl = bs + NC * KP;
+    const int m = tiles[3 * blockIdx.x], c = tiles[3 * blockIdx.x + 1];
+    const int i0 = tiles[3 * blockIdx.x + 2] + kFusedRows * blockIdx.z;
+    const int par = ((m & 1) + c) & 1;
+    const int nrows = chain_len(m, c, L);
+    if (i0 >= nrows) return;
+    const int b0 = blockIdx.y * NB;
+    const T* A = M + moff[(size_t)m * 2 + c] * ldm;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        const cplx<T>* col = bvec + (((int64_t)min(b0 + q, B - 1) * (p + 1) + m) * 2 + par) * P2;
+        const bool have = b0 + q < B;
+        for (int k = threadIdx.x; k < KP; k += 256) {
+            const cplx<T> v = have && k < K ? col[k] : mk<T>(T(0), T(0));
+            bs[(2 * q) * KP + k] = v.r;
+            bs[(2 * q + 1) * KP + k] = v.i;
+        }
+        if (threadIdx.x == 0) {
+            const cplx<T> v = have ? col[K] : mk<T>(T(0), T(0));
+            bl[2 * q] = v.r;
+            bl[2 * q + 1] = v.i;
+        }
+    }
+    __syncthreads();
+    const int iend = min(i0 + kFusedRows, nrows);
+    for (int r0 = i0 + warp * R; r0 < iend; r0 += 8 * R) {
+        T acc[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = T(0);
+        const T* row[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) row[r] = A + (int64_t)min(r0 + r, nrows - 1) * ldm;
+#pragma unroll 2
+        for (int k = lane * VA; k < K; k += CH) {   // ldm >= k + VA: rows are padded to 4
+            T mv[R][VA];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if constexpr (sizeof(T) == 4) {
+                    const float4 q4 = __ldg(reinterpret_cast<const float4*>(row[r] + k));
+                    mv[r][0] = q4.x; mv[r][1] = q4.y; mv[r][2] = q4.z; mv[r][3] = q4.w;
+                } else {
+                    const double2 q2 = __ldg(reinterpret_cast<const double2*>(row[r] + k));
+                    mv[r][0] = q2.x; mv[r][1] = q2.y;
+                }
+            }
+#pragma unroll
+            for (int col = 0; col < NC; ++col) {
+                T x[VA];
+                if constexpr (sizeof(T) == 4) {
+                    const float4 q4 = *reinterpret_cast<const float4*>(bs + col * KP + k);
+                    x[0] = q4.x; x[1] = q4.y; x[2] = q4.z; x[3] = q4.w;
+                } else {
+                    const double2 q2 = *reinterpret_cast<const double2*>(bs + col * KP + k);
+                    x[0] = q2.x; x[1] = q2.y;
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int a = 0; a < VA; ++a) acc[r * NC + col] = fma(mv[r][a], x[a], acc[r * NC + col]);
+            }
+        }
+        // butterfly: each level halves the sums a lane holds, then plain adds
+        int n = V;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const bool up = (lane & off) != 0;
+            if (n > 1) {
+                n >>= 1;
+#pragma unroll
+                for (int v = 0; v < V / 2; ++v)
+                    if (v < n) {
+                        const T give = up ? acc[v] : acc[v + n];
+                        acc[v] = (up ? acc[v + n] : acc[v]) + __shfl_xor_sync(0xffffffffu, give, off);
+                    }
+            } else {
+                acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], off);
+            }
+        }
+        constexpr int PER = V > 32 ? V / 32 : 1;
+        const int first = V >= 32 ? lane * PER : lane >> 1;   // V = 16: two lanes hold each sum
+#pragma unroll
+        for (int v = 0; v < PER; ++v) {
+            const int id = first + v, r = id / NC, col = id - r * NC;
+            const int i = r0 + r, b = b0 + (col >> 1);
+            if (r < R && i < iend && b < B && (V >= 32 || (lane & 1) == 0)) {
+                const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2 + m + c;
+                alm[((int64_t)b * nalm + base + 2 * i) * 2 + (col & 1)] =
+                    fma(A[(int64_t)i * ldm + K], bl[col], acc[v]);
+            }
         }
     }
 }
@@ -275,38 +480,64 @@ void launch_synth_apply(const hpx_plan_s* P, const T* alm, cudaStream_t s) {
 template void launch_synth_apply<float>(const hpx_plan_s*, const float*, cudaStream_t);
 template void launch_synth_apply<double>(const hpx_plan_s*, const double*, cudaStream_t);
 
-// Rows per block of the apply kernel for a batch of B maps (the plan builds its
-// tile list with this).
-int fused_tile_rows(int B) { return B > 8 ? 128 : (B > 2 ? 256 : 512); }
+// Rows per block of the apply kernels (the plan builds its tile list with this).
+int fused_tile_rows(bool fp64) { return fp64 ? kFusedRows : 128; }
 
 template <class T>
 void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Mrows) {
     const auto& g = P->g;
     const int ldm = P->fused_ldm;
     const T* M = (const T*)(Mrows ? Mrows : P->fusedM);
-    if (g.B > 8) {
-        dim3 grid(P->fused_ntiles, (g.B + 31) / 32);
-        fused_apply_kernel<T, 16, 16><<<grid, 256, 0, s>>>(M, P->fusedOff, P->fusedTiles,
-                                                           (const cplx<T>*)P->bvec, (cplx<T>*)alm, g.P2, ldm,
-                                                           g.p, g.L, g.B, g.nalm);
-    } else if (g.B > 2) {
-        dim3 grid(P->fused_ntiles, (g.B + 7) / 8);
-        fused_apply_kernel<T, 32, 4><<<grid, 128, 0, s>>>(M, P->fusedOff, P->fusedTiles,
-                                                          (const cplx<T>*)P->bvec, (cplx<T>*)alm, g.P2, ldm,
-                                                          g.p, g.L, g.B, g.nalm);
-    } else {
-        dim3 grid(P->fused_ntiles, (g.B + 1) / 2);
-        fused_apply_kernel<T, 64, 1><<<grid, 64, 0, s>>>(M, P->fusedOff, P->fusedTiles,
-                                                         (const cplx<T>*)P->bvec, (cplx<T>*)alm, g.P2, ldm,
-                                                         g.p, g.L, g.B, g.nalm);
+    if constexpr (sizeof(T) == 4) {
+        if (g.B > 8) {
+            dim3 grid(P->fused_ntiles, (g.B + 31) / 32);
+            fused_apply_kernel<T, 16, 16><<<grid, 256, 0, s>>>(M, P->fusedOff, P->fusedTiles,
+                                                               (const cplx<T>*)P->bvec, (cplx<T>*)alm, g.P2, ldm,
+                                                               g.p, g.L, g.B, g.nalm);
+            return;
+        }
     }
+    if constexpr (sizeof(T) == 4) {
+        if (!Mrows) {
+            auto run = [&](auto kern, int NB) {   // each operator read once: all maps in one block
+                const size_t smem = (size_t)2 * NB * ldm * sizeof(float);
+                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                kern<<<P->fused_ntiles, 128, smem, s>>>(M, P->fusedOff, P->fusedTiles, (const cplx<float>*)P->bvec,
+                                                        (cplx<float>*)alm, g.P2, ldm, g.p, g.L, g.B, g.nalm);
+            };
+            if (g.B == 1) run(fused_quad_kernel<1>, 1);
+            else if (g.B == 2) run(fused_quad_kernel<2>, 2);
+            else if (g.B <= 4) run(fused_quad_kernel<4>, 4);
+            else run(fused_quad_kernel<8>, 8);
+            return;
+        }
+    }
+    // maps per block: FP32 reads each operator once (up to 8 maps); FP64 computes for
+    // as few absent maps as possible (groups of at most 4, of equal size)
+    const int nb = sizeof(T) == 4 ? (g.B > 4 ? 8 : g.B > 2 ? 4 : g.B)
+                                  : (g.B + (g.B + 3) / 4 - 1) / ((g.B + 3) / 4);
+    constexpr int per = sizeof(T) == 4 ? 2 : 1;   // blocks of 64 rows per tile of the plan's list
+    auto run = [&](auto kern, int NB) {
+        constexpr int CH = 32 * 16 / sizeof(T);
+        const size_t smem = (size_t)2 * NB * ((g.P2 - 1 + CH - 1) / CH * CH + 1) * sizeof(T);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        dim3 grid(P->fused_ntiles, (g.B + NB - 1) / NB, per);
+        kern<<<grid, 256, smem, s>>>(M, P->fusedOff, P->fusedTiles, (const cplx<T>*)P->bvec, alm, g.P2, ldm, g.p,
+                                     g.L, g.B, g.nalm);
+    };
+    if (nb == 1) run(fused_rows_kernel<T, 1, 8>, 1);
+    else if (nb == 2) run(fused_rows_kernel<T, 2, 8>, 2);
+    else if (nb == 4) run(fused_rows_kernel<T, 4, 4>, 4);
+    else if constexpr (sizeof(T) == 4) run(fused_rows_kernel<T, 8, 4>, 8);
+    else run(fused_rows_kernel<T, 3, 4>, 3);
 }
 
 // Builds the per-order operators of a plan (called once by hpx_plan_ex).
-// D64 / skew64 are FP64 device copies of D and of the skewed sweep angles.
+// D64 / skew64 are FP64 device copies of D and of the skewed sweep angles.  form: 0
+// row-major, 1 the tensor-core tiles, 2 the groups of fused_quad_kernel.
 template <class T>
 int build_fused(hpx_plan_s* P, const double* D64, const cplx<double>* skew64, cudaStream_t s, void* out,
-                bool tiled) {
+                int form) {
     const auto& g = P->g;
     const int ncplx = (g.P2 + 1) / 2;
     const int ngroups = (ncplx + 31) / 32;
@@ -320,7 +551,7 @@ int build_fused(hpx_plan_s* P, const double* D64, const cplx<double>* skew64, cu
         const int blocks = (nitems * 32 + 63) / 64;
         build_fused_kernel<T><<<blocks, 64, 0, s>>>(D64, (T*)out, P->fusedOff, P->t.skOff, skew64, P->t.nq,
                                                     g.P2, P->fused_ldm, g.L, m_lo, m_cnt, ngroups, scratch,
-                                                    tiled ? P->tcOff : nullptr, P->tcFirst);
+                                                    form == 1 ? P->tcOff : nullptr, P->tcFirst, form == 2);
     }
     const cudaError_t e = cudaStreamSynchronize(s);
     cudaFree(scratch);
@@ -329,7 +560,7 @@ int build_fused(hpx_plan_s* P, const double* D64, const cplx<double>* skew64, cu
 
 template void launch_fused<float>(const hpx_plan_s*, float*, cudaStream_t, const void*);
 template void launch_fused<double>(const hpx_plan_s*, double*, cudaStream_t, const void*);
-template int build_fused<float>(hpx_plan_s*, const double*, const cplx<double>*, cudaStream_t, void*, bool);
-template int build_fused<double>(hpx_plan_s*, const double*, const cplx<double>*, cudaStream_t, void*, bool);
+template int build_fused<float>(hpx_plan_s*, const double*, const cplx<double>*, cudaStream_t, void*, int);
+template int build_fused<double>(hpx_plan_s*, const double*, const cplx<double>*, cudaStream_t, void*, int);
 
 }  // namespace hpx

@@ -221,7 +221,7 @@ bool packs_b(const hpx_plan_s* P);
 template <class T> void launch_dense(const hpx_plan_s* P, cudaStream_t s, const void* Dmat = nullptr);
 template <class T> void launch_cg(const hpx_plan_s* P, cudaStream_t s);
 template <class T> void launch_rot(const hpx_plan_s* P, T* alm, cudaStream_t s);
-int fused_tile_rows(int B);
+int fused_tile_rows(bool fp64);
 // per-order operators on the FP32 pipes; Mrows: row-major operators of the
 // layout of fusedM's SIMT form (NULL = fusedM), e.g. the synthesis operators synM
 template <class T> void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Mrows = nullptr);
@@ -246,7 +246,7 @@ void launch_timeout_selftest(const hpx_plan_s* P, int spins, cudaStream_t s);
 // (float or double) at x is NaN or infinite.
 void launch_finite_check(const void* x, int64_t n, bool fp64, int* status, cudaStream_t s);
 template <class T>
-int build_fused(hpx_plan_s* P, const double* D64, const cplx<double>* skew64, cudaStream_t s, void* out, bool tiled);
+int build_fused(hpx_plan_s* P, const double* D64, const cplx<double>* skew64, cudaStream_t s, void* out, int form);
 template <class T> void launch_synth_apply(const hpx_plan_s* P, const T* alm, cudaStream_t s);
 // float offset of element (row r of a tile with rp rows, column k) in the
 // tensor-core layout of M, relative to the tile's first chunk
