@@ -70,7 +70,7 @@ void free_plan(hpx_plan_s* P) {
     if (P->cap) cudaStreamDestroy(P->cap);
     auto& t = P->t;
     void* ptrs[] = {t.nphi, t.startN, t.startS, t.pow2, t.logn, t.fftL, t.logL, t.shOff, t.chOff,
-                    t.bhOff, t.shift, t.chirp, t.bhat, t.twid, t.ch4Off, t.bh4Off, t.chirp4, t.bhat4, t.poleN,
+                    t.bhOff, t.pw, t.shift, t.chirp, t.bhat, t.twid, t.ch4Off, t.bh4Off, t.chirp4, t.bhat4, t.poleN,
                     t.poleS, t.polew, t.rowptr,
                     t.ent, t.entw, t.dec, t.D, t.tstart, t.hwn, t.angOff, t.ang, t.skOff, t.skew, t.skewT, t.nrowptr, t.nent, t.nentw, t.nstart, t.swts, t.hstart, t.hwts, t.Es, t.shifted, t.C, t.cgH, P->Y, P->U, P->bvec,
                     P->fusedM, P->fusedOff, P->fusedTiles, P->tcOff, P->tcFirst, P->tcRinv, P->bscale, P->d_status, P->synM, P->ringList,
@@ -263,6 +263,11 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
     }
     t.rowptr = up.vec(tb.rowptr); t.ent = up.vec(tb.ent);
     t.entw = up.real(tb.entw, fp64); t.dec = up.real(tb.dec, fp64);
+    if (!fp64 && tb.M >= hpx::kPrewhitenMin) {
+        if (cudaMalloc(&t.pw, (size_t)(tb.p + 1) * 8) != cudaSuccess) { free_plan(P); set_err(HPX_ERR_OOM); return nullptr; }
+        P->bytes += (int64_t)(tb.p + 1) * 8;
+        hpx::launch_prewhiten_table(t.pw, tb.M);
+    }
     t.nstart = up.vec(tb.nstart); t.swts = up.real(tb.swts, fp64); t.spreadE = tb.spreadE;
     t.hstart = up.vec(tb.hstart); t.hwts = up.real(tb.hwts, fp64); t.spreadH = tb.spreadH;
     t.tstart = up.vec(tb.tstart); t.hwn = up.real(tb.hwn, fp64); t.interpE = tb.interpE;
@@ -296,7 +301,7 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
     if (cudaMalloc(&P->bvec, bSize) != cudaSuccess) { free_plan(P); set_err(HPX_ERR_OOM); return nullptr; }
     P->beta = P->Y;   // Y is dead once the NUFFT has read it
     P->ldu = (g.M / 2 + 2) & ~1;
-    const size_t uSize = (size_t)g.B * (g.L + 1) * P->ldu * es;
+    const size_t uSize = (size_t)g.B * std::max((size_t)(g.L + 1) * P->ldu, (size_t)((g.L + 2) / 2) * g.M) * es;
     if (cudaMalloc(&P->U, uSize) != cudaSuccess) { free_plan(P); set_err(HPX_ERR_OOM); return nullptr; }
     P->bytes += (int64_t)(std::max(ySize, bSize) + bSize + uSize);
     P->flags = d->flags;
@@ -491,18 +496,17 @@ void tune_shapes(hpx_plan_s* P, const void* maps, void* alm, cudaEvent_t e0, cud
             return;
         }
     }
-    float t[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+    float t[2] = {0.f, 0.f};
     for (int e = 0; e < 2; ++e) {
-        P->ringE = P->latE = e ? 32 : 16;
-        t[0][e] = time_stage(P, maps, alm, 0, e0, e1);
-        t[1][e] = time_stage(P, maps, alm, 1, e0, e1);
+        P->ringE = e ? 32 : 16;
+        t[e] = time_stage(P, maps, alm, 0, e0, e1);
     }
-    P->ringE = t[0][1] < t[0][0] ? 32 : 16;
-    P->latE = t[1][1] < t[1][0] ? 32 : 16;
+    P->ringE = t[1] < t[0] ? 32 : 16;
+    P->latE = 16;   // the grid FFT has one shape
     {   // the Bluestein ring classes: whole-ring or quarter-length convolutions
         P->ringForm = 1;
         const float t4 = time_stage(P, maps, alm, 0, e0, e1);
-        P->ringForm = t4 < t[0][P->ringE == 32 ? 1 : 0] ? 1 : 0;
+        P->ringForm = t4 < t[P->ringE == 32 ? 1 : 0] ? 1 : 0;
     }
     P->rotForm = 0;
     if (sweeps) {   // the three forms of the sweep kernel

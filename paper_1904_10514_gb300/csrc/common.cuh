@@ -127,8 +127,9 @@ __device__ __forceinline__ double s16d(int k) {
 }
 
 // In-register R-point DFT (R = 2, 4, 8, 16): radix-2 decimation in frequency,
-// then the bit-reversed outputs are renamed into natural order.
-template <class T, int R, bool INV>
+// then the bit-reversed outputs are renamed into natural order.  HZ: x[R/2..] are
+// zero and not read (the first stage copies and rotates).
+template <class T, int R, bool INV, bool HZ = false>
 __device__ __forceinline__ void reg_dft(cplx<T>* x) {
 #pragma unroll
     for (int half = R / 2; half >= 1; half >>= 1) {
@@ -137,9 +138,12 @@ __device__ __forceinline__ void reg_dft(cplx<T>* x) {
             if ((i & half) == 0) {
                 const int pos = i & (half - 1);
                 const int k16 = pos * (8 / half);   // e^{-2 pi i pos / (2 half)} = e^{-2 pi i k16 / 16}
-                const cplx<T> u = x[i], v = x[i + half];
-                x[i] = add(u, v);
-                const cplx<T> d = sub(u, v);
+                cplx<T> d = x[i];
+                if (!(HZ && half == R / 2)) {
+                    const cplx<T> u = x[i], v = x[i + half];
+                    x[i] = add(u, v);
+                    d = sub(u, v);
+                }
                 if (pos == 0) {
                     x[i + half] = d;
                 } else if (k16 == 4) {   // w = -i (forward) or +i (inverse)
@@ -174,29 +178,44 @@ __device__ __forceinline__ void reg_dft(cplx<T>* x) {
 
 // x[r] *= w^(r j), w^(r j) = tw[r j step] (conjugated for INV): w^j, w^2j,
 // w^4j, w^8j from the table; for r = 4 hi + lo the power is (w^4j)^hi (w^j)^lo,
-// with w^3j and w^12j formed once (at most two products per power).
+// with w^3j and w^12j formed once (at most two products per power).  In two steps, so
+// that the table reads can be issued before a barrier: Twiddles holds the four
+// powers, twiddle_by applies them.
+template <class T>
+struct Twiddles {
+    cplx<T> b1, b2, b4, b8;
+};
 template <class T, int R, bool INV>
-__device__ __forceinline__ void twiddle(cplx<T>* x, int j, int step, const cplx<T>* __restrict__ tw) {
+__device__ __forceinline__ Twiddles<T> load_twiddles(int j, int step, const cplx<T>* __restrict__ tw) {
     auto ld = [&](int r) {
         cplx<T> w = tw[r * j * step];
         if (INV) w.i = -w.i;
         return w;
     };
-    const cplx<T> b1 = ld(1);
-    const cplx<T> b2 = R > 2 ? ld(2) : b1;
-    const cplx<T> w3 = R > 2 ? mul(b1, b2) : b1;
-    const cplx<T> b4 = R > 4 ? ld(4) : b1;
-    const cplx<T> b8 = R > 8 ? ld(8) : b1;
-    const cplx<T> w12 = R > 8 ? mul(b4, b8) : b1;
+    Twiddles<T> t;
+    t.b1 = ld(1);
+    t.b2 = R > 2 ? ld(2) : t.b1;
+    t.b4 = R > 4 ? ld(4) : t.b1;
+    t.b8 = R > 8 ? ld(8) : t.b1;
+    return t;
+}
+template <class T, int R>
+__device__ __forceinline__ void twiddle_by(cplx<T>* x, const Twiddles<T>& t) {
+    const cplx<T> w3 = R > 2 ? mul(t.b1, t.b2) : t.b1;
+    const cplx<T> w12 = R > 8 ? mul(t.b4, t.b8) : t.b1;
 #pragma unroll
     for (int r = 1; r < R; ++r) {
         const int hi = r >> 2, lo = r & 3;
-        const cplx<T> wl = lo == 1 ? b1 : lo == 2 ? b2 : w3;
-        const cplx<T> wh = hi == 1 ? b4 : hi == 2 ? b8 : w12;
+        const cplx<T> wl = lo == 1 ? t.b1 : lo == 2 ? t.b2 : w3;
+        const cplx<T> wh = hi == 1 ? t.b4 : hi == 2 ? t.b8 : w12;
         if (hi == 0) x[r] = mul(x[r], wl);
         else if (lo == 0) x[r] = mul(x[r], wh);
         else x[r] = mul(mul(x[r], wh), wl);
     }
+}
+template <class T, int R, bool INV>
+__device__ __forceinline__ void twiddle(cplx<T>* x, int j, int step, const cplx<T>* __restrict__ tw) {
+    twiddle_by<T, R>(x, load_twiddles<T, R, INV>(j, step, tw));
 }
 
 template <class T, int R, int G, bool INV>

@@ -26,6 +26,7 @@ struct DevTables {
     int *rowptr = nullptr, *ent = nullptr;
     void *entw = nullptr, *dec = nullptr;   // T
     int* nstart = nullptr;                  // dense spreading table: first node per grid point
+    void* pw = nullptr;                     // cplx<float> [p+1]: undoes the difference of the FP32 grid FFT (k_nufft.cu)
     void* swts = nullptr;                   // T [spreadE][M]
     int spreadE = 0;
     int* tstart = nullptr;                  // interpolation (transpose of the half-grid spreading)
@@ -65,7 +66,8 @@ struct hpx_plan_s {
     hpx::DevTables t;
     // workspace
     void* Y = nullptr;      // cplx<T> [B][Q][p+1]: step-1 ring coefficients per latitude node
-    void* U = nullptr;      // cplx<T> [B][L+1][ldu]: spread half grids (t = 0..M/2) per column
+    void* U = nullptr;      // cplx<T>: analysis [B][(L+2)/2][M], the spread grid of each pair of orders (k_nufft.cu);
+                            // other direction [B][L+1][ldu], half grids (t = 0..M/2) per column (k_nufft2.cu)
     int ldu = 0;
     void* bvec = nullptr;   // cplx<T> [B][p+1][2][P2]: latitude NUFFT right-hand sides
     void* beta = nullptr;   // cplx<T> [B][p+1][2][P2]: order-0/1 Legendre coefficients (aliases Y)
@@ -204,6 +206,10 @@ void launch_ring_list(const RingJob<T>* jobs, const int4* items, int nitems, int
 // ring transforms of this many points or more run in launches of one length and
 // one kind (plain or Bluestein) with the compile-time FFT of fft_ct.cuh
 constexpr int kRingCtMin = 4096;
+// leaky first difference of the FP32 grid FFT of 4096 points and more (k_nufft.cu)
+constexpr float kPrewhiten = 0.875f;
+constexpr int kPrewhitenMin = 4096;
+void launch_prewhiten_table(void* pw, int M);
 
 // ew != 0: the rows of the equal-weight quadrature's ring stage (every m <= lmax,
 // aliased mod nphi, synthesis fold weights, times ew) instead of the analysis'

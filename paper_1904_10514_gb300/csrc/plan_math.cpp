@@ -414,7 +414,7 @@ std::string build_tables(int nside, int lmax, bool fp64, PlanTables& t) {
                 if (t.hstart[i] < t.hstart[i - 1]) return "half-grid spreading starts are not monotone";
             int rows32 = 0;
             for (int t0 = 0; t0 <= H; t0 += 32)
-                rows32 = std::max(rows32, t.hstart[std::min(t0 + 31, H)] + E - t.hstart[t0]);
+                rows32 = std::max(rows32, t.hstart[std::min(t0 + 32, H)] + E - t.hstart[std::max(t0 - 1, 0)]);
             t.spreadRows = rows32;
             // the same weights grouped by latitude node: node r sees the half-grid
             // points tstart[r] .. tstart[r] + En - 1 (a contiguous run, since the
