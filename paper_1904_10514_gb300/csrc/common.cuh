@@ -20,6 +20,13 @@ template <class T> __device__ __forceinline__ cplx<T> mul(cplx<T> a, cplx<T> b) 
 template <class T> __device__ __forceinline__ cplx<T> conjg(cplx<T> a) { return mk<T>(a.r, -a.i); }
 template <class T> __device__ __forceinline__ cplx<T> scale(cplx<T> a, T s) { return mk<T>(a.r * s, a.i * s); }
 
+// Hides from the compiler how an FP32 value came about, as a trip through memory
+// does: within what it sees it fuses a product into the sum that uses it, and a pass
+// kept in registers would round differently from one that goes through memory.
+template <class T> __device__ __forceinline__ void hide(cplx<T>& v) {
+    if constexpr (sizeof(T) == 4) asm("" : "+f"(v.r), "+f"(v.i));
+}
+
 // 8-byte asynchronous global -> shared copy; src_bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async8(void* dst, const void* src, int src_bytes) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);

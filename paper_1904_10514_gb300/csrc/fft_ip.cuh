@@ -201,7 +201,10 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
             twiddle_by<T, R>(x, t);
             reg_dft<T, R, false>(x);
 #pragma unroll
-            for (int q = 0; q < R; ++q) y[i + q * D] = mul(x[q], ker(tid + (i + q * D) * NG));
+            for (int q = 0; q < R; ++q) {
+                y[i + q * D] = mul(x[q], ker(tid + (i + q * D) * NG));
+                hide(y[i + q * D]);
+            }
         }
         reg_dft<T, 16, true>(y);
     }

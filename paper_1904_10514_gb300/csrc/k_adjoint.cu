@@ -12,10 +12,12 @@
 //   dense_adj  beta -> b:  D^T (latitude least squares and Legendre change of basis)
 //   nufft_adj  b -> y: deconvolution, inverse M-point FFT and interpolation from the
 //              fine grid to the DFS nodes (the transposed ES spreading, Sec. 3.2.2)
-//   ring_adj   y -> ring samples: transposed shift/Nyquist/padding and inverse
+//   ring_back  y -> ring samples: transposed shift/Nyquist/padding and inverse
 //              DFT per ring pair (Sec. 3.1)
 //   pole_adj   adds the transposed pole fit (Sec. 3.2.1) to the 3 rings per cap
-#include "fft_ct.cuh"
+#include <algorithm>
+
+#include "ring_blue.cuh"
 #include "plan.h"
 #include "plan_math.h"
 #include "sweep.cuh"
@@ -339,72 +341,6 @@ __global__ void __launch_bounds__(512) nufft_adj_kernel(const cplx<T>* __restric
     }
 }
 
-// ---------------------------------------------------------------- ring_adj
-template <class T>
-__global__ void __launch_bounds__(256) ring_adj_kernel(
-    const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ nphi_t,
-    const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int* __restrict__ pow2_t,
-    const int* __restrict__ logn_t, const int* __restrict__ fftL_t, const int* __restrict__ logL_t,
-    const int64_t* __restrict__ shOff_t, const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t,
-    const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat,
-    const cplx<T>* __restrict__ tw, int twlen, int p, int Q, int64_t npix, int npairs,
-    const int* __restrict__ ringlist) {
-    extern __shared__ unsigned char smem_raw[];
-    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
-    const int i = ringlist ? ringlist[blockIdx.x] : npairs - 1 - (int)blockIdx.x;
-    const int b = blockIdx.y;
-    const int n = nphi_t[i], h = n >> 1;
-    const int sN = startN_t[i], sS = startS_t[i];
-    const bool equator = (sN == sS);
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const cplx<T>* ph = shift + shOff_t[i];
-    const cplx<T>* rowN = Y + ((int64_t)b * Q + (i + 1)) * (p + 1);
-    const cplx<T>* rowS = Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1);
-    const bool bl = !pow2_t[i];
-    const cplx<T>* ch = chirp + chOff_t[i];
-    // X = H_N + i H_S with H the Hermitian extension of z_m = conj(ph_m) y_m
-    for (int m = tid; m <= h; m += nt) {
-        const cplx<T> w = conjg(ph[m]);
-        const cplx<T> zn = mul(w, rowN[m]);
-        const cplx<T> zs = equator ? mk<T>(T(0), T(0)) : mul(w, rowS[m]);
-        cplx<T> xm, xc;
-        if (m == 0 || m == h) {
-            xm = mk<T>(zn.r, zs.r);
-        } else {
-            xm = mk<T>(T(0.5) * (zn.r - zs.i), T(0.5) * (zn.i + zs.r));   // zn/2 + i zs/2
-            xc = mk<T>(T(0.5) * (zn.r + zs.i), T(0.5) * (-zn.i + zs.r));  // conj(zn)/2 + i conj(zs)/2
-        }
-        // Bluestein: transform conj(X) forward, premultiplied by the chirp
-        if (bl) {
-            buf[m] = mul(conjg(xm), ch[m]);
-            if (m != 0 && m != h) buf[n - m] = mul(conjg(xc), ch[n - m]);
-        } else {
-            buf[m] = xm;
-            if (m != 0 && m != h) buf[n - m] = xc;
-        }
-    }
-    if (bl) {
-        const int L = fftL_t[i];
-        for (int k = n + tid; k < L; k += nt) buf[k] = mk<T>(T(0), T(0));
-        __syncthreads();
-        const cplx<T>* bh = bhat + bhOff_t[i];
-        block_fft(buf, L, logL_t[i], tw, twlen, false);
-        for (int k = tid; k < L; k += nt) buf[k] = mul(buf[k], bh[k]);
-        __syncthreads();
-        block_fft(buf, L, logL_t[i], tw, twlen, true);
-        for (int k = tid; k < n; k += nt) buf[k] = conjg(mul(buf[k], ch[k]));
-        __syncthreads();
-    } else {
-        __syncthreads();
-        block_fft(buf, n, logn_t[i], tw, twlen, true);
-    }
-    T* f = maps + (int64_t)b * npix;
-    for (int k = tid; k < n; k += nt) {
-        f[sN + k] = buf[k].r;
-        if (!equator) f[sS + k] = buf[k].i;
-    }
-}
-
 template <class T>
 __global__ void pole_adj_kernel(const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ poleN,
                                 const int* __restrict__ poleS, const double* __restrict__ w, int npole, int p,
@@ -420,99 +356,236 @@ __global__ void pole_adj_kernel(const cplx<T>* __restrict__ Y, T* __restrict__ m
     }
 }
 
-// ring_adj_kernel for the ring classes of 4096 points and more, with the
-// compile-time FFT: the first pass reads the Hermitian extension X of each ring
-// pair straight from the rows of Y.
-template <class T, int LOGN, int NT, bool BLUE>
-__global__ void __launch_bounds__(NT, (LOGN <= 13 ? 1024 / NT : 1)) ring_adj_ct_kernel(
-    const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ nphi_t,
-    const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int64_t* __restrict__ shOff_t,
-    const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t, const cplx<T>* __restrict__ shift,
-    const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat, const cplx<T>* __restrict__ tw, int twlen,
-    int p, int Q, int64_t npix, const int* __restrict__ ringlist) {
-    extern __shared__ unsigned char smem_raw[];
-    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
-    const int i = ringlist[blockIdx.y];
-    const int b = blockIdx.x;
-    const int n = nphi_t[i], h = n >> 1;
-    const int sN = startN_t[i], sS = startS_t[i];
-    const bool equator = (sN == sS);
-    const int tid = threadIdx.x;
-    const int twstep = twlen >> LOGN;
-    const cplx<T>* ph = shift + shOff_t[i];
-    const cplx<T>* rowN = Y + ((int64_t)b * Q + (i + 1)) * (p + 1);
-    const cplx<T>* rowS = Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1);
-    // X_k = H_N + i H_S, H the Hermitian extension of z_m = conj(ph_m) y_m (k < n)
-    auto X = [&](int k) {
-        const int m = k <= h ? k : n - k;
-        const cplx<T> w = conjg(ph[m]);
-        const cplx<T> zn = mul(w, rowN[m]);
-        const cplx<T> zs = equator ? mk<T>(T(0), T(0)) : mul(w, rowS[m]);
-        if (m == 0 || m == h) return mk<T>(zn.r, zs.r);
-        if (k <= h) return mk<T>(T(0.5) * (zn.r - zs.i), T(0.5) * (zn.i + zs.r));   // zn/2 + i zs/2
-        return mk<T>(T(0.5) * (zn.r + zs.i), T(0.5) * (-zn.i + zs.r));              // conj(zn)/2 + i conj(zs)/2
-    };
-    auto to_smem = [&](int, int pi, cplx<T> v) { buf[pi] = v; };
-    if constexpr (!BLUE) {
-        ct::fft<T, LOGN, NT, true, false>(buf, tw, twstep, [&](int k, int) { return X(k); }, to_smem);
-    } else {
-        // inverse DFT of length n via Bluestein: transform conj(X) forward with the chirp
-        const cplx<T>* ch = chirp + chOff_t[i];
-        const cplx<T>* bh = bhat + bhOff_t[i];
-        ct::fft<T, LOGN, NT, false, false>(
-            buf, tw, twstep, [&](int k, int) { return k < n ? mul(conjg(X(k)), ch[k]) : mk<T>(T(0), T(0)); },
-            [&](int j, int pi, cplx<T> v) { buf[pi] = mul(v, bh[j]); });
-        ct::fft<T, LOGN, NT, true, true>(
-            buf, tw, twstep, [&](int, int pi) { return buf[pi]; },
-            [&](int j, int pi, cplx<T> v) { buf[pi] = j < n ? conjg(mul(v, ch[j])) : v; });
+// ---------------------------------------------------------------- rings, backwards
+// Both directions that end in maps finish with an inverse DFT per ring pair: the
+// north and south rings packed as z = f_N + i f_S, conj(z) = DFT(conj(Z)) with conj(Z_k)
+// formed on the fly from the pair's rows of Y (BackInput), on the in-place passes of
+// fft_ip.cuh (Bluestein rings of 4096 points and more: ring_blue.cuh), the pixels written straight from
+// registers by the last pass (plain rings) or the radix-4 step (Bluestein rings).
+//
+// adjoint (SYN = false): Z = H_N + i H_S with H the Hermitian extension of
+//     conj(ph_m) y_m (the transposed shift, Nyquist split and padding of Sec. 3.1);
+// synthesis (SYN = true): Z_k = sum of F_m e^{i m phi0} over m = k mod n, m in [-L, L],
+//     F_m = Y_m (Y_m / 2 for even m: ring weight 2), F_{-m} = conj(F_m).  With
+//     phi0 = pi / n every phase is +-e^{i pi k / n}: (-1)^q for m = k + q n and
+//     m = k - q n, so a rotation is made once per k; phi0 = 0: none.
+// Bound by the shared-memory passes and, in the synthesis, the reads of the aliased
+// orders.  Synthesis of 32 maps at Nside 512: 1266 us (plain and short rings, radix-2
+// passes) + 321 us (Bluestein rings, whole convolutions) before, 487 + 257 us now.
+template <class T, bool SYN>
+struct BackInput {
+    const cplx<T>*rowN, *rowS, *ph;
+    int n, L;
+    bool equator, sh;
+
+    __device__ __forceinline__ cplx<T> operator()(int k) const {
+        const cplx<T> zero = mk<T>(T(0), T(0));
+        if constexpr (!SYN) {
+            const int h = n >> 1, m = k <= h ? k : n - k;
+            if (m > L) return zero;
+            const cplx<T> w = conjg(ph[m]);
+            const cplx<T> zn = mul(w, rowN[m]);
+            const cplx<T> zs = equator ? zero : mul(w, rowS[m]);
+            if (m == 0 || m == h) return mk<T>(zn.r, -zs.r);
+            if (k <= h) return mk<T>(T(0.5) * (zn.r - zs.i), T(-0.5) * (zn.i + zs.r));   // conj(zn/2 + i zs/2)
+            return mk<T>(T(0.5) * (zn.r + zs.i), T(-0.5) * (-zn.i + zs.r));              // conj(conj(zn)/2 + i conj(zs)/2)
+        } else {
+            cplx<T> cN = zero, cS = zero;
+            T sg = T(1);
+            auto take = [&](int m, bool cj) {   // +-F_m or +-conj(F_m) of both rings
+                const T f = (m & 1) ? sg : T(0.5) * sg;
+                cplx<T> v = rowN[m];
+                if (m == 0) v.i = T(0);
+                cN.r += f * v.r;
+                cN.i += cj ? -(f * v.i) : f * v.i;
+                if (!equator) {
+                    v = rowS[m];
+                    if (m == 0) v.i = T(0);
+                    cS.r += f * v.r;
+                    cS.i += cj ? -(f * v.i) : f * v.i;
+                }
+            };
+            for (int m = k; m <= L; m += n) {
+                take(m, false);
+                if (sh) sg = -sg;
+            }
+            sg = sh ? T(-1) : T(1);
+            for (int m = n - k; m <= L; m += n) {
+                take(m, true);
+                if (sh) sg = -sg;
+            }
+            if (sh) {
+                T sn, cs;
+                if constexpr (sizeof(T) == 4) sincospif((float)k / (float)n, &sn, &cs);
+                else sincospi((double)k / (double)n, &sn, &cs);
+                const cplx<T> w = mk<T>(cs, sn);
+                cN = mul(w, cN);
+                cS = mul(w, cS);
+            }
+            return mk<T>(cN.r - cS.i, -(cN.i + cS.r));
+        }
     }
-    T* f = maps + (int64_t)b * npix;
-    for (int k = tid; k < n; k += NT) {
-        const cplx<T> v = buf[ct::padc(k)];
-        f[sN + k] = v.r;
-        if (!equator) f[sS + k] = v.i;
+};
+
+// Bluestein rings: four quarter transforms (ring_blue.cuh) of 2^LOGQ points, or one
+// convolution of the whole ring of 2^LOGN points.
+template <class T, int LOGQ, int NTQ, class V>
+__device__ __forceinline__ void ring_back_quarters(cplx<T>* buf, T* f, int sN, int sS, int n,
+                                                   const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
+                                                   const cplx<T>* __restrict__ tw, int twlen, V in) {
+    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ>(buf, n, ch, bh, tw, twlen, in);
+    const int jq = n >> 2;
+    for (int q = threadIdx.x; q < jq; q += 4 * NTQ) {
+        cplx<T> z[4];
+        R.combine(q, n, z);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            f[sN + q + r * jq] = z[r].r;
+            f[sS + q + r * jq] = -z[r].i;
+        }
     }
 }
 
-template <class T>
-void launch_ring_adj(const hpx_plan_s* P, T* maps, cudaStream_t s) {
+template <class T, int LOGN, int NT, class V>
+__device__ __forceinline__ void ring_back_whole(cplx<T>* buf, T* f, int sN, int sS, int n,
+                                                const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
+                                                const cplx<T>* __restrict__ tw, int twlen, V in) {
+    ip::convolve<T, LOGN, NT>(
+        buf, tw, twlen >> LOGN, threadIdx.x, [&](int k) { return k < n ? mul(in(k), ch[k]) : mk<T>(T(0), T(0)); },
+        [&](int k) { return bh[k]; },
+        [&](int k, cplx<T> v) {
+            if (k < n) {
+                const cplx<T> z = mul(v, ch[k]);
+                f[sN + k] = z.r;
+                f[sS + k] = -z.i;
+            }
+        });
+}
+
+// Rings of n = 2^LOGN points.
+template <class T, int LOGN, int NT, class V>
+__device__ __forceinline__ void ring_back_plain(cplx<T>* buf, T* f, int sN, int sS, const cplx<T>* __restrict__ tw,
+                                                int twlen, V in) {
+    constexpr int R = ip::out_radix(LOGN, NT);
+    ip::transform<T, LOGN, NT, false, R, R>(
+        buf, tw, twlen >> LOGN, threadIdx.x, [&](int k, int) { return in(k); },
+        [&](int k, int, int, cplx<T> v) {
+            f[sN + k] = v.r;
+            if (sN != sS) f[sS + k] = -v.i;
+        });
+}
+
+// One transform length per launch (KIND 0: rings of 2^LOGN points, KIND 2: Bluestein
+// rings as quarters of 2^LOGN points).
+template <class T, bool SYN, int LOGN, int NT, int MINB, int KIND>
+__global__ void __launch_bounds__(KIND ? 4 * NT : NT, MINB) ring_back_kernel(
+    const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ nphi_t,
+    const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int* __restrict__ shifted_t,
+    const int64_t* __restrict__ shOff_t, const int64_t* __restrict__ ch4Off_t, const int64_t* __restrict__ bh4Off_t,
+    const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp4, const cplx<T>* __restrict__ bhat4,
+    const cplx<T>* __restrict__ tw, int twlen, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
+    extern __shared__ unsigned char smem_raw[];
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
+    const int i = ringlist[blockIdx.y], b = blockIdx.x;
+    const int n = nphi_t[i], sN = startN_t[i], sS = startS_t[i];
+    const BackInput<T, SYN> in{Y + ((int64_t)b * Q + (i + 1)) * (p + 1), Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1),
+                               shift + shOff_t[i], n, L, sN == sS, shifted_t[i] != 0};
+    T* f = maps + (int64_t)b * npix;
+    if constexpr (KIND == 2)
+        ring_back_quarters<T, LOGN, NT>(buf, f, sN, sS, n, chirp4 + ch4Off_t[i], bhat4 + bh4Off_t[i], tw, twlen, in);
+    else
+        ring_back_plain<T, LOGN, NT>(buf, f, sN, sS, tw, twlen, in);
+}
+
+// Every transform of at most 2048 points in one launch of 128 threads per ring
+// pair; below 512 points the run-time length FFT.
+template <class T, bool SYN>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3) ring_back_short_kernel(
+    const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ nphi_t,
+    const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int* __restrict__ shifted_t,
+    const int* __restrict__ pow2_t, const int* __restrict__ logn_t, const int* __restrict__ logL_t,
+    const int64_t* __restrict__ shOff_t, const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t,
+    const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat,
+    const cplx<T>* __restrict__ tw, int twlen, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
+    extern __shared__ unsigned char smem_raw[];
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
+    const int i = ringlist[blockIdx.y], b = blockIdx.x;
+    const int n = nphi_t[i], sN = startN_t[i], sS = startS_t[i];
+    const BackInput<T, SYN> in{Y + ((int64_t)b * Q + (i + 1)) * (p + 1), Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1),
+                               shift + shOff_t[i], n, L, sN == sS, shifted_t[i] != 0};
+    T* f = maps + (int64_t)b * npix;
+    const cplx<T>*ch = chirp + chOff_t[i], *bh = bhat + bhOff_t[i];
+    if (pow2_t[i]) {
+        switch (logn_t[i]) {
+            case 11: ring_back_plain<T, 11, 128>(buf, f, sN, sS, tw, twlen, in); return;
+            case 10: ring_back_plain<T, 10, 128>(buf, f, sN, sS, tw, twlen, in); return;
+            case 9: ring_back_plain<T, 9, 128>(buf, f, sN, sS, tw, twlen, in); return;
+            default: break;
+        }
+    } else {
+        switch (logL_t[i]) {
+            case 11: ring_back_whole<T, 11, 128>(buf, f, sN, sS, n, ch, bh, tw, twlen, in); return;
+            case 10: ring_back_whole<T, 10, 128>(buf, f, sN, sS, n, ch, bh, tw, twlen, in); return;
+            case 9: ring_back_whole<T, 9, 128>(buf, f, sN, sS, n, ch, bh, tw, twlen, in); return;
+            default: break;
+        }
+    }
+    const int tid = threadIdx.x;
+    if (pow2_t[i]) {
+        for (int k = tid; k < n; k += 128) buf[pad(k)] = in(k);
+        __syncthreads();
+        block_fft_pad<T, 16>(buf, logn_t[i], tw, twlen, false);
+    } else {
+        const int N = 1 << logL_t[i];
+        for (int k = tid; k < N; k += 128) buf[pad(k)] = k < n ? mul(in(k), ch[k]) : mk<T>(T(0), T(0));
+        __syncthreads();
+        block_fft_pad<T, 16>(buf, logL_t[i], tw, twlen, false);
+        for (int k = tid; k < N; k += 128) buf[pad(k)] = mul(buf[pad(k)], bh[k]);
+        __syncthreads();
+        block_fft_pad<T, 16>(buf, logL_t[i], tw, twlen, true);
+        for (int k = tid; k < n; k += 128) buf[pad(k)] = mul(buf[pad(k)], ch[k]);
+        __syncthreads();
+    }
+    for (int k = tid; k < n; k += 128) {
+        const cplx<T> v = buf[pad(k)];
+        f[sN + k] = v.r;
+        if (sN != sS) f[sS + k] = -v.i;
+    }
+}
+
+template <class T, bool SYN>
+void launch_ring_back(const hpx_plan_s* P, T* maps, cudaStream_t s) {
     const auto& g = P->g;
     const auto& t = P->t;
-    auto old = [&](int blocks, size_t smem, const int* list) {
-        cudaFuncSetAttribute(ring_adj_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        dim3 grid(blocks, g.B);
-        ring_adj_kernel<T><<<grid, 256, smem, s>>>(
-            (const cplx<T>*)P->Y, maps, t.nphi, t.startN, t.startS, t.pow2, t.logn, t.fftL, t.logL, t.shOff,
-            t.chOff, t.bhOff, (const cplx<T>*)t.shift, (const cplx<T>*)t.chirp, (const cplx<T>*)t.bhat,
-            (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix, g.npairs, list);
-    };
-    if (!P->ringList) {
-        old(g.npairs, (size_t)g.smem_ring * sizeof(cplx<T>), nullptr);
-        return;
-    }
+    const cplx<T>*Y = (const cplx<T>*)P->Y, *shift = (const cplx<T>*)t.shift, *tw = (const cplx<T>*)t.twid;
     for (const auto& c : P->ringClasses) {
+        dim3 grid(g.B, c.count);
+        const int* list = P->ringList + c.first;
+        constexpr bool F = sizeof(T) == 4;
         if (c.N < kRingCtMin) {
-            old(c.count, (size_t)c.N * sizeof(cplx<T>), P->ringList + c.first);
+            auto kern = ring_back_short_kernel<T, SYN>;
+            const size_t smem = (size_t)std::max(ip::slots(c.N), c.N + c.N / 16) * sizeof(cplx<T>);
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            kern<<<grid, 128, smem, s>>>(Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.pow2, t.logn, t.logL,
+                                         t.shOff, t.chOff, t.bhOff, shift, (const cplx<T>*)t.chirp,
+                                         (const cplx<T>*)t.bhat, tw, g.Lmax, g.p, g.L, g.Q, g.npix, list);
             continue;
         }
-        const size_t smem = (size_t)(c.N + c.N / 16) * sizeof(cplx<T>);
-        dim3 grid(g.B, c.count);
+        const size_t smem = (size_t)(c.blue ? 4 * ip::slots(c.N / 4) : ip::slots(c.N)) * sizeof(cplx<T>);
         auto run = [&](auto kern, int threads) {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            kern<<<grid, threads, smem, s>>>((const cplx<T>*)P->Y, maps, t.nphi, t.startN, t.startS, t.shOff,
-                                             t.chOff, t.bhOff, (const cplx<T>*)t.shift, (const cplx<T>*)t.chirp,
-                                             (const cplx<T>*)t.bhat, (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q,
-                                             g.npix, P->ringList + c.first);
+            kern<<<grid, threads, smem, s>>>(Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.shOff, t.ch4Off,
+                                             t.bh4Off, shift, (const cplx<T>*)t.chirp4, (const cplx<T>*)t.bhat4, tw,
+                                             g.Lmax, g.p, g.L, g.Q, g.npix, list);
         };
         if (c.N == 4096) {
-            if (c.blue) run(ring_adj_ct_kernel<T, 12, 256, true>, 256);
-            else run(ring_adj_ct_kernel<T, 12, 256, false>, 256);
+            if (c.blue) run(ring_back_kernel<T, SYN, 10, 64, F ? 4 : 2, 2>, 256);
+            else run(ring_back_kernel<T, SYN, 12, 256, F ? 4 : 2, 0>, 256);
         } else if (c.N == 8192) {
-            if (c.blue) run(ring_adj_ct_kernel<T, 13, 512, true>, 512);
-            else run(ring_adj_ct_kernel<T, 13, 512, false>, 512);
-        } else {
-            if (c.blue) run(ring_adj_ct_kernel<T, 14, 512, true>, 512);
-            else run(ring_adj_ct_kernel<T, 14, 512, false>, 512);
+            if (c.blue) run(ring_back_kernel<T, SYN, 11, 128, F ? 2 : 1, 2>, 512);
+            else run(ring_back_kernel<T, SYN, 13, 256, F ? 2 : 1, 0>, 256);
+        } else if constexpr (F) {   // nside 2048 (FP32 only)
+            run(ring_back_kernel<T, SYN, 12, 256, 1, 2>, 1024);
         }
     }
 }
@@ -545,16 +618,14 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
         while ((1 << logM) < g.M) ++logM;
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
         cudaFuncSetAttribute(nufft_adj_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        // columns m > lmax carry no coefficients: their rows of Y are zero
-        cudaMemsetAsync(P->Y, 0, (size_t)g.B * g.Q * (g.p + 1) * sizeof(cplx<T>), s);
         dim3 grid(g.L + 1, g.B);
-        if (!launch_nufft2(P, s))
+        if (!launch_nufft2<T>(P, s))
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,
                                                     (const T*)t.nentw, (const T*)t.dec, (const cplx<T>*)t.twid,
                                                     g.Lmax, g.M, logM, g.p, g.Q, g.P2);
     }
     {
-        launch_ring_adj<T>(P, maps, s);
+        launch_ring_back<T, false>(P, maps, s);
         pole_adj_kernel<T><<<g.B, 128, 0, s>>>((const cplx<T>*)P->Y, maps, t.poleN, t.poleS, t.polew, t.npole,
                                                g.p, g.Q, g.npix);
     }
@@ -569,206 +640,10 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
 //      F_m(t) = (1/sqrt(2 pi)) sum_l a_l^m Pbar_l^m(cos t) = sum_j X_j cos|sin(j t);
 //   3. nufft_adj_kernel evaluates the cosine / sine series at the latitude nodes
 //      (type-2 NUFFT; for even m it returns w_r F_m(t_r) with w_r = 2 on rings);
-//   4. ring_synth_kernel folds the orders into the nphi frequencies of each ring,
+//   4. ring_back_kernel folds the orders into the nphi frequencies of each ring,
 //      F_m e^{i m phi0} summed over m = n mod nphi (m in [-lmax, lmax]), and
 //      transforms back to the ring's pixels (N and S rings packed as one complex
 //      sequence; Bluestein for the polar rings).
-template <class T>
-__global__ void __launch_bounds__(256) ring_synth_kernel(
-    const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ nphi_t,
-    const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int* __restrict__ shifted_t,
-    const int* __restrict__ pow2_t, const int* __restrict__ logn_t, const int* __restrict__ fftL_t,
-    const int* __restrict__ logL_t, const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t,
-    const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat, const cplx<T>* __restrict__ tw, int twlen,
-    int p, int L, int Q, int64_t npix, int npairs, const int* __restrict__ ringlist) {
-    extern __shared__ unsigned char smem_raw[];
-    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
-    const int i = ringlist ? ringlist[blockIdx.x] : npairs - 1 - (int)blockIdx.x;
-    const int b = blockIdx.y;
-    const int n = nphi_t[i];
-    const int sN = startN_t[i], sS = startS_t[i];
-    const bool equator = (sN == sS);
-    const int sh = shifted_t[i];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const cplx<T>* rowN = Y + ((int64_t)b * Q + (i + 1)) * (p + 1);
-    const cplx<T>* rowS = Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1);
-    const bool bl = !pow2_t[i];
-    const cplx<T>* ch = chirp + chOff_t[i];
-    // G_m = F_m e^{i m phi0}, phi0 = sh pi / n; F_m = Y / 2 for even m (ring weight 2)
-    auto G = [&](const cplx<T>* row, int m) {
-        cplx<T> v = row[m];
-        if (!(m & 1)) v = scale(v, T(0.5));
-        if (m == 0) return mk<T>(v.r, T(0));
-        if (!sh) return v;
-        const int r = m % (2 * n);
-        T sn, cs;
-        if (sizeof(T) == 4) {
-            float a, c;
-            sincospif((float)r / (float)n, &a, &c);
-            sn = (T)a; cs = (T)c;
-        } else {
-            double a, c;
-            sincospi((double)r / (double)n, &a, &c);
-            sn = (T)a; cs = (T)c;
-        }
-        return mul(v, mk<T>(cs, sn));
-    };
-    for (int k = tid; k < n; k += nt) {
-        cplx<T> cN = mk<T>(T(0), T(0)), cS = cN;
-        for (int m = k; m <= L; m += n) {   // m = k + q n >= 0
-            cN = add(cN, G(rowN, m));
-            if (!equator) cS = add(cS, G(rowS, m));
-        }
-        for (int m = n - k; m <= L; m += n) {   // -m = k - q n < 0: G_{-m} = conj(G_m)
-            if (m == 0) continue;
-            cN = add(cN, conjg(G(rowN, m)));
-            if (!equator) cS = add(cS, conjg(G(rowS, m)));
-        }
-        // z = cN + i cS; the forward transform runs on conj(z) = (cN.r - cS.i) - i (cN.i + cS.r)
-        const cplx<T> zconj = mk<T>(cN.r - cS.i, -(cN.i + cS.r));
-        buf[k] = bl ? mul(zconj, ch[k]) : zconj;
-    }
-    if (bl) {
-        const int Lb = fftL_t[i];
-        for (int k = n + tid; k < Lb; k += nt) buf[k] = mk<T>(T(0), T(0));
-        __syncthreads();
-        const cplx<T>* bh = bhat + bhOff_t[i];
-        block_fft(buf, Lb, logL_t[i], tw, twlen, false);
-        for (int k = tid; k < Lb; k += nt) buf[k] = mul(buf[k], bh[k]);
-        __syncthreads();
-        block_fft(buf, Lb, logL_t[i], tw, twlen, true);
-        for (int k = tid; k < n; k += nt) buf[k] = mul(buf[k], ch[k]);
-        __syncthreads();
-    } else {
-        __syncthreads();
-        block_fft(buf, n, logn_t[i], tw, twlen, false);
-    }
-    // Z = conj(DFT(conj z)): north = Re Z, south = Im Z = -Im DFT(conj z)
-    T* f = maps + (int64_t)b * npix;
-    for (int k = tid; k < n; k += nt) {
-        f[sN + k] = buf[k].r;
-        if (!equator) f[sS + k] = -buf[k].i;
-    }
-}
-
-// ring_synth_kernel for the launches of one transform length N = 2^LOGN >= 4096
-// (the ring classes of the analysis: N = nphi for plain rings, the Bluestein
-// convolution length otherwise) with the compile-time FFT of fft_ct.cuh: the
-// fold of the orders is the first pass's input and the pixels are written from
-// shared memory after the transform.
-template <class T, int LOGN, int NT, bool BLUE>
-__global__ void __launch_bounds__(NT, (LOGN <= 13 ? 1024 / NT : 1)) ring_synth_ct_kernel(
-    const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ nphi_t,
-    const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int* __restrict__ shifted_t,
-    const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t, const cplx<T>* __restrict__ chirp,
-    const cplx<T>* __restrict__ bhat, const cplx<T>* __restrict__ tw, int twlen, int p, int L, int Q,
-    int64_t npix, const int* __restrict__ ringlist) {
-    const int twstep = twlen >> LOGN;
-    extern __shared__ unsigned char smem_raw[];
-    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
-    const int i = ringlist[blockIdx.y];
-    const int b = blockIdx.x;
-    const int n = nphi_t[i];
-    const int sN = startN_t[i], sS = startS_t[i];
-    const bool equator = (sN == sS);
-    const int sh = shifted_t[i];
-    const int tid = threadIdx.x;
-    const cplx<T>* rowN = Y + ((int64_t)b * Q + (i + 1)) * (p + 1);
-    const cplx<T>* rowS = Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1);
-    // G_m = F_m e^{i m phi0}, phi0 = sh pi / n; F_m = Y / 2 for even m (ring weight 2)
-    auto G = [&](const cplx<T>* row, int m) {
-        cplx<T> v = row[m];
-        if (!(m & 1)) v = scale(v, T(0.5));
-        if (m == 0) return mk<T>(v.r, T(0));
-        if (!sh) return v;
-        const int r = m % (2 * n);
-        T sn, cs;
-        if constexpr (sizeof(T) == 4) {
-            sincospif((float)r / (float)n, &sn, &cs);
-        } else {
-            sincospi((double)r / (double)n, &sn, &cs);
-        }
-        return mul(v, mk<T>(cs, sn));
-    };
-    // conj(z_k), z = (folded north) + i (folded south)
-    auto fold = [&](int k) {
-        cplx<T> cN = mk<T>(T(0), T(0)), cS = cN;
-        for (int m = k; m <= L; m += n) {
-            cN = add(cN, G(rowN, m));
-            if (!equator) cS = add(cS, G(rowS, m));
-        }
-        for (int m = n - k; m <= L; m += n) {
-            if (m == 0) continue;
-            cN = add(cN, conjg(G(rowN, m)));
-            if (!equator) cS = add(cS, conjg(G(rowS, m)));
-        }
-        return mk<T>(cN.r - cS.i, -(cN.i + cS.r));
-    };
-    auto to_smem = [&](int, int pi, cplx<T> v) { buf[pi] = v; };
-    if constexpr (!BLUE) {
-        ct::fft<T, LOGN, NT, false, false>(buf, tw, twstep, [&](int k, int) { return fold(k); }, to_smem);
-    } else {
-        const cplx<T>* ch = chirp + chOff_t[i];
-        const cplx<T>* bh = bhat + bhOff_t[i];
-        ct::fft<T, LOGN, NT, false, false>(
-            buf, tw, twstep, [&](int k, int) { return k < n ? mul(fold(k), ch[k]) : mk<T>(T(0), T(0)); },
-            [&](int j, int pi, cplx<T> v) { buf[pi] = mul(v, bh[j]); });
-        ct::fft<T, LOGN, NT, true, true>(
-            buf, tw, twstep, [&](int, int pi) { return buf[pi]; },
-            [&](int j, int pi, cplx<T> v) { buf[pi] = j < n ? mul(v, ch[j]) : v; });
-    }
-    // Z = conj(DFT(conj z)): north = Re Z, south = Im Z = -Im DFT(conj z)
-    T* f = maps + (int64_t)b * npix;
-    for (int k = tid; k < n; k += NT) {
-        const cplx<T> v = buf[ct::padc(k)];
-        f[sN + k] = v.r;
-        if (!equator) f[sS + k] = -v.i;
-    }
-}
-
-template <class T>
-void launch_ring_synth(const hpx_plan_s* P, T* maps, cudaStream_t s) {
-    const auto& g = P->g;
-    const auto& t = P->t;
-    auto old = [&](int blocks, size_t smem, const int* list) {
-        cudaFuncSetAttribute(ring_synth_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        dim3 grid(blocks, g.B);
-        ring_synth_kernel<T><<<grid, 256, smem, s>>>(
-            (const cplx<T>*)P->Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.pow2, t.logn, t.fftL, t.logL,
-            t.chOff, t.bhOff, (const cplx<T>*)t.chirp, (const cplx<T>*)t.bhat, (const cplx<T>*)t.twid, g.Lmax, g.p,
-            g.L, g.Q, g.npix, g.npairs, list);
-    };
-    if (!P->ringList) {
-        old(g.npairs, (size_t)g.smem_ring * sizeof(cplx<T>), nullptr);
-        return;
-    }
-    for (const auto& c : P->ringClasses) {
-        if (c.N < kRingCtMin) {   // short rings: the radix-2 kernel, sized for the class's longest transform
-            old(c.count, (size_t)c.N * sizeof(cplx<T>), P->ringList + c.first);
-            continue;
-        }
-        const size_t smem = (size_t)(c.N + c.N / 16) * sizeof(cplx<T>);
-        dim3 grid(g.B, c.count);
-        auto run = [&](auto kern, int threads) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            kern<<<grid, threads, smem, s>>>((const cplx<T>*)P->Y, maps, t.nphi, t.startN, t.startS, t.shifted,
-                                             t.chOff, t.bhOff, (const cplx<T>*)t.chirp, (const cplx<T>*)t.bhat,
-                                             (const cplx<T>*)t.twid, g.Lmax, g.p, g.L, g.Q, g.npix,
-                                             P->ringList + c.first);
-        };
-        if (c.N == 4096) {
-            if (c.blue) run(ring_synth_ct_kernel<T, 12, 256, true>, 256);
-            else run(ring_synth_ct_kernel<T, 12, 256, false>, 256);
-        } else if (c.N == 8192) {
-            if (c.blue) run(ring_synth_ct_kernel<T, 13, 512, true>, 512);
-            else run(ring_synth_ct_kernel<T, 13, 512, false>, 512);
-        } else {
-            if (c.blue) run(ring_synth_ct_kernel<T, 14, 512, true>, 512);
-            else run(ring_synth_ct_kernel<T, 14, 512, false>, 512);
-        }
-    }
-}
-
 template <class T>
 void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, cudaEvent_t* ev) {
     const auto& g = P->g;
@@ -802,13 +677,13 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
         cudaFuncSetAttribute(nufft_adj_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         dim3 grid(g.L + 1, g.B);
-        if (!launch_nufft2(P, s))
+        if (!launch_nufft2<T>(P, s))
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,
                                                         (const T*)t.nentw, (const T*)t.dec, (const cplx<T>*)t.twid,
                                                         g.Lmax, g.M, logM, g.p, g.Q, g.P2);
     }
     if (ev) cudaEventRecord(ev[2], s);
-    launch_ring_synth<T>(P, maps, s);
+    launch_ring_back<T, true>(P, maps, s);
     if (ev)
         for (int k = 3; k <= hpx_plan_s::kStages; ++k) cudaEventRecord(ev[k], s);
 }

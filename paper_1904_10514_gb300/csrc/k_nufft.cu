@@ -431,11 +431,9 @@ __global__ void __launch_bounds__(NT, MINB) lat_fft_pair_kernel(
     const bool has1 = m0 + 1 <= L;
     const cplx<T>* src = U + ((int64_t)b * gridDim.y + blockIdx.y) * M;
     cplx<T> lo[G1][LO];
-    // undoes the difference; the factor is made opaque to the compiler, which else
-    // fuses the product differently with the sign of its imaginary part
-    auto undo = [&](cplx<T> v, cplx<T> w) {
+    auto undo = [&](cplx<T> v, cplx<T> w) {   // undoes the difference
         if constexpr (PW) {
-            asm volatile("" : "+f"(w.r), "+f"(w.i));
+            hide(w);   // (the sign of w.i else changes which product is fused)
             v = mul(v, w);
         }
         return v;

@@ -10,8 +10,10 @@
 // with X_j = bvec[b][m][j & 1][j >> 1] (odd m: the conj(i/2)-scaled sine
 // coefficients of the analysis' right-hand-side convention).
 //
-// Two kernels, the transposes of lat_fft_pair and spread_rb:
-//   ifft_pair_ct_kernel  one block per pair of orders (m even, m + 1) and map:
+// Two kernels, the transposes of lat_fft_pair and spread_rb.  6 maps, Nside 256, lmax
+// 400: 163 us as one radix-2 FFT and one strided column per block (the form left for
+// Nside 2), now 12 + 25 us.
+//   ifft_pair_kernel  one block per pair of orders (m even, m + 1) and map:
 //       the transposed truncation puts the deconvolved coefficients c_j on j = 0..p;
 //       the transposed symmetric extension of the half grid folds them into the
 //       two-sided spectra U_j = c_j, U_{-j} = s c_j, U_0 = (1 + s) c_0 (s = +1 for
@@ -27,47 +29,99 @@
 //       warp = 4 nodes, weights in registers), staging each order tile's grid
 //       window through shared memory, and writes 32 contiguous orders per node
 //       row of Y.
-#include "fft_ct.cuh"
+#include "fft_ip.cuh"
 #include "plan.h"
 
 namespace hpx {
 
-template <int LOGM, int NT>
-__global__ void __launch_bounds__(NT, (LOGM <= 13 ? 1024 / NT : 1)) ifft_pair_ct_kernel(
-    const cplx<float>* __restrict__ bvec, cplx<float>* __restrict__ U, const float* __restrict__ dec,
-    const cplx<float>* __restrict__ tw, int twlen, int p, int L, int P2, int ldu) {
-    constexpr int M = 1 << LOGM;
+template <class T, int LOGM, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) ifft_pair_kernel(const cplx<T>* __restrict__ bvec, cplx<T>* __restrict__ U,
+                                                             const T* __restrict__ dec, const cplx<T>* __restrict__ tw,
+                                                             int twlen, int p, int L, int P2, int ldu) {
+    constexpr int M = 1 << LOGM, R = ip::out_radix(LOGM, NT);
     constexpr int H = M >> 1;
     extern __shared__ unsigned char smem_raw[];
-    cplx<float>* buf = reinterpret_cast<cplx<float>*>(smem_raw);   // M (padded)
+    cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);   // slots(M)
     const int m0 = 2 * blockIdx.x, m1 = m0 + 1;
     const int b = blockIdx.y;
     const int tid = threadIdx.x;
     const bool has1 = m1 <= L;
-    const cplx<float>* in0 = bvec + ((int64_t)b * (p + 1) + m0) * 2 * P2;
-    const cplx<float>* in1 = in0 + 2 * P2;
-    auto c0 = [&](int j) { return scale(in0[(j & 1) * P2 + (j >> 1)], dec[j]); };
-    auto c1 = [&](int j) {
-        if (!has1) return mk<float>(0.f, 0.f);
-        const cplx<float> v = in1[(j & 1) * P2 + (j >> 1)];
-        return scale(mk<float>(0.5f * v.i, -0.5f * v.r), dec[j]);   // conj(i/2) v
+    const cplx<T>* in0 = bvec + ((int64_t)b * (p + 1) + m0) * 2 * P2;
+    const cplx<T>* in1 = in0 + 2 * P2;
+    // c0_j + c1_j (lower half) or c0_j - c1_j (upper half), c1 = conj(i/2) v deconvolved
+    auto both = [&](int j, T sg) {
+        const int o = (j & 1) * P2 + (j >> 1);
+        const T d = dec[j];
+        cplx<T> v = scale(in0[o], d);
+        if (has1) {
+            const cplx<T> w = in1[o];
+            const T hd = sg * T(0.5) * d;
+            v = mk<T>(v.r + hd * w.i, v.i - hd * w.r);
+        }
+        return v;
     };
-    auto ld = [&](int j, int) {
-        if (j == 0) return scale(c0(0), 2.f);
-        if (j <= p) return add(c0(j), c1(j));
-        if (j >= M - p) return sub(c0(M - j), c1(M - j));
-        return mk<float>(0.f, 0.f);
+    // j = t + r M/16, t < M/16: r <= 4 can hold j <= p = M/4, r >= 12 j >= M - p
+    auto ld = [&](int j, int r) {
+        if (r > 4 && r < 12) return mk<T>(T(0), T(0));
+        if (j == 0) return scale(in0[0], T(2) * dec[0]);
+        if (j <= p) return both(j, T(1));
+        if (j >= M - p) return both(M - j, T(-1));
+        return mk<T>(T(0), T(0));
     };
-    ct::fft<float, LOGM, NT, true, false>(buf, tw, twlen >> LOGM, ld,
-                                          [&](int, int pi, cplx<float> v) { buf[pi] = v; });
-    cplx<float>* out0 = U + ((int64_t)b * (L + 1) + m0) * ldu;
-    cplx<float>* out1 = out0 + ldu;
+    ip::transform<T, LOGM, NT, true, R, R>(
+        buf, tw, twlen / M, tid, ld, [&](int k, int, int, cplx<T> v) { buf[ip::slot(k)] = v; });
+    __syncthreads();
+    cplx<T>* out0 = U + ((int64_t)b * (L + 1) + m0) * ldu;
+    cplx<T>* out1 = out0 + ldu;
     for (int t = tid; t <= H; t += NT) {
-        const cplx<float> z = buf[ct::padc(t)], zr = buf[ct::padc((M - t) & (M - 1))];
-        cplx<float> v0 = scale(add(z, zr), 0.5f);
-        if (t == 0 || t == H) v0 = scale(v0, 0.5f);
+        const cplx<T> z = buf[ip::slot(t)], zr = buf[ip::slot((M - t) & (M - 1))];
+        cplx<T> v0 = scale(add(z, zr), T(0.5));
+        if (t == 0 || t == H) v0 = scale(v0, T(0.5));
         out0[t] = v0;
-        if (has1) out1[t] = scale(sub(z, zr), 0.5f);
+        if (has1) out1[t] = scale(sub(z, zr), T(0.5));
+    }
+}
+
+// 32 nodes x 32 orders of one map per block (FP64, and runs wider than the
+// register-blocked form below takes): the grid window of the 32 orders is staged in
+// shared memory, lane = order, warp = 4 nodes.  nrw: odd row stride of the window.
+template <class T>
+__global__ void __launch_bounds__(256) interp_kernel(const cplx<T>* __restrict__ U, cplx<T>* __restrict__ Y,
+                                                     const int* __restrict__ tstart, const T* __restrict__ hwn, int E,
+                                                     int H, int p, int Q, int L, int ldu, int nrw) {
+    extern __shared__ unsigned char smem_raw[];
+    cplx<T>* out = reinterpret_cast<cplx<T>*>(smem_raw);   // [32 nodes][33]
+    cplx<T>* us = out + 32 * 33;                           // [32 orders][nrw]
+    const int r0 = blockIdx.x * 32, m0 = blockIdx.y * 32, b = blockIdx.z;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int T0 = tstart[r0];
+    const cplx<T>* ub = U + (int64_t)b * (L + 1) * ldu;
+    for (int ml = warp; ml < 32; ml += 8)
+        for (int tt = lane; tt < nrw; tt += 32) {
+            const int m = m0 + ml, t = T0 + tt;
+            us[ml * nrw + tt] = (m <= L && t <= H) ? ub[(int64_t)m * ldu + t] : mk<T>(T(0), T(0));
+        }
+    __syncthreads();
+    const int odd = lane & 1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int r = r0 + 4 * warp + j;
+        T ar = T(0), ai = T(0);
+        if (r < Q) {
+            const cplx<T>* ur = us + lane * nrw + (tstart[r] - T0);
+            const T* w = hwn + 2 * r + odd;
+            for (int e = 0; e < E; ++e) {
+                const T we = w[(size_t)e * 2 * Q];
+                ar += we * ur[e].r;
+                ai += we * ur[e].i;
+            }
+        }
+        out[(4 * warp + j) * 33 + lane] = mk<T>(ar, ai);
+    }
+    __syncthreads();
+    for (int rl = warp; rl < 32; rl += 8) {
+        const int r = r0 + rl, m = m0 + lane;
+        if (r < Q && m <= L) Y[((int64_t)b * Q + r) * (p + 1) + m] = out[rl * 33 + lane];
     }
 }
 
@@ -107,11 +161,13 @@ __global__ void __launch_bounds__(256, 2) interp_rb_kernel(const cplx<float>* __
     }
     const cplx<float>* ub = U + (int64_t)b * (L + 1) * ldu;
     auto fetch = [&](int m0, cplx<float>* us) {
-        for (int idx = tid; idx < 32 * nrw; idx += 256) {
-            const int ml = idx / nrw, tt = idx - ml * nrw;
-            const int m = m0 + ml, t = T0 + tt;
-            const bool ok = m <= L && t <= H;
-            cp_async8(us + idx, ok ? ub + (int64_t)m * ldu + t : ub, ok ? 8 : 0);
+        for (int ml = warp; ml < 32; ml += 8) {
+            const int m = m0 + ml;
+            const cplx<float>* row = ub + (int64_t)m * ldu + T0;
+            for (int tt = lane; tt < nrw; tt += 32) {
+                const bool ok = m <= L && T0 + tt <= H;
+                cp_async8(us + ml * nrw + tt, ok ? row + tt : ub, ok ? 8 : 0);
+            }
         }
         cp_async_commit2();
     };
@@ -150,35 +206,56 @@ __global__ void __launch_bounds__(256, 2) interp_rb_kernel(const cplx<float>* __
     }
 }
 
-// Returns false where these kernels do not apply (FP64 plans, grids outside
-// 4096..16384 points, wider interpolation runs); the caller then runs
-// nufft_adj_kernel.
+// Returns false at nside 2 (16 grid points); the caller then runs nufft_adj_kernel.
+template <class T>
 bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
     const auto& g = P->g;
     const auto& t = P->t;
     constexpr int EW = 12, DM = 4, NS = 3;
-    if (P->precision != HPX_FP32 || !t.tstart || t.interpE > EW || t.interpD > DM) return false;
+    constexpr bool F = sizeof(T) == 4;
     int logM = 0;
     while ((1 << logM) < g.M) ++logM;
-    if (logM < 12 || logM > 14) return false;
-    const size_t smem1 = (size_t)(g.M + g.M / 16) * sizeof(cplx<float>);
+    if (logM < 5) return false;
+    const size_t smem1 = (size_t)ip::slots(g.M) * sizeof(cplx<T>);
     dim3 grid1((g.L + 2) / 2, g.B);
     auto run1 = [&](auto kern, int threads) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
-        kern<<<grid1, threads, smem1, s>>>((const cplx<float>*)P->bvec, (cplx<float>*)P->U, (const float*)t.dec,
-                                           (const cplx<float>*)t.twid, g.Lmax, g.p, g.L, g.P2, P->ldu);
+        kern<<<grid1, threads, smem1, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->U, (const T*)t.dec,
+                                           (const cplx<T>*)t.twid, g.Lmax, g.p, g.L, g.P2, P->ldu);
     };
-    if (logM == 12) run1(ifft_pair_ct_kernel<12, 256>, 256);
-    else if (logM == 13) run1(ifft_pair_ct_kernel<13, 512>, 512);
-    else run1(ifft_pair_ct_kernel<14, 512>, 512);
-    const int nrw = (t.interpRows + EW + DM) | 1;
-    const size_t smem2 = (size_t)(32 * 33 + NS * 32 * nrw) * sizeof(cplx<float>);
-    auto kern2 = interp_rb_kernel<EW, DM, NS>;
-    cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
-    dim3 grid2((g.Q + 31) / 32, g.B);
-    kern2<<<grid2, 256, smem2, s>>>((const cplx<float>*)P->U, (cplx<float>*)P->Y, t.tstart, (const float*)t.hwn,
-                                    t.interpE, g.M / 2, g.p, g.Q, g.L, P->ldu, nrw);
+    // the shapes of the analysis' grid FFT (k_nufft.cu)
+    if (logM == 5) run1(ifft_pair_kernel<T, 5, 32, 1>, 32);
+    else if (logM == 6) run1(ifft_pair_kernel<T, 6, 32, 1>, 32);
+    else if (logM == 7) run1(ifft_pair_kernel<T, 7, 32, 1>, 32);
+    else if (logM == 8) run1(ifft_pair_kernel<T, 8, 32, 1>, 32);
+    else if (logM == 9) run1(ifft_pair_kernel<T, 9, 32, 1>, 32);
+    else if (logM == 10) run1(ifft_pair_kernel<T, 10, 64, 1>, 64);
+    else if (logM == 11) run1(ifft_pair_kernel<T, 11, 128, F ? 8 : 1>, 128);
+    else if (logM == 12) run1(ifft_pair_kernel<T, 12, 256, F ? 4 : 1>, 256);
+    else if (logM == 13) run1(ifft_pair_kernel<T, 13, 256, F ? 2 : 1>, 256);
+    else if constexpr (F) run1(ifft_pair_kernel<T, 14, 512, 1>, 512);
+    if constexpr (F) {
+        if (t.interpE <= EW && t.interpD <= DM) {
+            const int nrw = (t.interpRows - t.interpE + EW + DM) | 1;   // first window start .. last window end
+            const size_t smem2 = (size_t)(32 * 33 + NS * 32 * nrw) * sizeof(cplx<float>);
+            auto kern2 = interp_rb_kernel<EW, DM, NS>;
+            cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+            dim3 grid2((g.Q + 31) / 32, g.B);
+            kern2<<<grid2, 256, smem2, s>>>((const cplx<float>*)P->U, (cplx<float>*)P->Y, t.tstart,
+                                            (const float*)t.hwn, t.interpE, g.M / 2, g.p, g.Q, g.L, P->ldu, nrw);
+            return true;
+        }
+    }
+    const int nrw = t.interpRows | 1;
+    const size_t smem2 = (size_t)(32 * 33 + 32 * nrw) * sizeof(cplx<T>);
+    cudaFuncSetAttribute(interp_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+    dim3 grid2((g.Q + 31) / 32, (g.L + 32) / 32, g.B);
+    interp_kernel<T><<<grid2, 256, smem2, s>>>((const cplx<T>*)P->U, (cplx<T>*)P->Y, t.tstart, (const T*)t.hwn,
+                                               t.interpE, g.M / 2, g.p, g.Q, g.L, P->ldu, nrw);
     return true;
 }
+
+template bool launch_nufft2<float>(const hpx_plan_s*, cudaStream_t);
+template bool launch_nufft2<double>(const hpx_plan_s*, cudaStream_t);
 
 }  // namespace hpx
