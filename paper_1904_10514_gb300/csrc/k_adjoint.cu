@@ -594,7 +594,14 @@ template <class T>
 void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, T wpos) {
     const auto& g = P->g;
     const auto& t = P->t;
-    {
+    if (P->fusedM) {   // the plan's operators, transposed
+        if constexpr (sizeof(T) == 4) {
+            if (P->use_tc) launch_adjoint_tc(P, (const float*)alm, s, (float)wpos);
+            else launch_operator_cols<T>(P, P->fusedM, g.B <= 8, alm, s, wpos, true);
+        } else {
+            launch_operator_cols<T>(P, P->fusedM, false, alm, s, wpos, true);
+        }
+    } else {
         const int ngroups = (2 * g.B + 31) / 32;
         const int nitems = (g.L + 1) * 2 * ngroups;
         const int blocks = (nitems * 32 + 127) / 128;
@@ -606,8 +613,6 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
         else
             rot_adj_kernel<T, KMAX><<<blocks, 128, 0, s>>>(alm, (T*)P->beta, t.skOff, (const cplx<T>*)t.skewT, t.nq,
                                                            g.P2, g.L, g.p, g.B, g.nalm, ngroups, nitems, wpos, true);
-    }
-    {
         const int nmp = g.L / 2 + 1;
         dim3 grid((nmp * g.B + AC - 1) / AC, (g.P2 + AK - 1) / AK, 4);
         dense_adj_kernel<T><<<grid, 256, 0, s>>>((const T*)t.D, (const cplx<T>*)P->beta, (cplx<T>*)P->bvec, g.P2,
@@ -652,7 +657,7 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
     if (sizeof(T) == 4 && P->synT) {
         launch_synth_tc(P, (const float*)alm, s);   // the same operators on the tensor cores
     } else if (P->synM) {
-        launch_synth_apply<T>(P, alm, s);   // the sweeps and Es composed per (m, c)
+        launch_operator_cols<T>(P, P->synM, false, alm, s, T(1), false);   // the sweeps and Es composed per (m, c)
     } else {
         const int ngroups = (2 * g.B + 31) / 32;
         const int nitems = (g.L + 1) * 2 * ngroups;

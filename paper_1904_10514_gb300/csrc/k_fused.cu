@@ -386,99 +386,154 @@ __global__ void __launch_bounds__(256) fused_rows_kernel(const T* __restrict__ M
     }
 }
 
-// ---------------------------------------------------------------- synthesis apply
-// The synthesis direction of the same composition: with Es the Legendre-0/1 ->
-// latitude-Fourier table in place of D, the build gives S_{m,c} = R_{m,c} Es
-// (rows i = degrees of the chain, columns k = latitude modes), and the
-// cosine/sine coefficients of F_m are the transposed contraction
-//     X[map][m][par][k] = sum_i S_{m,c}[i][k] a_{m+c+2i}^m[map].
-// Block = one (m, c, tile of 128 modes) x MB maps (16, or 32 so that batches of
-// 17+ maps read each operator once); 256 threads, each 4 modes x MB/8 maps;
-// degrees in chunks of 16 staged in shared memory.
-template <class T, int MB>
-__global__ void __launch_bounds__(256) synth_apply_kernel(const T* __restrict__ S, const int64_t* __restrict__ moff,
-                                                          const cplx<T>* __restrict__ alm, cplx<T>* __restrict__ bvec,
-                                                          int P2, int ldm, int p, int L, int B, int64_t nalm,
-                                                          int nkt) {
-    constexpr int KT = 128, IC = 16, QB = MB / 8;
-    __shared__ __align__(16) T As[IC][KT];
-    __shared__ cplx<T> Bs[IC][MB];
-    const int item = blockIdx.x;
-    const int kt = item % nkt, mc = item / nkt;
+// ---------------------------------------------------------------- transposed
+// The transposed contraction X[map][m][par][k] = sum_i O_{m,c}[i][k] a_{m+c+2i}^m[map] of
+// the same operators, 0 <= k < P2: the adjoint's first two stages (O = M, with the
+// coefficients' weights and without the imaginary parts that the analysis never
+// returns) and the synthesis' (O = S_{m,c} = R_{m,c} Es, built with Es, the
+// Legendre-0/1 -> latitude-Fourier table, in place of D: X are then the cosine / sine
+// coefficients of F_m).
+struct CoefWeights {
+    double pos;    // weight of the m > 0 coefficients (m = 0: 1)
+    bool dropim;   // ignore the imaginary parts at m = 0 and m = p
+};
+template <class T>
+__device__ __forceinline__ cplx<T> weighted(cplx<T> v, int m, int p, CoefWeights w) {
+    if (m > 0) v = scale(v, (T)w.pos);
+    if (w.dropim && (m == 0 || m == p)) v.i = T(0);
+    return v;
+}
+
+// FP64 plans and FP32 plans off the tensor cores.  A block takes one (m, c), NB maps
+// and 32 lanes x 16 bytes of k; its four warps take 32 rows each of every 128, the
+// coefficients of the rows sit in shared memory (read as broadcasts), each lane sums
+// its k over the warp's rows, and the four partial sums are added in warp order at
+// the end.  QUAD: the operator is in the groups of fused_quad_kernel, else row-major.
+// FP32 is bound by the operator's stream, FP64 by the FP64 pipe.  6 maps,
+// Nside 256, lmax 400 (synthesis): 96 us as matrix-matrix tiles, now 65 us.
+template <class T, int NB, bool QUAD>
+__global__ void __launch_bounds__(128) operator_cols_kernel(const T* __restrict__ M, const int64_t* __restrict__ moff,
+                                                            const cplx<T>* __restrict__ alm,
+                                                            cplx<T>* __restrict__ bvec, int P2, int ldm, int p, int L,
+                                                            int B, int64_t nalm, int nkt, CoefWeights w) {
+    constexpr int VA = 16 / sizeof(T), NC = 2 * NB, KT = 32 * VA;
+    __shared__ __align__(16) T as[128][NC];
+    __shared__ T red[3][VA * NC][32];
+    const int kt = blockIdx.x % nkt, mc = blockIdx.x / nkt;
     const int m = mc >> 1, c = mc & 1;
     const int par = ((m & 1) + c) & 1;
-    const int nrows = chain_len(m, c, L);
-    const int k0 = kt * KT, b0 = blockIdx.y * MB;
-    const T* A = S + moff[(size_t)m * 2 + c] * ldm;
+    const int n = chain_len(m, c, L);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int k = kt * KT + lane * VA, b0 = blockIdx.y * NB;
+    const bool on = k < P2;   // ldm >= k + VA: rows are padded to 4
+    const T* A = M + moff[(size_t)m * 2 + c] * ldm;
     const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2 + m + c;
-    const int tid = threadIdx.x, tk = tid & 31, tb = tid >> 5;
-    T accr[4][QB], acci[4][QB];
+    T acc[VA][NC];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < VA; ++a)
 #pragma unroll
-        for (int q = 0; q < QB; ++q) { accr[a][q] = T(0); acci[a][q] = T(0); }
-    for (int i0 = 0; i0 < nrows; i0 += IC) {
-        for (int e = tid; e < IC * KT; e += 256) {
-            const int ii = e / KT, kk = e % KT;
-            const int i = i0 + ii, k = k0 + kk;
-            As[ii][kk] = (i < nrows && k < ldm) ? A[(size_t)i * ldm + k] : T(0);
-        }
-        for (int e = tid; e < IC * MB; e += 256) {
-            const int ii = e / MB, bb = e % MB;
-            const int i = i0 + ii, b = b0 + bb;
-            Bs[ii][bb] = (i < nrows && b < B) ? alm[(int64_t)b * nalm + base + 2 * i] : mk<T>(T(0), T(0));
+        for (int q = 0; q < NC; ++q) acc[a][q] = T(0);
+    for (int r0 = 0; r0 < n; r0 += 128) {
+        for (int e = threadIdx.x; e < 128 * NB; e += 128) {
+            const int q = e >> 7, i = r0 + (e & 127);
+            cplx<T> v = mk<T>(T(0), T(0));
+            if (i < n && b0 + q < B) v = weighted<T>(alm[(int64_t)(b0 + q) * nalm + base + 2 * i], m, p, w);
+            as[e & 127][2 * q] = v.r;
+            as[e & 127][2 * q + 1] = v.i;
         }
         __syncthreads();
+        const int g0 = r0 + 32 * warp, cnt = min(32, n - g0);
+        if (on && cnt > 0) {
+            // row i of the group: stride between rows and first element
+            const T* row = QUAD ? A + (int64_t)g0 * ldm + (int64_t)(k >> 2) * 4 * cnt : A + (int64_t)g0 * ldm + k;
+            const int64_t step = QUAD ? 4 : ldm;
+            auto one = [&](int i, const T (&v)[VA]) {
+                const T* x = as[32 * warp + i];
 #pragma unroll
-        for (int ii = 0; ii < IC; ++ii) {
-            T a[4];
+                for (int q = 0; q < NC; ++q)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) a[r] = As[ii][tk * 4 + r];
-            cplx<T> x[QB];
-#pragma unroll
-            for (int q = 0; q < QB; ++q) x[q] = Bs[ii][tb * QB + q];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int q = 0; q < QB; ++q) {
-                    accr[r][q] += a[r] * x[q].r;
-                    acci[r][q] += a[r] * x[q].i;
+                    for (int a = 0; a < VA; ++a) acc[a][q] = fma(v[a], x[q], acc[a][q]);
+            };
+            auto load = [&](int i, T (&v)[VA]) {
+                if constexpr (sizeof(T) == 4) {
+                    const float4 f = __ldg(reinterpret_cast<const float4*>(row + i * step));
+                    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+                } else {
+                    const double2 f = __ldg(reinterpret_cast<const double2*>(row + i * step));
+                    v[0] = f.x; v[1] = f.y;
                 }
+            };
+            int i = 0;
+            for (; i + 8 <= cnt; i += 8) {
+                T v[8][VA];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) load(i + u, v[u]);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) one(i + u, v[u]);
+            }
+            for (; i < cnt; ++i) {
+                T v[VA];
+                load(i, v);
+                one(i, v);
+            }
         }
         __syncthreads();
     }
+    if (warp > 0)
 #pragma unroll
-    for (int q = 0; q < QB; ++q) {
-        const int b = b0 + tb * QB + q;
-        if (b >= B) continue;
-        cplx<T>* out = bvec + (((int64_t)b * (p + 1) + m) * 2 + par) * P2;
+        for (int a = 0; a < VA; ++a)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int k = k0 + tk * 4 + r;
-            if (k < P2) out[k] = mk<T>(accr[r][q], acci[r][q]);
-        }
+            for (int q = 0; q < NC; ++q) red[warp - 1][a * NC + q][lane] = acc[a][q];
+    __syncthreads();
+    if (warp > 0 || !on) return;
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+#pragma unroll
+        for (int a = 0; a < VA; ++a)
+#pragma unroll
+            for (int q = 0; q < NC; ++q) acc[a][q] += red[u][a * NC + q][lane];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        if (b0 + q >= B) continue;
+        cplx<T>* out = bvec + (((int64_t)(b0 + q) * (p + 1) + m) * 2 + par) * P2 + k;
+#pragma unroll
+        for (int a = 0; a < VA; ++a)
+            if (k + a < P2) out[a] = mk<T>(acc[a][2 * q], acc[a][2 * q + 1]);
     }
 }
 
 template <class T>
-void launch_synth_apply(const hpx_plan_s* P, const T* alm, cudaStream_t s) {
+void launch_operator_cols(const hpx_plan_s* P, const void* M, bool quad, const T* alm, cudaStream_t s, T wpos,
+                          bool dropim) {
     const auto& g = P->g;
-    const int nkt = (g.P2 + 127) / 128;
-    if (g.B > 16) {
-        dim3 grid((g.L + 1) * 2 * nkt, (g.B + 31) / 32);
-        synth_apply_kernel<T, 32><<<grid, 256, 0, s>>>((const T*)P->synM, P->fusedOff, (const cplx<T>*)alm,
-                                                       (cplx<T>*)P->bvec, g.P2, P->fused_ldm, g.p, g.L, g.B, g.nalm,
-                                                       nkt);
-    } else {
-        dim3 grid((g.L + 1) * 2 * nkt, (g.B + 15) / 16);
-        synth_apply_kernel<T, 16><<<grid, 256, 0, s>>>((const T*)P->synM, P->fusedOff, (const cplx<T>*)alm,
-                                                       (cplx<T>*)P->bvec, g.P2, P->fused_ldm, g.p, g.L, g.B, g.nalm,
-                                                       nkt);
+    const int kt = 32 * 16 / sizeof(T), nkt = (g.P2 + kt - 1) / kt;
+    // maps per block as launch_fused: FP32 as many as possible (8), FP64 no absent ones
+    const int nb = sizeof(T) == 4 ? (g.B > 4 ? 8 : g.B > 2 ? 4 : g.B)
+                                  : (g.B + (g.B + 3) / 4 - 1) / ((g.B + 3) / 4);
+    auto run = [&](auto kern, int NB) {
+        dim3 grid((g.L + 1) * 2 * nkt, (g.B + NB - 1) / NB);
+        kern<<<grid, 128, 0, s>>>((const T*)M, P->fusedOff, (const cplx<T>*)alm, (cplx<T>*)P->bvec, g.P2,
+                                  P->fused_ldm, g.p, g.L, g.B, g.nalm, nkt, CoefWeights{(double)wpos, dropim});
+    };
+    if constexpr (sizeof(T) == 4) {
+        if (quad) {
+            if (nb == 1) run(operator_cols_kernel<T, 1, true>, 1);
+            else if (nb == 2) run(operator_cols_kernel<T, 2, true>, 2);
+            else if (nb == 4) run(operator_cols_kernel<T, 4, true>, 4);
+            else run(operator_cols_kernel<T, 8, true>, 8);
+            return;
+        }
     }
+    if (nb == 1) run(operator_cols_kernel<T, 1, false>, 1);
+    else if (nb == 2) run(operator_cols_kernel<T, 2, false>, 2);
+    else if (nb == 4) run(operator_cols_kernel<T, 4, false>, 4);
+    else if constexpr (sizeof(T) == 4) run(operator_cols_kernel<T, 8, false>, 8);
+    else run(operator_cols_kernel<T, 3, false>, 3);
 }
 
-template void launch_synth_apply<float>(const hpx_plan_s*, const float*, cudaStream_t);
-template void launch_synth_apply<double>(const hpx_plan_s*, const double*, cudaStream_t);
+template void launch_operator_cols<float>(const hpx_plan_s*, const void*, bool, const float*, cudaStream_t, float, bool);
+template void launch_operator_cols<double>(const hpx_plan_s*, const void*, bool, const double*, cudaStream_t, double,
+                                           bool);
 
 // Rows per block of the apply kernels (the plan builds its tile list with this).
 int fused_tile_rows(bool fp64) { return fp64 ? kFusedRows : 128; }
