@@ -39,3 +39,20 @@ def test_operators_match_sweeps(nside, lmax, B, prec):
         u, v = u.reshape(B, -1), v.reshape(B, -1)
         d = torch.linalg.vector_norm(u - v, dim=1) / torch.linalg.vector_norm(v, dim=1)
         assert float(d.max()) <= TOL[prec], (name, d)
+
+
+@pytest.mark.parametrize("B", [8, 9, 33])
+@pytest.mark.parametrize("nside,lmax", [(16, 21), (64, 128)])
+def test_equal_weight_analysis(nside, lmax, B):
+    """hpx_healpix_analysis through the transposed synthesis tiles."""
+    import paper_1904_10514_gb300 as hp
+    x = torch.as_tensor(np.random.default_rng(B).standard_normal((B, 12 * nside * nside)), dtype=torch.float32,
+                        device="cuda")
+    out = []
+    for sweeps in (False, True):
+        plan = hp.Plan(nside, lmax, B, "fp32", sweeps=sweeps, synthesis=True)
+        out.append(plan.healpix_analysis(x, niter=1).clone())
+        torch.cuda.synchronize()
+        plan.close()
+    d = torch.linalg.vector_norm(out[0] - out[1], dim=1) / torch.linalg.vector_norm(out[1], dim=1)
+    assert float(d.max()) <= TOL["fp32"], d
