@@ -615,8 +615,9 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
                                                            g.P2, g.L, g.p, g.B, g.nalm, ngroups, nitems, wpos, true);
         const int nmp = g.L / 2 + 1;
         dim3 grid((nmp * g.B + AC - 1) / AC, (g.P2 + AK - 1) / AK, 4);
-        dense_adj_kernel<T><<<grid, 256, 0, s>>>((const T*)t.D, (const cplx<T>*)P->beta, (cplx<T>*)P->bvec, g.P2,
-                                                 g.p, g.L, g.B);
+        if (sizeof(T) == 8 || !launch_dense_adj_big(P, s, t.D))
+            dense_adj_kernel<T><<<grid, 256, 0, s>>>((const T*)t.D, (const cplx<T>*)P->beta, (cplx<T>*)P->bvec, g.P2,
+                                                     g.p, g.L, g.B);
     }
     {
         int logM = 0;
@@ -672,8 +673,9 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
                                                            g.P2, g.L, g.p, g.B, g.nalm, ngroups, nitems, T(1), false);
         const int nmp = g.L / 2 + 1;
         dim3 grid((nmp * g.B + AC - 1) / AC, (g.P2 + AK - 1) / AK, 4);
-        dense_adj_kernel<T><<<grid, 256, 0, s>>>((const T*)t.Es, (const cplx<T>*)P->beta, (cplx<T>*)P->bvec, g.P2,
-                                                 g.p, g.L, g.B);
+        if (sizeof(T) == 8 || !launch_dense_adj_big(P, s, t.Es))
+            dense_adj_kernel<T><<<grid, 256, 0, s>>>((const T*)t.Es, (const cplx<T>*)P->beta, (cplx<T>*)P->bvec, g.P2,
+                                                     g.p, g.L, g.B);
     }
     if (ev) cudaEventRecord(ev[1], s);
     {

@@ -226,6 +226,9 @@ template <class T> void launch_lat_fft(const hpx_plan_s* P, cudaStream_t s, bool
 bool packs_b(const hpx_plan_s* P);
 
 template <class T> void launch_dense(const hpx_plan_s* P, cudaStream_t s, const void* Dmat = nullptr);
+// the transposed contraction (beta -> bvec) of an FP32 plan with D or another table of its shape;
+// false for small ones (then dense_adj_kernel)
+bool launch_dense_adj_big(const hpx_plan_s* P, cudaStream_t s, const void* Dmat);
 template <class T> void launch_cg(const hpx_plan_s* P, cudaStream_t s);
 template <class T> void launch_rot(const hpx_plan_s* P, T* alm, cudaStream_t s);
 int fused_tile_rows(bool fp64);
