@@ -508,14 +508,14 @@ void tune_shapes(hpx_plan_s* P, const void* maps, void* alm, cudaEvent_t e0, cud
         const float t4 = time_stage(P, maps, alm, 0, e0, e1);
         P->ringForm = t4 < t[P->ringE == 32 ? 1 : 0] ? 1 : 0;
     }
-    P->rotForm = 0;
+    P->rotForm = 2;
     if (sweeps) {   // the three forms of the sweep kernel
         float best = 0.f;
-        for (int f = 0; f < 3; ++f) {
+        for (int f = 2; f >= 0; --f) {
             const int keep = P->rotForm;
             P->rotForm = f;
             const float tf = time_stage(P, maps, alm, 2, e0, e1);
-            if (f == 0 || tf < best) best = tf;
+            if (f == 2 || tf < best) best = tf;
             else P->rotForm = keep;
         }
     }

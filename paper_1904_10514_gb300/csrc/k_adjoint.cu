@@ -146,13 +146,21 @@ __device__ __forceinline__ void sweep_pass_adj_staged(float* chain, int64_t ldc,
         const cplx<float>* slot = ring + (t % RB) * SL;
         const float x0 = reinterpret_cast<const float*>(slot + 32)[lane];
         const cplx<float>* row = slot + coff;
-#pragma unroll
-        for (int k = K - 1; k >= 0; --k) {
-            const float x = (k == 0) ? x0 : pipe[k - 1];
-            const cplx<float> cs = row[k];
+        auto rotate = [&](int k, cplx<float> cs, float x) {
             const float o = cs.i * x + cs.r * carry[k];
             carry[k] = cs.r * x - cs.i * carry[k];
             pipe[k] = o;
+        };
+        if constexpr (K == 1) {
+            rotate(0, row[0], x0);
+        } else {
+#pragma unroll
+            for (int k = K - 2; k >= 0; k -= 2) {   // two stages per 16-byte read (coff is even)
+                cplx<float> ca, cb;
+                load2(row + k, ca, cb);
+                rotate(k + 1, cb, pipe[k]);
+                rotate(k, ca, k == 0 ? x0 : pipe[k - 1]);
+            }
         }
         const int j = n_in + 2 * K - 2 - t;
         if (live && j >= 0 && j < n_in + K) chain[(int64_t)j * ldc] = pipe[K - 1];
@@ -161,13 +169,16 @@ __device__ __forceinline__ void sweep_pass_adj_staged(float* chain, int64_t ldc,
     __syncwarp();
 }
 
-// rot_adj_kernel for FP32 with the staged passes (one real column per lane,
-// warps of 2 per block; the whole warp stays in the passes).
+// rot_adj_kernel for FP32 with the staged passes: one real column per lane and G
+// orders of one parity and chain per warp, as rot_staged_real_kernel of the forward
+// sweeps: sweep S0 + q is undone for the orders i > q, q descending, then the first
+// S0 sweeps of all of them (warps of 2 per block; the whole warp stays in the
+// passes).  8 maps, Nside 2048: 73 ms with one order per warp, now 40.4 ms
 template <int KMAX>
 __global__ void __launch_bounds__(64, 8) rot_adj_staged_kernel(const float* __restrict__ alm, float* __restrict__ beta2,
                                                               const int64_t* __restrict__ skOff,
                                                               const cplx<float>* __restrict__ skewT, int nq, int P2,
-                                                              int L, int p, int B, int64_t nalm, int ngroups,
+                                                              int L, int p, int B, int64_t nalm, int G, int ngroups,
                                                               int nitems, float wpos, bool dropim) {
     constexpr int RB = 8;
     constexpr int SL = SweepRing<RB>::kSlot;
@@ -177,19 +188,20 @@ __global__ void __launch_bounds__(64, 8) rot_adj_staged_kernel(const float* __re
     if (warp >= nitems) return;   // whole warps leave together
     cplx<float>* ring = rings[(threadIdx.x >> 5) & 1];
     const int g = warp % ngroups;
-    const int c = (warp / ngroups) & 1;
-    const int m = L - warp / (2 * ngroups);
-    const int m0 = m & 1;
-    const int S = (m - m0) >> 1;
+    const int c = (warp / ngroups) & 1, m0 = (warp / (2 * ngroups)) & 1;
+    const int S0 = G * (L / 2 / G - warp / (4 * ngroups));
+    if (m0 + 2 * S0 > L) return;
+    const int W = 32 / G, o = lane / W;
+    const int m = m0 + 2 * (S0 + o);
     const int ncol = 2 * B;
-    const int col = 32 * g + lane;
-    const bool live = col < ncol;
+    const int col = 32 * g + lane - o * W;
+    const bool live = col < ncol && m <= L;
     const int par = (m0 + c) & 1;
     const int q0 = (m0 == 1 && c == 1) ? 1 : 0;
-    float* chain = beta2 + (((int64_t)m * 2 + par) * P2 + q0) * ncol + (live ? col : 0);
+    float* chain = live ? beta2 + (((int64_t)m * 2 + par) * P2 + q0) * ncol + col : beta2;
     const int64_t ldc = ncol;
-    int n = chain_len(m, c, L);
     if (live) {   // order-m chain from the weighted input coefficients
+        const int n = chain_len(m, c, L);
         const int b = col >> 1, ri = col & 1;
         const float w = (m == 0) ? 1.f : wpos;
         const bool drop = dropim && ri == 1 && (m == 0 || m == p);
@@ -198,12 +210,18 @@ __global__ void __launch_bounds__(64, 8) rot_adj_staged_kernel(const float* __re
         for (int i = 0; i < n; ++i) chain[(int64_t)i * ldc] = drop ? 0.f : w * in[(base + 2 * i) * 2];
     }
     __syncwarp();
-    const int F = S / KMAX, r = S % KMAX;
     auto block = [&](int s_lo, int K) {
         const int e = 32 - (s_lo & 31) - K;
         return skewT + (skOff[(size_t)(m0 * 2 + c) * nq + (s_lo >> 5)] + e) * 32;
     };
     auto coff = [&](int s_lo, int K) { return 32 - (s_lo & 31) - K; };
+    for (int q = G - 2; q >= 0; --q) {
+        if (m0 + 2 * (S0 + q + 1) > L) continue;
+        sweep_pass_adj_staged<1, RB>(chain, ldc, chain_len(m0 + 2 * (S0 + q + 1), c, L), live && o > q,
+                                     block(S0 + q, 1), coff(S0 + q, 1), ring);
+    }
+    int n = chain_len(m0 + 2 * S0, c, L);
+    const int F = S0 / KMAX, r = S0 % KMAX;
 #define HPX_SUBPASS_ADJ(KK)                                                                        \
     if (KK < KMAX && (r & KK)) {                                                                   \
         const int s_lo = F * KMAX + (r & ~(2 * KK - 1));                                           \
@@ -604,12 +622,14 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
     } else {
         const int ngroups = (2 * g.B + 31) / 32;
         const int nitems = (g.L + 1) * 2 * ngroups;
+        const int G = sweep_orders_per_warp(g.B), sitems = (g.L / 2 / G + 1) * 4 * ngroups;
+        (void)G; (void)sitems; (void)nitems;
         const int blocks = (nitems * 32 + 127) / 128;
         constexpr int KMAX = sizeof(T) == 4 ? 32 : 16;
         if constexpr (sizeof(T) == 4)   // angle rows and inputs staged ahead of use
-            rot_adj_staged_kernel<32><<<(nitems * 32 + 63) / 64, 64, 0, s>>>(
+            rot_adj_staged_kernel<32><<<(sitems * 32 + 63) / 64, 64, 0, s>>>(
                 (const float*)alm, (float*)P->beta, t.skOff, (const cplx<float>*)t.skewT, t.nq, g.P2, g.L, g.p, g.B,
-                g.nalm, ngroups, nitems, (float)wpos, true);
+                g.nalm, G, ngroups, sitems, (float)wpos, true);
         else
             rot_adj_kernel<T, KMAX><<<blocks, 128, 0, s>>>(alm, (T*)P->beta, t.skOff, (const cplx<T>*)t.skewT, t.nq,
                                                            g.P2, g.L, g.p, g.B, g.nalm, ngroups, nitems, wpos, true);
@@ -662,12 +682,14 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
     } else {
         const int ngroups = (2 * g.B + 31) / 32;
         const int nitems = (g.L + 1) * 2 * ngroups;
+        const int G = sweep_orders_per_warp(g.B), sitems = (g.L / 2 / G + 1) * 4 * ngroups;
+        (void)G; (void)sitems; (void)nitems;
         const int blocks = (nitems * 32 + 127) / 128;
         constexpr int KMAX = sizeof(T) == 4 ? 32 : 16;
         if constexpr (sizeof(T) == 4)
-            rot_adj_staged_kernel<32><<<(nitems * 32 + 63) / 64, 64, 0, s>>>(
+            rot_adj_staged_kernel<32><<<(sitems * 32 + 63) / 64, 64, 0, s>>>(
                 (const float*)alm, (float*)P->beta, t.skOff, (const cplx<float>*)t.skewT, t.nq, g.P2, g.L, g.p, g.B,
-                g.nalm, ngroups, nitems, 1.f, false);
+                g.nalm, G, ngroups, sitems, 1.f, false);
         else
             rot_adj_kernel<T, KMAX><<<blocks, 128, 0, s>>>(alm, (T*)P->beta, t.skOff, (const cplx<T>*)t.skewT, t.nq,
                                                            g.P2, g.L, g.p, g.B, g.nalm, ngroups, nitems, T(1), false);

@@ -87,44 +87,52 @@ __global__ void __launch_bounds__(64, (KMAX == 32 ? 6 : 10)) rot_staged_kernel(c
     for (int i = 0; i < n; ++i) out[base + 2 * i] = chain[(int64_t)i * ldc];
 }
 
-// FP32, one real column per lane (sweep_pass_staged_real): warp = (m, chain c,
-// group of 32 real columns: re and im of 16 maps), so a batch of B maps fills
-// 2B lanes.  Output: the lane's part of a_{m+c+2i}^m.
+// FP32, one real column per lane (sweep_pass_staged_real).  The sweep from order m' to
+// m' + 2 is the same for every order above m', so a warp takes G = 32 / W orders m0 +
+// 2 (S0 + i), i < G, of one parity m0 and chain c together, W = the power of two >= 2B
+// lanes each (re and im of the maps; G = 1 and 2B columns in groups of 32 from 16
+// maps on): the first S0 sweeps of all of them, then sweep S0 + q for the orders
+// i > q.  8 maps, Nside 2048: 147 ms with one complex column per lane (8 of 32 lanes
+// busy), now 41.4 ms
 template <int KMAX>
 __global__ void __launch_bounds__(64, 8) rot_staged_real_kernel(cplx<float>* __restrict__ beta2,
                                                                cplx<float>* __restrict__ alm,
                                                                const int64_t* __restrict__ skOff,
                                                                const cplx<float>* __restrict__ skew, int nq, int P2,
-                                                               int L, int B, int64_t nalm, int ngroups, int nitems) {
+                                                               int L, int B, int64_t nalm, int G, int ngroups,
+                                                               int nitems) {
     constexpr int SL = SweepRing<kRotRing>::kSlot;
     __shared__ __align__(16) cplx<float> rings[2][kRotRing * SL];
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= nitems) return;   // whole warps leave together (nitems counts warps)
     cplx<float>* ring = rings[(threadIdx.x >> 5) & 1];
+    // items: (order group descending, parity, chain, column group)
     const int g = warp % ngroups;
-    const int c = (warp / ngroups) & 1;
-    const int m = L - warp / (2 * ngroups);
-    const int m0 = m & 1;
-    const int S = (m - m0) >> 1;
-    const int rc = 32 * g + lane;   // real column: 2 map + part
-    const bool live = rc < 2 * B;
+    const int c = (warp / ngroups) & 1, m0 = (warp / (2 * ngroups)) & 1;
+    const int S0 = G * (L / 2 / G - warp / (4 * ngroups));
+    const int W = 32 / G, i = lane / W;
+    const int m = m0 + 2 * (S0 + i);
+    if (m0 + 2 * S0 > L) return;   // (odd orders end one group earlier)
+    const int rc = 32 * g + lane - i * W;   // real column: 2 map + part
+    const bool live = rc < 2 * B && m <= L;
     const int par = (m0 + c) & 1;
     const int q0 = (m0 == 1 && c == 1) ? 1 : 0;
-    float* chain = reinterpret_cast<float*>(beta2 + (((int64_t)m * 2 + par) * P2 + q0) * B) + (live ? rc : 0);
+    float* chain = reinterpret_cast<float*>(beta2 + (((int64_t)m * 2 + par) * P2 + q0) * B) + rc;
+    if (!live) chain = reinterpret_cast<float*>(beta2);
     const int64_t ldc = 2 * (int64_t)B;
     int n = chain_len(m0, c, L);
     int s0 = 0;
     auto block = [&](int s) {
         return skew + (skOff[(size_t)(m0 * 2 + c) * nq + (s >> 5)] + 2 * (s & 31)) * 32;
     };
-    while (S - s0 >= KMAX && n > 0) {
+    while (S0 - s0 >= KMAX && n > 0) {
         sweep_pass_staged_real<KMAX, kRotRing>(chain, ldc, n, live, block(s0), s0 & 31, ring);
         n -= KMAX;
         s0 += KMAX;
     }
 #define HPX_SUBPASS(KK)                                                                      \
-    if (KK < KMAX && S - s0 >= KK && n > 0) {                                                \
+    if (KK < KMAX && S0 - s0 >= KK && n > 0) {                                               \
         sweep_pass_staged_real<KK, kRotRing>(chain, ldc, n, live, block(s0), s0 & 31, ring); \
         n -= KK;                                                                             \
         s0 += KK;                                                                            \
@@ -135,10 +143,13 @@ __global__ void __launch_bounds__(64, 8) rot_staged_real_kernel(cplx<float>* __r
     HPX_SUBPASS(2)
     HPX_SUBPASS(1)
 #undef HPX_SUBPASS
+    for (int q = 0; q < G - 1 && n > 0 && m0 + 2 * (S0 + q + 1) <= L; ++q, --n)
+        sweep_pass_staged_real<1, kRotRing>(chain, ldc, n, live && i > q, block(S0 + q), (S0 + q) & 31, ring);
     if (!live) return;
     float* out = reinterpret_cast<float*>(alm + (int64_t)(rc >> 1) * nalm) + (rc & 1);
     const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2 + m + c;
-    for (int i = 0; i < n; ++i) out[2 * (base + 2 * i)] = chain[(int64_t)i * ldc];
+    const int len = chain_len(m, c, L);
+    for (int j = 0; j < len; ++j) out[2 * (base + 2 * j)] = chain[(int64_t)j * ldc];
 }
 
 template <class T, int KMAX>
@@ -297,15 +308,16 @@ void launch_rot(const hpx_plan_s* P, T* alm, cudaStream_t s) {
         const int threads = 64;
         const int blocks = (nitems * 32 + threads - 1) / threads;
         if constexpr (sizeof(T) == 4) {
-            // the plan's form (HPX_FLAG_AUTOTUNE): one complex column per lane with 32
-            // stages per pass (168 registers, 12 warps per SM) or 16 (twice the passes
-            // over the chains, 20 warps per SM), or one real column per lane with 32
-            // stages (128 registers, 16 warps per SM, 2B lanes for B maps)
+            // the plan's form: one real column per lane with 32 stages (2, the default:
+            // the fastest measured at 8 and at 32 maps), or by HPX_FLAG_AUTOTUNE one
+            // complex column per lane with 32 stages per pass (168 registers, 12 warps
+            // per SM) or 16 (twice the passes over the chains, 20 warps per SM)
             if (P->rotForm == 2) {   // one real column per lane
-                const int rgroups = (2 * g.B + 31) / 32, ritems = (g.L + 1) * 2 * rgroups;
+                const int G = sweep_orders_per_warp(g.B);
+                const int rgroups = (2 * g.B + 31) / 32, ritems = (g.L / 2 / G + 1) * 4 * rgroups;
                 rot_staged_real_kernel<32><<<(ritems * 32 + threads - 1) / threads, threads, 0, s>>>(
                     (cplx<float>*)P->beta, (cplx<float>*)alm, P->t.skOff, (const cplx<float>*)P->t.skew, P->t.nq,
-                    g.P2, g.L, g.B, g.nalm, rgroups, ritems);
+                    g.P2, g.L, g.B, g.nalm, G, rgroups, ritems);
             } else if (P->rotForm == 1)
                 rot_staged_kernel<16><<<blocks, threads, 0, s>>>((cplx<float>*)P->beta, (cplx<float>*)alm,
                                                                 P->t.skOff, (const cplx<float>*)P->t.skew, P->t.nq,

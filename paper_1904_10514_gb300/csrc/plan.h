@@ -146,7 +146,7 @@ struct hpx_plan_s {
     // form of the FP32 run-time sweeps (HPX_FLAG_AUTOTUNE): 0 = one complex column
     // per lane, 32 stages per pass; 1 = the same with 16 stages; 2 = one real
     // column per lane, 32 stages
-    int rotForm = 0;
+    int rotForm = 2;
     // the tensor-core paths' packed b: written by the grid-FFT kernel (0) or by
     // a separate full-line pass over FP32 b (1; HPX_FLAG_AUTOTUNE)
     int packSep = 0;

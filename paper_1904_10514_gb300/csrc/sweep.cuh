@@ -70,6 +70,14 @@ __device__ __forceinline__ float rot_lo(float c, float s, float carry, float x) 
     return __fmaf_rn(c, x, -__fmul_rn(s, carry));
 }
 
+// Orders that a warp of real lanes sweeps together (k_rot.cu): as many as fit 32
+// lanes with 2B real columns each, rounded up to a power of two.
+inline int sweep_orders_per_warp(int B) {
+    int w = 1;
+    while (w < 2 * B) w <<= 1;
+    return w < 32 ? 32 / w : 1;
+}
+
 template <int RB>
 struct SweepRing {
     static constexpr int kSlot = 64;   // complex per slot: 32 angles + 32 lane inputs
@@ -156,12 +164,21 @@ __device__ __forceinline__ void sweep_pass_staged_real(float* chain, int64_t ldc
         const cplx<float>* slot = ring + (t % RB) * SL;
         const float x0 = reinterpret_cast<const float*>(slot + 32)[lane];
         const cplx<float>* row = slot + coff;
+        if constexpr (K == 1) {
+            const cplx<float> cs = row[0];
+            pipe[0] = rot_hi(cs.r, cs.i, carry[0], x0);
+            carry[0] = rot_lo(cs.r, cs.i, carry[0], x0);
+        } else {
 #pragma unroll
-        for (int k = K - 1; k >= 0; --k) {
-            const float x = (k == 0) ? x0 : pipe[k - 1];
-            const cplx<float> cs = row[k];
-            pipe[k] = rot_hi(cs.r, cs.i, carry[k], x);
-            carry[k] = rot_lo(cs.r, cs.i, carry[k], x);
+            for (int k = K - 2; k >= 0; k -= 2) {   // two stages per 16-byte read
+                cplx<float> ca, cb;
+                load2(row + k, ca, cb);
+                pipe[k + 1] = rot_hi(cb.r, cb.i, carry[k + 1], pipe[k]);
+                carry[k + 1] = rot_lo(cb.r, cb.i, carry[k + 1], pipe[k]);
+                const float x = (k == 0) ? x0 : pipe[k - 1];
+                pipe[k] = rot_hi(ca.r, ca.i, carry[k], x);
+                carry[k] = rot_lo(ca.r, ca.i, carry[k], x);
+            }
         }
         const int j = t - 2 * K + 1;
         if (live && j >= 0 && j < nout) chain[(int64_t)j * ldc] = pipe[K - 1];
