@@ -409,8 +409,11 @@ __device__ __forceinline__ cplx<T> weighted(cplx<T> v, int m, int p, CoefWeights
 // coefficients of the rows sit in shared memory (read as broadcasts), each lane sums
 // its k over the warp's rows, and the four partial sums are added in warp order at
 // the end.  QUAD: the operator is in the groups of fused_quad_kernel, else row-major.
-// FP32 is bound by the operator's stream, FP64 by the FP64 pipe.  6 maps,
-// Nside 256, lmax 400 (synthesis): 96 us as matrix-matrix tiles, now 65 us.
+// P2 = Nside + 1 is one past a multiple of the tiles from Nside 128 (FP32) or 64 (FP64)
+// on: the last blocks of the grid take that k, a warp each, instead of a tile of one.
+// FP32 is bound by the latency of the tiles' loads, FP64 by the FP64 pipe.  6 maps,
+// Nside 256, lmax 400 (synthesis): 96 us as matrix-matrix tiles, 65 us with a tile for
+// the last k, now 54 us.
 template <class T, int NB, bool QUAD>
 __global__ void __launch_bounds__(128) operator_cols_kernel(const T* __restrict__ M, const int64_t* __restrict__ moff,
                                                             const cplx<T>* __restrict__ alm,
@@ -419,12 +422,44 @@ __global__ void __launch_bounds__(128) operator_cols_kernel(const T* __restrict_
     constexpr int VA = 16 / sizeof(T), NC = 2 * NB, KT = 32 * VA;
     __shared__ __align__(16) T as[128][NC];
     __shared__ T red[3][VA * NC][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b0 = blockIdx.y * NB;
+    const int ntile = 2 * (L + 1) * nkt;
+    if ((int)blockIdx.x >= ntile) {   // the k past the tiles, one (m, c) per warp, lane = row
+        const int mc = 4 * (blockIdx.x - ntile) + warp, m = mc >> 1, c = mc & 1, k = nkt * KT;
+        if (m > L) return;
+        const int n = chain_len(m, c, L), par = ((m & 1) + c) & 1;
+        const T* A = M + moff[(size_t)m * 2 + c] * ldm;
+        const cplx<T>* in = alm + (int64_t)b0 * nalm + (int64_t)m * (2 * L + 1 - m) / 2 + m + c;
+        cplx<T> acc[NB];
+#pragma unroll
+        for (int q = 0; q < NB; ++q) acc[q] = mk<T>(T(0), T(0));
+        for (int i = lane; i < n; i += 32) {
+            const int g0 = i & ~31;
+            const T v = QUAD ? A[(int64_t)g0 * ldm + (int64_t)(k >> 2) * 4 * min(32, n - g0) + 4 * lane]
+                             : A[(int64_t)i * ldm + k];
+#pragma unroll
+            for (int q = 0; q < NB; ++q)
+                if (b0 + q < B) {
+                    const cplx<T> x = weighted<T>(in[q * nalm + 2 * i], m, p, w);
+                    acc[q].r = fma(v, x.r, acc[q].r);
+                    acc[q].i = fma(v, x.i, acc[q].i);
+                }
+        }
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            for (int o = 16; o > 0; o >>= 1) {
+                acc[q].r += __shfl_xor_sync(0xffffffffu, acc[q].r, o);
+                acc[q].i += __shfl_xor_sync(0xffffffffu, acc[q].i, o);
+            }
+            if (lane == 0 && b0 + q < B) bvec[(((int64_t)(b0 + q) * (p + 1) + m) * 2 + par) * P2 + k] = acc[q];
+        }
+        return;
+    }
     const int kt = blockIdx.x % nkt, mc = blockIdx.x / nkt;
     const int m = mc >> 1, c = mc & 1;
     const int par = ((m & 1) + c) & 1;
     const int n = chain_len(m, c, L);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int k = kt * KT + lane * VA, b0 = blockIdx.y * NB;
+    const int k = kt * KT + lane * VA;
     const bool on = k < P2;   // ldm >= k + VA: rows are padded to 4
     const T* A = M + moff[(size_t)m * 2 + c] * ldm;
     const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2 + m + c;
@@ -506,12 +541,14 @@ template <class T>
 void launch_operator_cols(const hpx_plan_s* P, const void* M, bool quad, const T* alm, cudaStream_t s, T wpos,
                           bool dropim) {
     const auto& g = P->g;
-    const int kt = 32 * 16 / sizeof(T), nkt = (g.P2 + kt - 1) / kt;
+    const int kt = 32 * 16 / sizeof(T);
+    const bool tail = g.P2 > kt && g.P2 % kt == 1;
+    const int nkt = tail ? g.P2 / kt : (g.P2 + kt - 1) / kt;
     // maps per block as launch_fused: FP32 as many as possible (8), FP64 no absent ones
     const int nb = sizeof(T) == 4 ? (g.B > 4 ? 8 : g.B > 2 ? 4 : g.B)
                                   : (g.B + (g.B + 3) / 4 - 1) / ((g.B + 3) / 4);
     auto run = [&](auto kern, int NB) {
-        dim3 grid((g.L + 1) * 2 * nkt, (g.B + NB - 1) / NB);
+        dim3 grid((g.L + 1) * 2 * nkt + (tail ? (g.L + 2) / 2 : 0), (g.B + NB - 1) / NB);
         kern<<<grid, 128, 0, s>>>((const T*)M, P->fusedOff, (const cplx<T>*)alm, (cplx<T>*)P->bvec, g.P2,
                                   P->fused_ldm, g.p, g.L, g.B, g.nalm, nkt, CoefWeights{(double)wpos, dropim});
     };

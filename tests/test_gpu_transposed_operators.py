@@ -41,6 +41,13 @@ def test_operators_match_sweeps(nside, lmax, B, prec):
         assert float(d.max()) <= TOL[prec], (name, d)
 
 
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("nside,lmax,B", [(128, 0, 1), (128, 61, 3), (256, 31, 8), (256, 33, 5)])
+def test_last_k(nside, lmax, B, prec):
+    """Nside + 1 modes: one past the tiles of 128 (FP32) or 64 (FP64)."""
+    test_operators_match_sweeps(nside, lmax, B, prec)
+
+
 @pytest.mark.parametrize("B", [8, 9, 33])
 @pytest.mark.parametrize("nside,lmax", [(16, 21), (64, 128)])
 def test_equal_weight_analysis(nside, lmax, B):
