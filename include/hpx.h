@@ -86,12 +86,11 @@ extern "C" {
  *   undefined).  Costs one extra read of the input. */
 #define HPX_FLAG_CHECKED 8u
 /* HPX_FLAG_AUTOTUNE: at plan creation, on scratch buffers allocated and freed
- *   inside hpx_plan_ex: (1) time the ring-FFT and grid-FFT stages of the plan's
- *   batch with 16 and with 32 elements per thread (launch shapes of the
- *   compile-time FFT kernels), for FP32 plans that run the sweeps per call the
- *   three forms of the sweep kernel, for the tensor-core paths the two
+ *   inside hpx_plan_ex: (1) time, for FP32 plans that run the sweeps per call,
+ *   the three forms of the sweep kernel, for the tensor-core paths the two
  *   placements of the packing of b, and the two forms of the Bluestein ring
- *   classes of 4096 points and more, and keep the fastest of each
+ *   classes of 4096 points and more (a near tie goes to the quarter-length
+ *   form), and keep the fastest of each
  *   (hpx_plan_tuning; remembered per nside, lmax, batch, precision and path for
  *   the process's later plans); (2) when the
  *   per-order operators were built, time one analysis
@@ -242,8 +241,9 @@ int64_t hpx_plan_bytes(const hpx_plan_s* plan);
 int hpx_plan_flags(const hpx_plan_s* plan);
 /* Kernel launches of one hpx_analyze call (ring FFTs: one per transform length). */
 int hpx_plan_launches(const hpx_plan_s* plan);
-/* Launch shapes in effect (HPX_FLAG_AUTOTUNE, else 16, 16, 0, 0 and 0):
- * elements per thread of the ring-FFT and of the grid-FFT kernels, the form of
+/* Launch shapes in effect (HPX_FLAG_AUTOTUNE, else 16, 16, 2, 0 and 0):
+ * elements per thread of the ring-FFT and of the grid-FFT kernels (16 or 32;
+ * both values name the one shape these kernels have), the form of
  * the FP32 run-time Givens sweeps of 4 maps or more (0: one complex column per
  * lane, 32 stages per pass; 1: the same with 16 stages; 2: one real column per
  * lane, 32 stages), whether the tensor-core paths' FP16-pair right-hand sides

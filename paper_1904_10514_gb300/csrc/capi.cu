@@ -496,17 +496,14 @@ void tune_shapes(hpx_plan_s* P, const void* maps, void* alm, cudaEvent_t e0, cud
             return;
         }
     }
-    float t[2] = {0.f, 0.f};
-    for (int e = 0; e < 2; ++e) {
-        P->ringE = e ? 32 : 16;
-        t[e] = time_stage(P, maps, alm, 0, e0, e1);
-    }
-    P->ringE = t[1] < t[0] ? 32 : 16;
-    P->latE = 16;   // the grid FFT has one shape
-    {   // the Bluestein ring classes: whole-ring or quarter-length convolutions
+    P->ringE = P->latE = 16;   // the FFT kernels have one shape
+    {   // the Bluestein ring classes: whole-ring or quarter-length convolutions; a tie goes to
+        // the latter, so that the choice, which changes the last bits, does not hang on noise
+        P->ringForm = 0;
+        const float whole = time_stage(P, maps, alm, 0, e0, e1);
         P->ringForm = 1;
-        const float t4 = time_stage(P, maps, alm, 0, e0, e1);
-        P->ringForm = t4 < t[P->ringE == 32 ? 1 : 0] ? 1 : 0;
+        const float quarters = time_stage(P, maps, alm, 0, e0, e1);
+        P->ringForm = quarters < 1.02f * whole ? 1 : 0;
     }
     P->rotForm = 2;
     if (sweeps) {   // the three forms of the sweep kernel

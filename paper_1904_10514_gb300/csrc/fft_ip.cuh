@@ -103,18 +103,20 @@ __host__ __device__ constexpr int last_radix(int logn) { return radix(logn, npas
 __host__ __device__ constexpr int out_radix(int logn, int nt) { return logn == 13 && nt == 256 ? 32 : last_radix(logn); }
 
 // Last pass, after a barrier: outputs j + q S (S = N / R, group j = tid + gg NT) to
-// st(index, q, gg, value) for q < LO or q >= HI.
-template <class T, int LOGN, int NT, bool INV, int LO, int HI, class ST>
+// st(index, q, gg, value) for q < LO or q >= HI.  PRE: the first group's twiddles are
+// read ahead of the barrier.
+template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE, class ST>
 __device__ __forceinline__ void last_pass(const cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, int tid,
                                           ST st) {
     constexpr int N = 1 << LOGN, R = last_radix(LOGN), S = N / R, G = (S + NT - 1) / NT;
-    Twiddles<T> t = load_twiddles<T, R, INV>(min(tid, S - 1), twstep, tw);
+    Twiddles<T> t;
+    if constexpr (PRE) t = load_twiddles<T, R, INV>(min(tid, S - 1), twstep, tw);
     __syncthreads();
 #pragma unroll
     for (int gg = 0; gg < G; ++gg) {
         const int j = tid + gg * NT;
         if (S % NT != 0 && j >= S) break;
-        if (gg > 0) t = load_twiddles<T, R, INV>(j, twstep, tw);
+        if (!PRE || gg > 0) t = load_twiddles<T, R, INV>(j, twstep, tw);
         const cplx<T>* e = a + slot(j);
         cplx<T> x[R];
 #pragma unroll
@@ -162,7 +164,7 @@ __device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>
 // The whole transform: ld(i, r) as first_pass, st(index, q, gg, value) as last_pass.
 // st may store to the positions of a (natural order): a thread only produces
 // positions that it alone has read.  Ends without a barrier.
-template <class T, int LOGN, int NT, bool INV, int LO, int HI, class LD, class ST>
+template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE = true, class LD, class ST>
 __device__ __forceinline__ void transform(cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, int tid, LD ld,
                                           ST st) {
     first_pass<T, LOGN, NT, INV, false>(a, tid, ld);
@@ -171,7 +173,7 @@ __device__ __forceinline__ void transform(cplx<T>* a, const cplx<T>* __restrict_
         last_passes_8192<T, NT, INV, LO, HI>(a, tw, twstep, tid, st);
     } else {
         inner_passes<T, LOGN, NT, INV>(a, tw, twstep, tid);
-        last_pass<T, LOGN, NT, INV, LO, HI>(a, tw, twstep, tid, st);
+        last_pass<T, LOGN, NT, INV, LO, HI, PRE>(a, tw, twstep, tid, st);
     }
 }
 
@@ -187,7 +189,6 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
     first_pass<T, LOGN, NT, false, true>(a, tid, [&](int i, int) { return ld(i); });
     inner_passes<T, LOGN, NT, false>(a, tw, twstep, tid);
     const bool on = NG == NT || tid < NG;
-    Twiddles<T> t = load_twiddles<T, R, false>(min(tid, NG - 1), twstep, tw);
     __syncthreads();
     cplx<T> y[16];
     if (on) {
@@ -197,8 +198,7 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
             cplx<T> x[R];
 #pragma unroll
             for (int q = 0; q < R; ++q) x[q] = e[slot((i + q * D) * NG)];
-            if (i > 0) t = load_twiddles<T, R, false>(tid + i * NG, twstep, tw);
-            twiddle_by<T, R>(x, t);
+            twiddle_by<T, R>(x, load_twiddles<T, R, false>(tid + i * NG, twstep, tw));
             reg_dft<T, R, false>(x);
 #pragma unroll
             for (int q = 0; q < R; ++q) {
@@ -215,7 +215,7 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
         for (int r = 0; r < 16; ++r) to[r] = y[r];
     }
     inner_passes<T, LOGN, NT, true>(a, tw, twstep, tid);
-    last_pass<T, LOGN, NT, true, R / 2, R>(a, tw, twstep, tid, [&](int i, int, int, cplx<T> v) { st(i, v); });
+    last_pass<T, LOGN, NT, true, R / 2, R, false>(a, tw, twstep, tid, [&](int i, int, int, cplx<T> v) { st(i, v); });
 }
 
 }  // namespace ip

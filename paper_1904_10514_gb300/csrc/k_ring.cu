@@ -20,6 +20,7 @@
 
 #include "fft_ct.cuh"
 #include "plan.h"
+#include "ring_blue.cuh"
 
 namespace hpx {
 
@@ -36,14 +37,15 @@ constexpr int kRingThreads = 512;
 //     Y_m (odd m) at +-m, so the plain transpose carries 1 (even m > 0), 2 (odd m)
 //     and 1/2 (m = 0); the transpose for the coefficient inner product with
 //     weight 2 for m > 0 halves the m > 0 ones: 1/2 for even m, 1 for odd m.
-//     0 for L < m <= p.
+// Rows are written up to order min(p, L); nothing reads the orders above.
 template <class T, class BUF>
 __device__ __forceinline__ void ring_rows_out(BUF zat, int n, int p, int L, const cplx<T>* __restrict__ ph, bool sh,
                                               T ew, cplx<T>* rowN, cplx<T>* rowS, bool equator, int tid, int nt) {
     const int h = n >> 1;
-    for (int m = tid; m <= p; m += nt) {
+    const int last = min(p, L);
+    for (int m = tid; m <= last; m += nt) {
         cplx<T> cN = mk<T>(T(0), T(0)), cS = cN;
-        if (ew == T(0) ? m <= h : m <= L) {
+        if (ew != T(0) || m <= h) {
             const int k = m % n;
             const cplx<T> zm = zat(k);
             const cplx<T> zc = conjg(zat(k == 0 ? 0 : n - k));
@@ -72,14 +74,58 @@ __device__ __forceinline__ void ring_rows_out(BUF zat, int n, int p, int L, cons
     }
 }
 
-// The same step for the launches of one transform length N = 2^LOGN >= 4096
-// whose ring pairs are all of one kind (BLUE: Bluestein rings of convolution
-// length N; else rings of N points): the FFT length, the thread count
-// (N / 16 or N / 32) and the pass structure are compile-time constants
-// (fft_ct.cuh), and the kind of ring is known, so neither transform carries
-// the other's code.
-template <class T, int LOGN, int NT, bool BLUE>
-__global__ void __launch_bounds__(NT, ((1 << LOGN) / NT == 16 ? (LOGN <= 13 ? 1024 / NT : 1) : 512 / NT)) ring_ct_kernel(
+// One ring pair by the block of NT threads (quarters: 4 NT), transform length and kind
+// fixed: rings of n = N = 2^LOGN points (plain), Bluestein rings with a convolution
+// of N = 2^LOGN >= 2n - 1 points (whole; the inverse transform's last pass applies
+// the output chirp), or with four of 2^LOGN >= n/2 points (quarters).
+template <class T, int LOGN, int NT>
+__device__ __forceinline__ void ring_plain(cplx<T>* buf, const T* __restrict__ f, int sN, int sS,
+                                           const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw, int twlen,
+                                           int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
+    constexpr int N = 1 << LOGN, R = ip::out_radix(LOGN, NT);
+    const bool equator = sN == sS;
+    ip::transform<T, LOGN, NT, false, R, R, false>(
+        buf, tw, twlen / N, threadIdx.x,
+        [&](int k, int) { return mk<T>(f[sN + k], equator ? T(0) : f[sS + k]); },
+        [&](int k, int, int, cplx<T> v) { buf[ip::slot(k)] = v; });
+    __syncthreads();
+    ring_rows_out<T>([&](int k) { return buf[ip::slot(k)]; }, N, p, L, ph, sh, ew, rowN, rowS, equator, threadIdx.x,
+                     NT);
+}
+template <class T, int LOGN, int NT>
+__device__ __forceinline__ void ring_whole(cplx<T>* buf, const T* __restrict__ f, int sN, int sS, int n,
+                                           const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
+                                           const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw, int twlen,
+                                           int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
+    constexpr int N = 1 << LOGN;
+    ip::convolve<T, LOGN, NT>(
+        buf, tw, twlen / N, threadIdx.x,
+        [&](int k) { return k < n ? mul(mk<T>(f[sN + k], f[sS + k]), ch[k]) : mk<T>(T(0), T(0)); },
+        [&](int k) { return bh[k]; },
+        [&](int k, cplx<T> v) {
+            if (k < n) buf[ip::slot(k)] = mul(v, ch[k]);
+        });
+    __syncthreads();
+    ring_rows_out<T>([&](int k) { return buf[ip::slot(k)]; }, n, p, L, ph, sh, ew, rowN, rowS, false, threadIdx.x, NT);
+}
+template <class T, int LOGQ, int NTQ>
+__device__ __forceinline__ void ring_quarters(cplx<T>* buf, const T* __restrict__ f, int sN, int sS, int n,
+                                              const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
+                                              const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw,
+                                              int twlen, int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
+    constexpr int NT = 4 * NTQ;
+    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ>(
+        buf, n, ch, bh, tw, twlen, [&](int k) { return mk<T>(f[sN + k], f[sS + k]); });
+    R.natural(n, threadIdx.x, NT);
+    ring_rows_out<T>([&](int k) { return R.at(k, n); }, n, p, L, ph, sh, ew, rowN, rowS, false, threadIdx.x, NT);
+}
+
+// The ring stage for the launches of one transform length and kind (KIND 0 plain, 1
+// whole, 2 quarters).  Bound by the shared-memory passes.  32 maps, Nside 1024: the
+// stage 1900 us on Stockham passes, now 1835; 200 maps of mixed Nside 6.53 to 5.71 ms
+// per call with the spreading and grid FFT (short rings most of it).
+template <class T, int LOGN, int NT, int MINB, int KIND>
+__global__ void __launch_bounds__(KIND == 2 ? 4 * NT : NT, MINB) ring_ip_kernel(
     const T* __restrict__ maps, cplx<T>* __restrict__ Y, const int* __restrict__ nphi_t,
     const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int64_t* __restrict__ shOff_t,
     const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t, const cplx<T>* __restrict__ shift,
@@ -90,44 +136,28 @@ __global__ void __launch_bounds__(NT, ((1 << LOGN) / NT == 16 ? (LOGN <= 13 ? 10
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
     const int i = ringlist[blockIdx.y];
     const int b = blockIdx.x;
-    const int n = nphi_t[i];
     const int sN = startN_t[i], sS = startS_t[i];
-    const bool equator = (sN == sS);
     const T* f = maps + (mapIdx ? mapIdx[b] : (int64_t)b * npix);
-    const int tid = threadIdx.x;
-    const int twstep = twlen >> LOGN;
-    auto sample = [&](int k) { return mk<T>(f[sN + k], equator ? T(0) : f[sS + k]); };
-    auto to_smem = [&](int, int pi, cplx<T> v) { buf[pi] = v; };
-    if constexpr (!BLUE) {
-        ct::fft<T, LOGN, NT, false, false>(buf, tw, twstep, [&](int k, int) { return sample(k); }, to_smem);
-    } else {
-        // Bluestein: chirped samples in, times the transformed kernel out; the
-        // inverse transform applies the output chirp in its last pass
-        const cplx<T>* ch = chirp + chOff_t[i];
-        const cplx<T>* bh = bhat + bhOff_t[i];
-        ct::fft<T, LOGN, NT, false, false>(
-            buf, tw, twstep, [&](int k, int) { return k < n ? mul(sample(k), ch[k]) : mk<T>(T(0), T(0)); },
-            [&](int j, int pi, cplx<T> v) { buf[pi] = mul(v, bh[j]); });
-        ct::fft<T, LOGN, NT, true, true>(
-            buf, tw, twstep, [&](int, int pi) { return buf[pi]; },
-            [&](int j, int pi, cplx<T> v) { buf[pi] = j < n ? mul(v, ch[j]) : v; });
-    }
     cplx<T>* rowN = Y + ((int64_t)b * Q + (i + 1)) * (p + 1);
     cplx<T>* rowS = Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1);
-    ring_rows_out<T>([&](int k) { return buf[ct::padc(k)]; }, n, p, L, shift + shOff_t[i], shifted_t[i] != 0, ew,
-                     rowN, rowS, equator, tid, NT);
+    const cplx<T>* ph = shift + shOff_t[i];
+    const bool sh = shifted_t[i] != 0;
+    if constexpr (KIND == 0) {
+        ring_plain<T, LOGN, NT>(buf, f, sN, sS, ph, tw, twlen, p, L, ew, sh, rowN, rowS);
+    } else {
+        const cplx<T>*ch = chirp + chOff_t[i], *bh = bhat + bhOff_t[i];
+        if constexpr (KIND == 1)
+            ring_whole<T, LOGN, NT>(buf, f, sN, sS, nphi_t[i], ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS);
+        else
+            ring_quarters<T, LOGN, NT>(buf, f, sN, sS, nphi_t[i], ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS);
+    }
 }
 
-// A Bluestein ring of nphi = 4j points as four transforms of j points: with
-// t = 4u + s the DFT is Z[q + r j] = sum_s (-i)^{s r} W^{s q} Y_s[q]
-// (W = e^{-2 pi i / nphi}, q < j, r < 4), Y_s the DFT of the subsequence
-// z[4u + s].  Each Y_s is a Bluestein convolution of L/4 = 2^(LOGN-2) points
-// (L the ring's convolution length, L/4 >= 2j), run on NT/4 threads of the
-// block beside the other three (compile-time FFT, one padded quarter of the
-// buffer each): a quarter of the transformed-kernel table per ring and one
-// radix-16 pass fewer than the full-length convolution.  The radix-4 step writes
-// Z into the free tail of the quarters (quarter r, from slot padc(j)), and the
-// output rows follow as in ring_ct_kernel.
+// Ring form 1 at convolutions of 4096 points (four of 1024), on the Stockham passes of
+// fft_ct.cuh: at a last radix of 4 the compiler fuses other products of the passes of
+// ring_quarters into sums, which changes the last bits, and the times are the same.
+// The radix-4 step writes Z into the free tail of the quarters (quarter r, from slot
+// padc(j)).
 template <class T, int LOGN, int NT>
 __global__ void __launch_bounds__(NT, (LOGN <= 13 ? 1024 / NT : 1)) ring4_ct_kernel(
     const T* __restrict__ maps, cplx<T>* __restrict__ Y, const int* __restrict__ nphi_t,
@@ -187,9 +217,15 @@ __global__ void __launch_bounds__(NT, (LOGN <= 13 ? 1024 / NT : 1)) ring4_ct_ker
         n, p, L, shift + shOff_t[i], shifted_t[i] != 0, ew, rowN, rowS, false, tid, NT);
 }
 
-// The step for ring pair i of map b by the whole block (runtime transform
-// length; the generic form behind ring_fft_kernel and ring_list_kernel).
-template <class T, int E>
+// The step for ring pair i of map b by the whole block (the generic form behind
+// ring_fft_kernel and ring_list_kernel): with NT = kRingShortThreads threads the
+// Bluestein transforms of 512 .. 2048 points (one code path per length, the same for
+// the whole block) run on fft_ip.cuh, the others, and all of them with NT = 0 (a
+// block of any size), on the run-time length FFT of common.cuh.  (Rings of 512 to
+// 2048 points stay there: on fft_ip.cuh the compiler fuses other products into sums
+// beside the other lengths, which changes their last bits.)
+constexpr int kRingShortThreads = 128;
+template <class T, int E, int NT>
 __device__ __forceinline__ void ring_pair(
     cplx<T>* buf, int i, int b, const T* __restrict__ maps, cplx<T>* __restrict__ Y, const int* __restrict__ nphi_t,
     const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int* __restrict__ pow2_t,
@@ -203,6 +239,22 @@ __device__ __forceinline__ void ring_pair(
     const bool equator = (sN == sS);
     const T* f = maps + (mapIdx ? mapIdx[b] : (int64_t)b * npix);
     const int tid = threadIdx.x, nt = blockDim.x;
+    cplx<T>* rowN = Y + ((int64_t)b * Q + (i + 1)) * (p + 1);
+    cplx<T>* rowS = Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1);
+    if constexpr (NT > 0) {
+        static_assert(NT == 128, "short rings: 16 elements per thread at 2048 points");
+        const cplx<T>* ph = shift + shOff_t[i];
+        const bool sh = shifted_t[i] != 0;
+        if (!pow2_t[i]) {
+            const cplx<T>*ch = chirp + chOff_t[i], *bh = bhat + bhOff_t[i];
+            switch (logL_t[i]) {
+                case 11: ring_whole<T, 11, NT>(buf, f, sN, sS, n, ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS); return;
+                case 10: ring_whole<T, 10, NT>(buf, f, sN, sS, n, ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS); return;
+                case 9: ring_whole<T, 9, NT>(buf, f, sN, sS, n, ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS); return;
+                default: break;
+            }
+        }
+    }
 
     auto sample = [&](int k) { return mk<T>(f[sN + k], equator ? T(0) : f[sS + k]); };
     auto same = [](int, cplx<T> v) { return v; };
@@ -245,15 +297,14 @@ __device__ __forceinline__ void ring_pair(
         __syncthreads();
     }
 
-    cplx<T>* rowN = Y + ((int64_t)b * Q + (i + 1)) * (p + 1);
-    cplx<T>* rowS = Y + ((int64_t)b * Q + (Q - 2 - i)) * (p + 1);
     ring_rows_out<T>([&](int k) { return buf[pad(k)]; }, n, p, L, shift + shOff_t[i], shifted_t[i] != 0, ew, rowN,
                      rowS, equator, tid, nt);
 }
 
-
-template <class T, int E>
-__global__ void __launch_bounds__(kRingThreads, (E <= 16 ? 2 : 1)) ring_fft_kernel(
+// Every ring pair of transforms up to 2048 points (NT = 128 threads), one launch:
+// alone, each of the short classes' launches is bound by its latency.
+template <class T, int E, int NT>
+__global__ void __launch_bounds__(NT > 0 ? NT : kRingThreads, NT > 0 ? (sizeof(T) == 4 ? 6 : 3) : (E <= 16 ? 2 : 1)) ring_fft_kernel(
     const T* __restrict__ maps, cplx<T>* __restrict__ Y, const int* __restrict__ nphi_t,
     const int* __restrict__ startN_t, const int* __restrict__ startS_t,
     const int* __restrict__ pow2_t, const int* __restrict__ logn_t, const int* __restrict__ fftL_t,
@@ -267,8 +318,9 @@ __global__ void __launch_bounds__(kRingThreads, (E <= 16 ? 2 : 1)) ring_fft_kern
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
     // largest rings first: blockIdx.y = 0 is the equator
     const int i = ringlist ? ringlist[blockIdx.y] : npairs - 1 - (int)blockIdx.y;
-    ring_pair<T, E>(buf, i, blockIdx.x, maps, Y, nphi_t, startN_t, startS_t, pow2_t, logn_t, fftL_t, logL_t, shOff_t,
-                    chOff_t, bhOff_t, shift, chirp, bhat, tw, twlen, p, Q, npix, ew, shifted_t, L, mapIdx);
+    ring_pair<T, E, NT>(buf, i, blockIdx.x, maps, Y, nphi_t, startN_t, startS_t, pow2_t, logn_t, fftL_t, logL_t,
+                        shOff_t, chOff_t, bhOff_t, shift, chirp, bhat, tw, twlen, p, Q, npix, ew, shifted_t, L,
+                        mapIdx);
 }
 
 // The short-ring part of the ring stage of every sub-plan of an uneven batch
@@ -283,7 +335,7 @@ __global__ void __launch_bounds__(kRingThreads, (E <= 16 ? 2 : 1)) ring_fft_kern
 // 2048 points, 32 for the shorter ones, each group its own launch.  The
 // longer transforms run in the sub-plans' compile-time kernels.
 template <class T, int NT>
-__global__ void __launch_bounds__(NT, (NT == 32 ? 16 : 8)) ring_list_kernel(const RingJob<T>* __restrict__ jobs,
+__global__ void __launch_bounds__(NT, (NT == 32 ? 16 : sizeof(T) == 4 ? 6 : 3)) ring_list_kernel(const RingJob<T>* __restrict__ jobs,
                                                                           const int4* __restrict__ items,
                                                                           int nitems, const T* __restrict__ maps_base) {
     extern __shared__ unsigned char smem_raw[];
@@ -291,12 +343,17 @@ __global__ void __launch_bounds__(NT, (NT == 32 ? 16 : 8)) ring_list_kernel(cons
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 w = items[it];
         const RingJob<T>& J = jobs[w.x];
-        ring_pair<T, 16>(buf, w.y, w.z, maps_base + J.mapoff, J.Y, J.nphi, J.startN, J.startS, J.pow2, J.logn,
-                         J.fftL, J.logL, J.shOff, J.chOff, J.bhOff, J.shift, J.chirp, J.bhat, J.tw, J.twlen, J.p, J.Q,
-                         J.npix, T(0), J.shifted, J.L, J.mapIdx);
+        ring_pair<T, 16, (NT == kRingShortThreads ? NT : 0)>(
+            buf, w.y, w.z, maps_base + J.mapoff, J.Y, J.nphi, J.startN, J.startS, J.pow2, J.logn, J.fftL, J.logL,
+            J.shOff, J.chOff, J.bhOff, J.shift, J.chirp, J.bhat, J.tw, J.twlen, J.p, J.Q, J.npix, T(0), J.shifted,
+            J.L, J.mapIdx);
         __syncthreads();   // the next item overwrites the shared buffer
     }
 }
+
+// Slots of the shared buffer of a short-ring block for transforms up to N points:
+// the padded array of common.cuh or a transform of fft_ip.cuh.
+inline int ring_short_slots(int N) { return std::max(N + N / 16, ip::slots(N)); }
 
 template <class T>
 void launch_ring_list(const RingJob<T>* jobs, const int4* items, int nitems, int nlong, const T* maps_base,
@@ -306,12 +363,12 @@ void launch_ring_list(const RingJob<T>* jobs, const int4* items, int nitems, int
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     auto run = [&](auto kern, int threads, int maxN, const int4* first, int n, int perSM) {
         if (n <= 0) return;
-        const size_t smem = (size_t)(maxN + maxN / 16) * sizeof(cplx<T>);
+        const size_t smem = (size_t)ring_short_slots(maxN) * sizeof(cplx<T>);
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         kern<<<std::min(n, sms * perSM), threads, smem, s>>>(jobs, first, n, maps_base);
     };
     // items [0, nlong): 1024 or 2048 points; [nlong, nitems): 512 or fewer
-    run(ring_list_kernel<T, 128>, 128, 2048, items, nlong, 8);
+    run(ring_list_kernel<T, 128>, 128, 2048, items, nlong, sizeof(T) == 4 ? 6 : 3);
     run(ring_list_kernel<T, 32>, 32, 512, items + nlong, nitems - nlong, 16);
 }
 
@@ -363,10 +420,11 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
     const auto& t = P->t;
     auto launch = [&](int N, int nrings, const int* list) {
         // E elements per thread: blocks of N / E threads (at least one warp)
-        const bool big = N > 16 * kRingThreads;
-        const int threads = std::max(32, N / (big ? 32 : 16));
-        const size_t smem = (size_t)(N + N / 16) * sizeof(cplx<T>);
-        auto kern = big ? ring_fft_kernel<T, 32> : ring_fft_kernel<T, 16>;
+        const bool big = N > 16 * kRingThreads, brief = N <= 16 * kRingShortThreads;
+        const int threads = brief ? kRingShortThreads : std::max(32, N / (big ? 32 : 16));
+        const size_t smem = (size_t)(brief ? ring_short_slots(N) : N + N / 16) * sizeof(cplx<T>);
+        auto kern = brief ? ring_fft_kernel<T, 16, kRingShortThreads>
+                          : big ? ring_fft_kernel<T, 32, 0> : ring_fft_kernel<T, 16, 0>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         dim3 grid(g.B, nrings);
         kern<<<grid, threads, smem, s>>>(
@@ -386,43 +444,40 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
             launch(c.N, c.count, P->ringList + c.first);
             continue;
         }
-        const size_t smem = (size_t)(c.N + c.N / 16) * sizeof(cplx<T>);
         dim3 grid(g.B, c.count);
-        auto run = [&](auto kern, int threads) {
+        const bool quarters = c.blue && P->ringForm == 1;
+        if (quarters && c.N == 4096) {
+            const size_t smem = (size_t)(c.N + c.N / 16) * sizeof(cplx<T>);
+            auto kern = ring4_ct_kernel<T, 12, 256>;
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            kern<<<grid, threads, smem, s>>>(maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.shOff, t.chOff,
-                                             t.bhOff, (const cplx<T>*)t.shift, (const cplx<T>*)t.chirp,
-                                             (const cplx<T>*)t.bhat, (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q,
-                                             g.npix, P->ringList + c.first, ew, t.shifted, g.L, P->mapIdx);
-        };
-        if (c.blue && P->ringForm == 1) {   // four quarter-length Bluestein transforms, N / 16 threads
-            auto run4 = [&](auto kern, int threads) {
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                kern<<<grid, threads, smem, s>>>(maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.shOff,
-                                                 t.ch4Off, t.bh4Off, (const cplx<T>*)t.shift,
-                                                 (const cplx<T>*)t.chirp4, (const cplx<T>*)t.bhat4,
-                                                 (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix,
-                                                 P->ringList + c.first, ew, t.shifted, g.L, P->mapIdx);
-            };
-            if (c.N == 4096) run4(ring4_ct_kernel<T, 12, 256>, 256);
-            else if (c.N == 8192) run4(ring4_ct_kernel<T, 13, 512>, 512);
-            else run4(ring4_ct_kernel<T, 14, 512>, 512);
+            kern<<<grid, 256, smem, s>>>(maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.shOff, t.ch4Off, t.bh4Off,
+                                         (const cplx<T>*)t.shift, (const cplx<T>*)t.chirp4, (const cplx<T>*)t.bhat4,
+                                         (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix, P->ringList + c.first, ew,
+                                         t.shifted, g.L, P->mapIdx);
             continue;
         }
-        // elements per thread: 16 (N / 16 threads) or, when the plan's tuning chose
-        // it, 32 (N / 32 threads, two groups per thread and pass)
-        const bool e32 = P->ringE == 32;
+        const size_t smem = (size_t)(quarters ? 4 * ip::slots(c.N / 4) : ip::slots(c.N)) * sizeof(cplx<T>);
+        auto run = [&](auto kern, int threads) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            kern<<<grid, threads, smem, s>>>(
+                maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.shOff, quarters ? t.ch4Off : t.chOff,
+                quarters ? t.bh4Off : t.bhOff, (const cplx<T>*)t.shift,
+                (const cplx<T>*)(quarters ? t.chirp4 : t.chirp), (const cplx<T>*)(quarters ? t.bhat4 : t.bhat),
+                (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix, P->ringList + c.first, ew, t.shifted, g.L,
+                P->mapIdx);
+        };
+        // 16 elements per thread (32 for plain rings of 8192 points)
+        constexpr bool F = sizeof(T) == 4;
         if (c.N == 4096) {
-            if (e32) { if (c.blue) run(ring_ct_kernel<T, 12, 128, true>, 128); else run(ring_ct_kernel<T, 12, 128, false>, 128); }
-            else if (c.blue) run(ring_ct_kernel<T, 12, 256, true>, 256);
-            else run(ring_ct_kernel<T, 12, 256, false>, 256);
+            if (c.blue) run(ring_ip_kernel<T, 12, 256, F ? 4 : 2, 1>, 256);
+            else run(ring_ip_kernel<T, 12, 256, F ? 4 : 2, 0>, 256);
         } else if (c.N == 8192) {
-            if (e32) { if (c.blue) run(ring_ct_kernel<T, 13, 256, true>, 256); else run(ring_ct_kernel<T, 13, 256, false>, 256); }
-            else if (c.blue) run(ring_ct_kernel<T, 13, 512, true>, 512);
-            else run(ring_ct_kernel<T, 13, 512, false>, 512);
-        } else {
-            if (c.blue) run(ring_ct_kernel<T, 14, 512, true>, 512);
-            else run(ring_ct_kernel<T, 14, 512, false>, 512);
+            if (quarters) run(ring_ip_kernel<T, 11, 128, F ? 2 : 1, 2>, 512);
+            else if (c.blue) run(ring_ip_kernel<T, 13, 512, F ? 2 : 1, 1>, 512);
+            else run(ring_ip_kernel<T, 13, 256, F ? 2 : 1, 0>, 256);
+        } else if constexpr (F) {   // nside 2048 (FP32 only): every ring of 16384 is a Bluestein ring
+            if (quarters) run(ring_ip_kernel<T, 12, 256, 1, 2>, 1024);
+            else run(ring_ip_kernel<T, 14, 1024, 1, 1>, 1024);
         }
     }
 }

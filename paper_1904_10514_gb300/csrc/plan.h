@@ -137,8 +137,8 @@ struct hpx_plan_s {
     int64_t* dTcOff = nullptr;
     int dNtiles = 0;
     float tuned_ms[2] = {0.f, 0.f};   // HPX_FLAG_AUTOTUNE: ms per analysis, operators / sweeps
-    // launch shapes of the compile-time FFT kernels: elements per thread (16 or 32)
-    // of the ring stage and of the grid FFT (HPX_FLAG_AUTOTUNE times both)
+    // elements per thread of the ring stage and of the grid FFT as hpx_plan_tuning reports
+    // them (both kernels have one shape)
     int ringE = 16, latE = 16;
     // Bluestein ring classes of 4096 points and more: one convolution of the whole
     // ring (0) or four of its quarter-length subsequences (1; HPX_FLAG_AUTOTUNE)
