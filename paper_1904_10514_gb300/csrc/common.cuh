@@ -206,6 +206,29 @@ __device__ __forceinline__ Twiddles<T> load_twiddles(int j, int step, const cplx
     t.b8 = R > 8 ? ld(8) : t.b1;
     return t;
 }
+// The same powers from the compact tables of the passes of span S (twc_offset): rows
+// w^(r j), r = 1, 2, 4, 8 below R, S entries each, so that consecutive threads read
+// consecutive entries (in the table of all twlen powers every read of the span-16
+// pass touches 16 lines).
+__host__ __device__ constexpr int twc_offset(int S, int R) {
+    return (S == 16 ? 0 : S == 256 ? 160 : 2720) + S * (R == 2 ? 0 : R == 4 ? 1 : R == 8 ? 3 : 6);
+}
+constexpr int kTwcSize = 2720 + 3 * 4096;   // spans 16 and 256: radix 2..16, span 4096: radix 2, 4
+template <class T, int R, int S, bool INV>
+__device__ __forceinline__ Twiddles<T> load_twiddles_c(int j, const cplx<T>* __restrict__ twc) {
+    const cplx<T>* row = twc + twc_offset(S, R) + j;
+    auto ld = [&](int q) {
+        cplx<T> w = row[q * S];
+        if (INV) w.i = -w.i;
+        return w;
+    };
+    Twiddles<T> t;
+    t.b1 = ld(0);
+    t.b2 = R > 2 ? ld(1) : t.b1;
+    t.b4 = R > 4 ? ld(2) : t.b1;
+    t.b8 = R > 8 ? ld(3) : t.b1;
+    return t;
+}
 template <class T, int R>
 __device__ __forceinline__ void twiddle_by(cplx<T>* x, const Twiddles<T>& t) {
     const cplx<T> w3 = R > 2 ? mul(t.b1, t.b2) : t.b1;

@@ -22,11 +22,11 @@ __device__ __forceinline__ int padc(int i) { return i + (i >> 4); }
 // LD(nat, padded) -> value and ST(nat, padded, value): element access; for the
 // in-place shared-memory passes they read / write a[padded].  BAR: a barrier
 // between the loads and the stores (the pass reads and writes the same array).
-// tw: e^{-2 pi i t / twlen}, twstep = twlen / N.
+// tw: the compact twiddle tables (twc_offset, common.cuh).
 // tid: this thread's index among the NT threads of the transform (a block may
 // run several transforms side by side, each on its own NT threads and array).
 template <class T, int N, int R, int LOGS, int NT, bool INV, bool BAR, class LD, class ST>
-__device__ __forceinline__ void pass(const cplx<T>* __restrict__ tw, int twstep, LD ld, ST st, int tid) {
+__device__ __forceinline__ void pass(const cplx<T>* __restrict__ tw, LD ld, ST st, int tid) {
     constexpr int S = 1 << LOGS;
     constexpr int NG = N / R;
     constexpr int G = (NG + NT - 1) / NT;
@@ -49,7 +49,7 @@ __device__ __forceinline__ void pass(const cplx<T>* __restrict__ tw, int twstep,
         const int k = tid + gg * NT;
         if (NG % NT == 0 || k < NG) {
             const int j = k & (S - 1);
-            if (S > 1) twiddle<T, R, INV>(x[gg], j, twstep * (N / (S * R)), tw);
+            if constexpr (S > 1) twiddle_by<T, R>(x[gg], load_twiddles_c<T, R, S, INV>(j, tw));
             reg_dft<T, R, INV>(x[gg]);
             if constexpr (S == 1) {
                 static_assert(R == 16, "pass: the span-1 pass is radix 16");
@@ -68,18 +68,18 @@ __device__ __forceinline__ void pass(const cplx<T>* __restrict__ tw, int twstep,
 
 // Passes of span 16^s, s >= 1, up to the last one, over the padded array a.
 template <class T, int LOGN, int LOGS, int NT, bool INV, class ST>
-__device__ __forceinline__ void rest(cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, ST last_st, int tid) {
+__device__ __forceinline__ void rest(cplx<T>* a, const cplx<T>* __restrict__ tw, ST last_st, int tid) {
     constexpr int N = 1 << LOGN;
     constexpr int LEFT = LOGN - LOGS;   // log2 of the radices still to apply
     auto lds = [&](int, int pi) { return a[pi]; };
     auto sts = [&](int, int pi, cplx<T> v) { a[pi] = v; };
     if constexpr (LEFT > 4) {
-        pass<T, N, 16, LOGS, NT, INV, true>(tw, twstep, lds, sts, tid);
+        pass<T, N, 16, LOGS, NT, INV, true>(tw, lds, sts, tid);
         __syncthreads();
-        rest<T, LOGN, LOGS + 4, NT, INV>(a, tw, twstep, last_st, tid);
+        rest<T, LOGN, LOGS + 4, NT, INV>(a, tw, last_st, tid);
     } else {
         constexpr int R = 1 << LEFT;
-        pass<T, N, R, LOGS, NT, INV, true>(tw, twstep, lds, last_st, tid);
+        pass<T, N, R, LOGS, NT, INV, true>(tw, lds, last_st, tid);
     }
 }
 
@@ -90,15 +90,15 @@ __device__ __forceinline__ void rest(cplx<T>* a, const cplx<T>* __restrict__ tw,
 // barrier.  The barriers are the block's: side-by-side transforms (tid = the
 // thread's index in its transform's group) run their passes in step.
 template <class T, int LOGN, int NT, bool INV, bool SYNC, class LD, class ST>
-__device__ __forceinline__ void fft(cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, LD ld, ST st,
+__device__ __forceinline__ void fft(cplx<T>* a, const cplx<T>* __restrict__ tw, LD ld, ST st,
                                     int tid = -1) {
     constexpr int N = 1 << LOGN;
     static_assert(LOGN >= 8, "fft: at least 256 points");
     if (tid < 0) tid = threadIdx.x;
     auto sts = [&](int, int pi, cplx<T> v) { a[pi] = v; };
-    pass<T, N, 16, 0, NT, INV, SYNC>(tw, twstep, ld, sts, tid);
+    pass<T, N, 16, 0, NT, INV, SYNC>(tw, ld, sts, tid);
     __syncthreads();
-    rest<T, LOGN, 4, NT, INV>(a, tw, twstep, st, tid);
+    rest<T, LOGN, 4, NT, INV>(a, tw, st, tid);
     __syncthreads();
 }
 

@@ -3,7 +3,7 @@
 // A transform of N = 2^LOGN points (LOGN >= 5) is decimation in time with register
 // passes of radix 16, ..., 16 and a last one of 2, 4, 8 or 16: the radices, twiddle
 // products and order of operations of the Stockham passes in common.cuh, so both
-// give the same bits.  What differs is where the values live: element with pass
+// give the same bits.  Twiddles come from the compact tables (twc_offset, common.cuh).  What differs is where the values live: element with pass
 // digits d_0 (of the first pass), d_1, ... sits at position d_0 + 16 d_1 + 256 d_2 ...
 // at slot(position), so
 //   * every pass but the first reads and writes the same positions (one barrier
@@ -21,11 +21,13 @@
 namespace hpx {
 namespace ip {
 
-// One spare slot every 16, every 256 and four every 4096 elements: the 8-byte
-// accesses of the passes are free of bank conflicts, those of the first pass's
-// stores at most two ways.
-__host__ __device__ constexpr int slot(int i) { return i + (i >> 4) + (i >> 8) + ((i >> 12) << 2); }
-__host__ __device__ constexpr int slots(int n) { return slot(n); }   // of an n-point transform
+// One spare slot every 16 and every 256 elements, 8 where bit 12 is set and 20 where
+// bit 13 is: the 8-byte accesses of the passes are free of bank conflicts, but for the
+// first pass's stores at 512 to 2048 points (two to four ways).
+__host__ __device__ constexpr int slot(int i) {
+    return i + (i >> 4) + (i >> 8) + ((i >> 9) & 24) + ((i >> 11) & 4);
+}
+__host__ __device__ constexpr int slots(int n) { return slot(n - 1) + 1; }   // of an n-point transform
 
 __host__ __device__ constexpr int npass(int logn) { return (logn + 3) / 4; }
 // radix of pass i (from 0); its span (product of the radices before it) is 16^i
@@ -68,16 +70,16 @@ __device__ __forceinline__ void first_pass(cplx<T>* a, int tid, LD ld) {
 // Pass I of span S = 16^I and radix R over the whole transform, in place, after a
 // barrier; the first group's twiddles are read ahead of it.
 template <class T, int LOGN, int I, int NT, bool INV>
-__device__ __forceinline__ void inner_pass(cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, int tid) {
+__device__ __forceinline__ void inner_pass(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid) {
     constexpr int N = 1 << LOGN, R = radix(LOGN, I), S = 1 << (4 * I), NG = N / R, G = (NG + NT - 1) / NT;
-    Twiddles<T> t = load_twiddles<T, R, INV>(tid & (S - 1), twstep * (N / (S * R)), tw);
+    Twiddles<T> t = load_twiddles_c<T, R, S, INV>(tid & (S - 1), tw);
     __syncthreads();
 #pragma unroll
     for (int gg = 0; gg < G; ++gg) {
         const int k = tid + gg * NT;
         if (NG % NT != 0 && k >= NG) break;
         const int j = k & (S - 1);
-        if (gg > 0 && NT % S != 0) t = load_twiddles<T, R, INV>(j, twstep * (N / (S * R)), tw);
+        if (gg > 0 && NT % S != 0) t = load_twiddles_c<T, R, S, INV>(j, tw);
         cplx<T>* e = a + slot((k / S) * (S * R) + j);
         cplx<T> x[R];
 #pragma unroll
@@ -91,10 +93,10 @@ __device__ __forceinline__ void inner_pass(cplx<T>* a, const cplx<T>* __restrict
 
 // The passes between the first and the last.
 template <class T, int LOGN, int NT, bool INV, int I = 1>
-__device__ __forceinline__ void inner_passes(cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, int tid) {
+__device__ __forceinline__ void inner_passes(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid) {
     if constexpr (I < npass(LOGN) - 1) {
-        inner_pass<T, LOGN, I, NT, INV>(a, tw, twstep, tid);
-        inner_passes<T, LOGN, NT, INV, I + 1>(a, tw, twstep, tid);
+        inner_pass<T, LOGN, I, NT, INV>(a, tw, tid);
+        inner_passes<T, LOGN, NT, INV, I + 1>(a, tw, tid);
     }
 }
 
@@ -106,17 +108,17 @@ __host__ __device__ constexpr int out_radix(int logn, int nt) { return logn == 1
 // st(index, q, gg, value) for q < LO or q >= HI.  PRE: the first group's twiddles are
 // read ahead of the barrier.
 template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE, class ST>
-__device__ __forceinline__ void last_pass(const cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, int tid,
+__device__ __forceinline__ void last_pass(const cplx<T>* a, const cplx<T>* __restrict__ tw, int tid,
                                           ST st) {
     constexpr int N = 1 << LOGN, R = last_radix(LOGN), S = N / R, G = (S + NT - 1) / NT;
     Twiddles<T> t;
-    if constexpr (PRE) t = load_twiddles<T, R, INV>(min(tid, S - 1), twstep, tw);
+    if constexpr (PRE) t = load_twiddles_c<T, R, S, INV>(min(tid, S - 1), tw);
     __syncthreads();
 #pragma unroll
     for (int gg = 0; gg < G; ++gg) {
         const int j = tid + gg * NT;
         if (S % NT != 0 && j >= S) break;
-        if (!PRE || gg > 0) t = load_twiddles<T, R, INV>(j, twstep, tw);
+        if (!PRE || gg > 0) t = load_twiddles_c<T, R, S, INV>(j, tw);
         const cplx<T>* e = a + slot(j);
         cplx<T> x[R];
 #pragma unroll
@@ -134,11 +136,11 @@ __device__ __forceinline__ void last_pass(const cplx<T>* a, const cplx<T>* __res
 // one behind the reads (st may store anywhere in a): outputs j + 256 q, q < LO or
 // q >= HI, to st(index, q, 0, value).
 template <class T, int NT, bool INV, int LO, int HI, class ST>
-__device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep,
+__device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>* __restrict__ tw,
                                                  int tid, ST st) {
     static_assert(NT == 256, "one thread per j");
     const cplx<T>* e = a + slot(tid);
-    const Twiddles<T> t = load_twiddles<T, 16, INV>(tid, twstep * 2, tw);
+    const Twiddles<T> t = load_twiddles_c<T, 16, 256, INV>(tid, tw);
     __syncthreads();
     cplx<T> x[16], y[16];
 #pragma unroll
@@ -154,7 +156,7 @@ __device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>
     for (int q = 0; q < 16; ++q) {
         const int k = tid + 256 * q;
         cplx<T> z[2] = {x[q], y[q]};
-        twiddle<T, 2, INV>(z, k, twstep, tw);
+        twiddle_by<T, 2>(z, load_twiddles_c<T, 2, 4096, INV>(k, tw));
         reg_dft<T, 2, INV>(z);
         if (q < LO || q >= HI) st(k, q, 0, z[0]);
         if (q + 16 < LO || q + 16 >= HI) st(k + 4096, q + 16, 0, z[1]);
@@ -165,15 +167,15 @@ __device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>
 // st may store to the positions of a (natural order): a thread only produces
 // positions that it alone has read.  Ends without a barrier.
 template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE = true, class LD, class ST>
-__device__ __forceinline__ void transform(cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, int tid, LD ld,
+__device__ __forceinline__ void transform(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid, LD ld,
                                           ST st) {
     first_pass<T, LOGN, NT, INV, false>(a, tid, ld);
     if constexpr (LOGN == 13 && NT == 256) {
-        inner_pass<T, LOGN, 1, NT, INV>(a, tw, twstep, tid);
-        last_passes_8192<T, NT, INV, LO, HI>(a, tw, twstep, tid, st);
+        inner_pass<T, LOGN, 1, NT, INV>(a, tw, tid);
+        last_passes_8192<T, NT, INV, LO, HI>(a, tw, tid, st);
     } else {
-        inner_passes<T, LOGN, NT, INV>(a, tw, twstep, tid);
-        last_pass<T, LOGN, NT, INV, LO, HI, PRE>(a, tw, twstep, tid, st);
+        inner_passes<T, LOGN, NT, INV>(a, tw, tid);
+        last_pass<T, LOGN, NT, INV, LO, HI, PRE>(a, tw, tid, st);
     }
 }
 
@@ -182,12 +184,12 @@ __device__ __forceinline__ void transform(cplx<T>* a, const cplx<T>* __restrict_
 // outputs i < N/2.  The barriers are the block's: side-by-side convolutions run
 // their passes in step.  Ends without one.
 template <class T, int LOGN, int NT, class LD, class KER, class ST>
-__device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__ tw, int twstep, int tid, LD ld,
+__device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid, LD ld,
                                          KER ker, ST st) {
     constexpr int N = 1 << LOGN, R = radix(LOGN, npass(LOGN) - 1), NG = N / 16, D = 16 / R;
     static_assert(NT >= NG, "the turn keeps one group per thread");
     first_pass<T, LOGN, NT, false, true>(a, tid, [&](int i, int) { return ld(i); });
-    inner_passes<T, LOGN, NT, false>(a, tw, twstep, tid);
+    inner_passes<T, LOGN, NT, false>(a, tw, tid);
     const bool on = NG == NT || tid < NG;
     __syncthreads();
     cplx<T> y[16];
@@ -198,7 +200,7 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
             cplx<T> x[R];
 #pragma unroll
             for (int q = 0; q < R; ++q) x[q] = e[slot((i + q * D) * NG)];
-            twiddle_by<T, R>(x, load_twiddles<T, R, false>(tid + i * NG, twstep, tw));
+            twiddle_by<T, R>(x, load_twiddles_c<T, R, N / R, false>(tid + i * NG, tw));
             reg_dft<T, R, false>(x);
 #pragma unroll
             for (int q = 0; q < R; ++q) {
@@ -214,8 +216,8 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
 #pragma unroll
         for (int r = 0; r < 16; ++r) to[r] = y[r];
     }
-    inner_passes<T, LOGN, NT, true>(a, tw, twstep, tid);
-    last_pass<T, LOGN, NT, true, R / 2, R, false>(a, tw, twstep, tid, [&](int i, int, int, cplx<T> v) { st(i, v); });
+    inner_passes<T, LOGN, NT, true>(a, tw, tid);
+    last_pass<T, LOGN, NT, true, R / 2, R, false>(a, tw, tid, [&](int i, int, int, cplx<T> v) { st(i, v); });
 }
 
 }  // namespace ip

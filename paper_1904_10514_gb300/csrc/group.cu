@@ -342,6 +342,7 @@ bool build_ring_list(hpx_plan_s* G) {
         J.shOff = t.shOff; J.chOff = t.chOff; J.bhOff = t.bhOff;
         J.shift = (const cplx<T>*)t.shift; J.chirp = (const cplx<T>*)t.chirp; J.bhat = (const cplx<T>*)t.bhat;
         J.tw = (const cplx<T>*)t.twid;
+        J.twc = (const cplx<T>*)t.twc;
         J.twlen = S->g.Lmax; J.p = S->g.p; J.Q = S->g.Q; J.L = S->g.L; J.npix = S->g.npix;
         jobs.push_back(J);
         // transform length of every ring pair, from the host copy of the geometry

@@ -450,8 +450,8 @@ struct BackInput {
 template <class T, int LOGQ, int NTQ, class V>
 __device__ __forceinline__ void ring_back_quarters(cplx<T>* buf, T* f, int sN, int sS, int n,
                                                    const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
-                                                   const cplx<T>* __restrict__ tw, int twlen, V in) {
-    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ>(buf, n, ch, bh, tw, twlen, in);
+                                                   const cplx<T>* __restrict__ tw, V in) {
+    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ>(buf, n, ch, bh, tw, in);
     const int jq = n >> 2;
     for (int q = threadIdx.x; q < jq; q += 4 * NTQ) {
         cplx<T> z[4];
@@ -467,9 +467,9 @@ __device__ __forceinline__ void ring_back_quarters(cplx<T>* buf, T* f, int sN, i
 template <class T, int LOGN, int NT, class V>
 __device__ __forceinline__ void ring_back_whole(cplx<T>* buf, T* f, int sN, int sS, int n,
                                                 const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
-                                                const cplx<T>* __restrict__ tw, int twlen, V in) {
+                                                const cplx<T>* __restrict__ tw, V in) {
     ip::convolve<T, LOGN, NT>(
-        buf, tw, twlen >> LOGN, threadIdx.x, [&](int k) { return k < n ? mul(in(k), ch[k]) : mk<T>(T(0), T(0)); },
+        buf, tw, threadIdx.x, [&](int k) { return k < n ? mul(in(k), ch[k]) : mk<T>(T(0), T(0)); },
         [&](int k) { return bh[k]; },
         [&](int k, cplx<T> v) {
             if (k < n) {
@@ -483,10 +483,10 @@ __device__ __forceinline__ void ring_back_whole(cplx<T>* buf, T* f, int sN, int 
 // Rings of n = 2^LOGN points.
 template <class T, int LOGN, int NT, class V>
 __device__ __forceinline__ void ring_back_plain(cplx<T>* buf, T* f, int sN, int sS, const cplx<T>* __restrict__ tw,
-                                                int twlen, V in) {
+                                                V in) {
     constexpr int R = ip::out_radix(LOGN, NT);
     ip::transform<T, LOGN, NT, false, R, R>(
-        buf, tw, twlen >> LOGN, threadIdx.x, [&](int k, int) { return in(k); },
+        buf, tw, threadIdx.x, [&](int k, int) { return in(k); },
         [&](int k, int, int, cplx<T> v) {
             f[sN + k] = v.r;
             if (sN != sS) f[sS + k] = -v.i;
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(KIND ? 4 * NT : NT, MINB) ring_back_kernel(
     const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int* __restrict__ shifted_t,
     const int64_t* __restrict__ shOff_t, const int64_t* __restrict__ ch4Off_t, const int64_t* __restrict__ bh4Off_t,
     const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp4, const cplx<T>* __restrict__ bhat4,
-    const cplx<T>* __restrict__ tw, int twlen, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
+    const cplx<T>* __restrict__ tw, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
     extern __shared__ unsigned char smem_raw[];
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
     const int i = ringlist[blockIdx.y], b = blockIdx.x;
@@ -510,9 +510,9 @@ __global__ void __launch_bounds__(KIND ? 4 * NT : NT, MINB) ring_back_kernel(
                                shift + shOff_t[i], n, L, sN == sS, shifted_t[i] != 0};
     T* f = maps + (int64_t)b * npix;
     if constexpr (KIND == 2)
-        ring_back_quarters<T, LOGN, NT>(buf, f, sN, sS, n, chirp4 + ch4Off_t[i], bhat4 + bh4Off_t[i], tw, twlen, in);
+        ring_back_quarters<T, LOGN, NT>(buf, f, sN, sS, n, chirp4 + ch4Off_t[i], bhat4 + bh4Off_t[i], tw, in);
     else
-        ring_back_plain<T, LOGN, NT>(buf, f, sN, sS, tw, twlen, in);
+        ring_back_plain<T, LOGN, NT>(buf, f, sN, sS, tw, in);
 }
 
 // Every transform of at most 2048 points in one launch of 128 threads per ring
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3) ring_back_short_k
     const int* __restrict__ pow2_t, const int* __restrict__ logn_t, const int* __restrict__ logL_t,
     const int64_t* __restrict__ shOff_t, const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t,
     const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat,
-    const cplx<T>* __restrict__ tw, int twlen, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
+    const cplx<T>* __restrict__ tw, const cplx<T>* __restrict__ twc, int twlen, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
     extern __shared__ unsigned char smem_raw[];
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
     const int i = ringlist[blockIdx.y], b = blockIdx.x;
@@ -535,16 +535,16 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3) ring_back_short_k
     const cplx<T>*ch = chirp + chOff_t[i], *bh = bhat + bhOff_t[i];
     if (pow2_t[i]) {
         switch (logn_t[i]) {
-            case 11: ring_back_plain<T, 11, 128>(buf, f, sN, sS, tw, twlen, in); return;
-            case 10: ring_back_plain<T, 10, 128>(buf, f, sN, sS, tw, twlen, in); return;
-            case 9: ring_back_plain<T, 9, 128>(buf, f, sN, sS, tw, twlen, in); return;
+            case 11: ring_back_plain<T, 11, 128>(buf, f, sN, sS, twc, in); return;
+            case 10: ring_back_plain<T, 10, 128>(buf, f, sN, sS, twc, in); return;
+            case 9: ring_back_plain<T, 9, 128>(buf, f, sN, sS, twc, in); return;
             default: break;
         }
     } else {
         switch (logL_t[i]) {
-            case 11: ring_back_whole<T, 11, 128>(buf, f, sN, sS, n, ch, bh, tw, twlen, in); return;
-            case 10: ring_back_whole<T, 10, 128>(buf, f, sN, sS, n, ch, bh, tw, twlen, in); return;
-            case 9: ring_back_whole<T, 9, 128>(buf, f, sN, sS, n, ch, bh, tw, twlen, in); return;
+            case 11: ring_back_whole<T, 11, 128>(buf, f, sN, sS, n, ch, bh, twc, in); return;
+            case 10: ring_back_whole<T, 10, 128>(buf, f, sN, sS, n, ch, bh, twc, in); return;
+            case 9: ring_back_whole<T, 9, 128>(buf, f, sN, sS, n, ch, bh, twc, in); return;
             default: break;
         }
     }
@@ -586,15 +586,16 @@ void launch_ring_back(const hpx_plan_s* P, T* maps, cudaStream_t s) {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             kern<<<grid, 128, smem, s>>>(Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.pow2, t.logn, t.logL,
                                          t.shOff, t.chOff, t.bhOff, shift, (const cplx<T>*)t.chirp,
-                                         (const cplx<T>*)t.bhat, tw, g.Lmax, g.p, g.L, g.Q, g.npix, list);
+                                         (const cplx<T>*)t.bhat, tw, (const cplx<T>*)t.twc, g.Lmax, g.p, g.L, g.Q, g.npix,
+                                         list);
             continue;
         }
         const size_t smem = (size_t)(c.blue ? 4 * ip::slots(c.N / 4) : ip::slots(c.N)) * sizeof(cplx<T>);
         auto run = [&](auto kern, int threads) {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             kern<<<grid, threads, smem, s>>>(Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.shOff, t.ch4Off,
-                                             t.bh4Off, shift, (const cplx<T>*)t.chirp4, (const cplx<T>*)t.bhat4, tw,
-                                             g.Lmax, g.p, g.L, g.Q, g.npix, list);
+                                             t.bh4Off, shift, (const cplx<T>*)t.chirp4, (const cplx<T>*)t.bhat4,
+                                             (const cplx<T>*)t.twc, g.p, g.L, g.Q, g.npix, list);
         };
         if (c.N == 4096) {
             if (c.blue) run(ring_back_kernel<T, SYN, 10, 64, F ? 4 : 2, 2>, 256);

@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(32) lat_fft_small_kernel(const cplx<T>* __rest
 template <class T, int LOGM, int NT, int MINB, bool PW>
 __global__ void __launch_bounds__(NT, MINB) lat_fft_pair_kernel(
     const cplx<T>* __restrict__ U, cplx<T>* __restrict__ bvec, const T* __restrict__ dec,
-    const cplx<T>* __restrict__ pw, const cplx<T>* __restrict__ tw, int twlen, int p, int L, int P2,
+    const cplx<T>* __restrict__ pw, const cplx<T>* __restrict__ tw, int p, int L, int P2,
     float* __restrict__ bscale, unsigned char* __restrict__ bpk) {
     constexpr int M = 1 << LOGM, R = ip::out_radix(LOGM, NT), NG1 = M / R, G1 = (NG1 + NT - 1) / NT;
     constexpr int LO = R == 2 ? 1 : R / 4 + 1, HI = R == 2 ? 1 : 3 * R / 4;
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(NT, MINB) lat_fft_pair_kernel(
         return v;
     };
     ip::transform<T, LOGM, NT, false, LO, HI>(
-        u, tw, twlen / M, tid, [&](int t, int r) { return src[r < 8 || (r == 8 && t == M / 2) ? t : M + M / 2 - t]; },
+        u, tw, tid, [&](int t, int r) { return src[r < 8 || (r == 8 && t == M / 2) ? t : M + M / 2 - t]; },
         [&](int j, int q, int gg, cplx<T> v) {
             // (the ranges of gg and q are known at compile time)
             if (q < LO && gg * NT + q * NG1 <= M / 4) {
@@ -566,7 +566,7 @@ void launch_lat_fft(const hpx_plan_s* P, cudaStream_t s, bool packed) {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             kern<<<dim3(g.B, (g.L + 2) / 2), threads, smem, s>>>(
                 (const cplx<T>*)P->U, (cplx<T>*)P->bvec, (const T*)P->t.dec, (const cplx<T>*)P->t.pw,
-                (const cplx<T>*)P->t.twid, g.Lmax, g.p, g.L, g.P2, bsc, inFft ? P->bpk : nullptr);
+                (const cplx<T>*)P->t.twc, g.p, g.L, g.P2, bsc, inFft ? P->bpk : nullptr);
         };
         // 16 elements per thread, at least a warp; 32 at 8192 points, where the last two
         // passes run on them in registers (with 512 threads and four passes: 1.61 ms

@@ -80,12 +80,12 @@ __device__ __forceinline__ void ring_rows_out(BUF zat, int n, int p, int L, cons
 // the output chirp), or with four of 2^LOGN >= n/2 points (quarters).
 template <class T, int LOGN, int NT>
 __device__ __forceinline__ void ring_plain(cplx<T>* buf, const T* __restrict__ f, int sN, int sS,
-                                           const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw, int twlen,
+                                           const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw,
                                            int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
     constexpr int N = 1 << LOGN, R = ip::out_radix(LOGN, NT);
     const bool equator = sN == sS;
     ip::transform<T, LOGN, NT, false, R, R, false>(
-        buf, tw, twlen / N, threadIdx.x,
+        buf, tw, threadIdx.x,
         [&](int k, int) { return mk<T>(f[sN + k], equator ? T(0) : f[sS + k]); },
         [&](int k, int, int, cplx<T> v) { buf[ip::slot(k)] = v; });
     __syncthreads();
@@ -95,11 +95,10 @@ __device__ __forceinline__ void ring_plain(cplx<T>* buf, const T* __restrict__ f
 template <class T, int LOGN, int NT>
 __device__ __forceinline__ void ring_whole(cplx<T>* buf, const T* __restrict__ f, int sN, int sS, int n,
                                            const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
-                                           const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw, int twlen,
+                                           const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw,
                                            int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
-    constexpr int N = 1 << LOGN;
     ip::convolve<T, LOGN, NT>(
-        buf, tw, twlen / N, threadIdx.x,
+        buf, tw, threadIdx.x,
         [&](int k) { return k < n ? mul(mk<T>(f[sN + k], f[sS + k]), ch[k]) : mk<T>(T(0), T(0)); },
         [&](int k) { return bh[k]; },
         [&](int k, cplx<T> v) {
@@ -112,24 +111,25 @@ template <class T, int LOGQ, int NTQ>
 __device__ __forceinline__ void ring_quarters(cplx<T>* buf, const T* __restrict__ f, int sN, int sS, int n,
                                               const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
                                               const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw,
-                                              int twlen, int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
+                                              int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
     constexpr int NT = 4 * NTQ;
     const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ>(
-        buf, n, ch, bh, tw, twlen, [&](int k) { return mk<T>(f[sN + k], f[sS + k]); });
+        buf, n, ch, bh, tw, [&](int k) { return mk<T>(f[sN + k], f[sS + k]); });
     R.natural(n, threadIdx.x, NT);
     ring_rows_out<T>([&](int k) { return R.at(k, n); }, n, p, L, ph, sh, ew, rowN, rowS, false, threadIdx.x, NT);
 }
 
 // The ring stage for the launches of one transform length and kind (KIND 0 plain, 1
 // whole, 2 quarters).  Bound by the shared-memory passes.  32 maps, Nside 1024: the
-// stage 1900 us on Stockham passes, now 1835; 200 maps of mixed Nside 6.53 to 5.71 ms
-// per call with the spreading and grid FFT (short rings most of it).
+// stage 1900 us on Stockham passes, 1835 in place, now 1598 with compact twiddles
+// (quarters of 8192 points 948 to 767, rings of 4096 559 to 513); 200 maps of mixed
+// Nside 6.53 to 5.63 ms per call with the spreading and grid FFT.
 template <class T, int LOGN, int NT, int MINB, int KIND>
 __global__ void __launch_bounds__(KIND == 2 ? 4 * NT : NT, MINB) ring_ip_kernel(
     const T* __restrict__ maps, cplx<T>* __restrict__ Y, const int* __restrict__ nphi_t,
     const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int64_t* __restrict__ shOff_t,
     const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t, const cplx<T>* __restrict__ shift,
-    const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat, const cplx<T>* __restrict__ tw, int twlen,
+    const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat, const cplx<T>* __restrict__ tw,
     int p, int Q, int64_t npix, const int* __restrict__ ringlist, T ew, const int* __restrict__ shifted_t, int L,
     const int64_t* __restrict__ mapIdx) {
     extern __shared__ unsigned char smem_raw[];
@@ -143,13 +143,13 @@ __global__ void __launch_bounds__(KIND == 2 ? 4 * NT : NT, MINB) ring_ip_kernel(
     const cplx<T>* ph = shift + shOff_t[i];
     const bool sh = shifted_t[i] != 0;
     if constexpr (KIND == 0) {
-        ring_plain<T, LOGN, NT>(buf, f, sN, sS, ph, tw, twlen, p, L, ew, sh, rowN, rowS);
+        ring_plain<T, LOGN, NT>(buf, f, sN, sS, ph, tw, p, L, ew, sh, rowN, rowS);
     } else {
         const cplx<T>*ch = chirp + chOff_t[i], *bh = bhat + bhOff_t[i];
         if constexpr (KIND == 1)
-            ring_whole<T, LOGN, NT>(buf, f, sN, sS, nphi_t[i], ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS);
+            ring_whole<T, LOGN, NT>(buf, f, sN, sS, nphi_t[i], ch, bh, ph, tw, p, L, ew, sh, rowN, rowS);
         else
-            ring_quarters<T, LOGN, NT>(buf, f, sN, sS, nphi_t[i], ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS);
+            ring_quarters<T, LOGN, NT>(buf, f, sN, sS, nphi_t[i], ch, bh, ph, tw, p, L, ew, sh, rowN, rowS);
     }
 }
 
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(NT, (LOGN <= 13 ? 1024 / NT : 1)) ring4_ct_ker
     const T* __restrict__ maps, cplx<T>* __restrict__ Y, const int* __restrict__ nphi_t,
     const int* __restrict__ startN_t, const int* __restrict__ startS_t, const int64_t* __restrict__ shOff_t,
     const int64_t* __restrict__ ch4Off_t, const int64_t* __restrict__ bh4Off_t, const cplx<T>* __restrict__ shift,
-    const cplx<T>* __restrict__ chirp4, const cplx<T>* __restrict__ bhat4, const cplx<T>* __restrict__ tw, int twlen,
+    const cplx<T>* __restrict__ chirp4, const cplx<T>* __restrict__ bhat4, const cplx<T>* __restrict__ tw,
     int p, int Q, int64_t npix, const int* __restrict__ ringlist, T ew, const int* __restrict__ shifted_t, int L,
     const int64_t* __restrict__ mapIdx) {
     constexpr int LOGQ = LOGN - 2, NQ = 1 << LOGQ, NTQ = NT / 4;
@@ -181,15 +181,14 @@ __global__ void __launch_bounds__(NT, (LOGN <= 13 ? 1024 / NT : 1)) ring4_ct_ker
     cplx<T>* qb = buf + s * QS;
     const cplx<T>* ch = chirp4 + ch4Off_t[i];
     const cplx<T>* bh = bhat4 + bh4Off_t[i];
-    const int twstep = twlen >> LOGQ;
     ct::fft<T, LOGQ, NTQ, false, false>(
-        qb, tw, twstep,
+        qb, tw,
         [&](int u, int) {
             return u < jq ? mul(mk<T>(f[sN + 4 * u + s], f[sS + 4 * u + s]), ch[u]) : mk<T>(T(0), T(0));
         },
         [&](int k, int pi, cplx<T> v) { qb[pi] = mul(v, bh[k]); }, ltid);
     ct::fft<T, LOGQ, NTQ, true, true>(
-        qb, tw, twstep, [&](int, int pi) { return qb[pi]; },
+        qb, tw, [&](int, int pi) { return qb[pi]; },
         [&](int k, int pi, cplx<T> v) { qb[pi] = k < jq ? mul(v, ch[k]) : v; }, ltid);
     const int S0 = ct::padc(jq);   // first slot past the Y_s values (S0 + jq <= QS)
     for (int q = tid; q < jq; q += NT) {
@@ -233,7 +232,7 @@ __device__ __forceinline__ void ring_pair(
     const int64_t* __restrict__ shOff_t, const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t,
     const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat,
     const cplx<T>* __restrict__ tw, int twlen, int p, int Q, int64_t npix, T ew, const int* __restrict__ shifted_t,
-    int L, const int64_t* __restrict__ mapIdx) {
+    int L, const int64_t* __restrict__ mapIdx, const cplx<T>* __restrict__ twc) {
     const int n = nphi_t[i];
     const int sN = startN_t[i], sS = startS_t[i];
     const bool equator = (sN == sS);
@@ -248,9 +247,9 @@ __device__ __forceinline__ void ring_pair(
         if (!pow2_t[i]) {
             const cplx<T>*ch = chirp + chOff_t[i], *bh = bhat + bhOff_t[i];
             switch (logL_t[i]) {
-                case 11: ring_whole<T, 11, NT>(buf, f, sN, sS, n, ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS); return;
-                case 10: ring_whole<T, 10, NT>(buf, f, sN, sS, n, ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS); return;
-                case 9: ring_whole<T, 9, NT>(buf, f, sN, sS, n, ch, bh, ph, tw, twlen, p, L, ew, sh, rowN, rowS); return;
+                case 11: ring_whole<T, 11, NT>(buf, f, sN, sS, n, ch, bh, ph, twc, p, L, ew, sh, rowN, rowS); return;
+                case 10: ring_whole<T, 10, NT>(buf, f, sN, sS, n, ch, bh, ph, twc, p, L, ew, sh, rowN, rowS); return;
+                case 9: ring_whole<T, 9, NT>(buf, f, sN, sS, n, ch, bh, ph, twc, p, L, ew, sh, rowN, rowS); return;
                 default: break;
             }
         }
@@ -313,14 +312,14 @@ __global__ void __launch_bounds__(NT > 0 ? NT : kRingThreads, NT > 0 ? (sizeof(T
     const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp,
     const cplx<T>* __restrict__ bhat, const cplx<T>* __restrict__ tw, int twlen, int p, int Q,
     int64_t npix, int npairs, const int* __restrict__ ringlist, T ew, const int* __restrict__ shifted_t, int L,
-    const int64_t* __restrict__ mapIdx) {
+    const int64_t* __restrict__ mapIdx, const cplx<T>* __restrict__ twc) {
     extern __shared__ unsigned char smem_raw[];
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
     // largest rings first: blockIdx.y = 0 is the equator
     const int i = ringlist ? ringlist[blockIdx.y] : npairs - 1 - (int)blockIdx.y;
     ring_pair<T, E, NT>(buf, i, blockIdx.x, maps, Y, nphi_t, startN_t, startS_t, pow2_t, logn_t, fftL_t, logL_t,
                         shOff_t, chOff_t, bhOff_t, shift, chirp, bhat, tw, twlen, p, Q, npix, ew, shifted_t, L,
-                        mapIdx);
+                        mapIdx, twc);
 }
 
 // The short-ring part of the ring stage of every sub-plan of an uneven batch
@@ -346,7 +345,7 @@ __global__ void __launch_bounds__(NT, (NT == 32 ? 16 : sizeof(T) == 4 ? 6 : 3)) 
         ring_pair<T, 16, (NT == kRingShortThreads ? NT : 0)>(
             buf, w.y, w.z, maps_base + J.mapoff, J.Y, J.nphi, J.startN, J.startS, J.pow2, J.logn, J.fftL, J.logL,
             J.shOff, J.chOff, J.bhOff, J.shift, J.chirp, J.bhat, J.tw, J.twlen, J.p, J.Q, J.npix, T(0), J.shifted,
-            J.L, J.mapIdx);
+            J.L, J.mapIdx, J.twc);
         __syncthreads();   // the next item overwrites the shared buffer
     }
 }
@@ -430,7 +429,7 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
         kern<<<grid, threads, smem, s>>>(
             maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.pow2, t.logn, t.fftL, t.logL, t.shOff,
             t.chOff, t.bhOff, (const cplx<T>*)t.shift, (const cplx<T>*)t.chirp, (const cplx<T>*)t.bhat,
-            (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix, g.npairs, list, ew, t.shifted, g.L, P->mapIdx);
+            (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix, g.npairs, list, ew, t.shifted, g.L, P->mapIdx, (const cplx<T>*)t.twc);
     };
     if (!P->ringList) {   // one launch sized for the largest transform
         launch(g.smem_ring, g.npairs, nullptr);
@@ -452,7 +451,7 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             kern<<<grid, 256, smem, s>>>(maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.shOff, t.ch4Off, t.bh4Off,
                                          (const cplx<T>*)t.shift, (const cplx<T>*)t.chirp4, (const cplx<T>*)t.bhat4,
-                                         (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix, P->ringList + c.first, ew,
+                                         (const cplx<T>*)t.twc, g.p, g.Q, g.npix, P->ringList + c.first, ew,
                                          t.shifted, g.L, P->mapIdx);
             continue;
         }
@@ -463,8 +462,7 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
                 maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.shOff, quarters ? t.ch4Off : t.chOff,
                 quarters ? t.bh4Off : t.bhOff, (const cplx<T>*)t.shift,
                 (const cplx<T>*)(quarters ? t.chirp4 : t.chirp), (const cplx<T>*)(quarters ? t.bhat4 : t.bhat),
-                (const cplx<T>*)t.twid, g.Lmax, g.p, g.Q, g.npix, P->ringList + c.first, ew, t.shifted, g.L,
-                P->mapIdx);
+                (const cplx<T>*)t.twc, g.p, g.Q, g.npix, P->ringList + c.first, ew, t.shifted, g.L, P->mapIdx);
         };
         // 16 elements per thread (32 for plain rings of 8192 points)
         constexpr bool F = sizeof(T) == 4;

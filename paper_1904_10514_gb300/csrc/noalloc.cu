@@ -37,7 +37,7 @@ __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Offsets {
-    size_t nphi, startN, startS, pow2, logn, fftL, logL, shOff, chOff, bhOff, shift, chirp, bhat, twid,
+    size_t nphi, startN, startS, pow2, logn, fftL, logL, shOff, chOff, bhOff, shift, chirp, bhat, twid, twc,
         poleN, poleS, polew, rowptr, ent, entw, dec, D, angOff, ang, skOff, skew, nstart, swts, shifted;
     size_t Y, bvec;
     int npole;
@@ -116,7 +116,7 @@ extern "C" int hpx_analyze_noalloc(int nside, int lmax, const float* maps, float
             o.pow2 = img.vec(tb.pow2); o.logn = img.vec(tb.logn); o.fftL = img.vec(tb.fftL); o.logL = img.vec(tb.logL);
             o.shOff = img.vec(tb.shOff); o.chOff = img.vec(tb.chOff); o.bhOff = img.vec(tb.bhOff);
             o.shift = img.real(tb.shift); o.chirp = img.real(tb.chirp); o.bhat = img.real(tb.bhat);
-            o.twid = img.real(tb.twid);
+            o.twid = img.real(tb.twid); o.twc = img.real(tb.twc);
             o.poleN = img.vec(tb.poleN); o.poleS = img.vec(tb.poleS); o.polew = img.vec(tb.polew);
             o.npole = (int)tb.polew.size();
             o.rowptr = img.vec(tb.rowptr); o.ent = img.vec(tb.ent); o.entw = img.real(tb.entw);
@@ -156,7 +156,7 @@ extern "C" int hpx_analyze_noalloc(int nside, int lmax, const float* maps, float
     t.pow2 = (int*)(b + o.pow2); t.logn = (int*)(b + o.logn); t.fftL = (int*)(b + o.fftL);
     t.logL = (int*)(b + o.logL); t.shOff = (int64_t*)(b + o.shOff); t.chOff = (int64_t*)(b + o.chOff);
     t.bhOff = (int64_t*)(b + o.bhOff); t.shift = b + o.shift; t.chirp = b + o.chirp; t.bhat = b + o.bhat;
-    t.twid = b + o.twid; t.poleN = (int*)(b + o.poleN); t.poleS = (int*)(b + o.poleS);
+    t.twid = b + o.twid; t.twc = b + o.twc; t.poleN = (int*)(b + o.poleN); t.poleS = (int*)(b + o.poleS);
     t.polew = (double*)(b + o.polew); t.npole = o.npole; t.rowptr = (int*)(b + o.rowptr);
     t.ent = (int*)(b + o.ent); t.entw = b + o.entw; t.dec = b + o.dec; t.D = b + o.D;
     t.angOff = (int64_t*)(b + o.angOff); t.ang = b + o.ang;

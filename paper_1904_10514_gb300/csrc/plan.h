@@ -18,6 +18,7 @@ struct DevTables {
         *fftL = nullptr, *logL = nullptr;
     int64_t *shOff = nullptr, *chOff = nullptr, *bhOff = nullptr;
     void *shift = nullptr, *chirp = nullptr, *bhat = nullptr, *twid = nullptr;   // cplx<T>
+    void* twc = nullptr;                            // cplx<T>: compact twiddle tables (twc_offset, common.cuh)
     int64_t *ch4Off = nullptr, *bh4Off = nullptr;   // quarter-length Bluestein tables (ring form 1)
     void *chirp4 = nullptr, *bhat4 = nullptr;       // cplx<T>
     int *poleN = nullptr, *poleS = nullptr;
@@ -196,7 +197,7 @@ struct RingJob {
     cplx<T>* Y;
     const int *nphi, *startN, *startS, *pow2, *logn, *fftL, *logL, *shifted;
     const int64_t *shOff, *chOff, *bhOff;
-    const cplx<T> *shift, *chirp, *bhat, *tw;
+    const cplx<T> *shift, *chirp, *bhat, *tw, *twc;
     int twlen, p, Q, L;
     int64_t npix;
 };

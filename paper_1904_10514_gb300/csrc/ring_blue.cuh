@@ -61,13 +61,13 @@ struct RingQuarters {
 template <class T, int LOGQ, int NTQ, class IN>
 __device__ __forceinline__ RingQuarters<T> quarter_transforms(cplx<T>* buf, int n, const cplx<T>* __restrict__ ch,
                                                               const cplx<T>* __restrict__ bh,
-                                                              const cplx<T>* __restrict__ tw, int twlen, IN in) {
+                                                              const cplx<T>* __restrict__ tw, IN in) {
     constexpr int NQ = 1 << LOGQ, QS = ip::slots(NQ);
     const int jq = n >> 2;
     const int s = threadIdx.x / NTQ, ltid = threadIdx.x - s * NTQ;
     cplx<T>* qb = buf + s * QS;
     ip::convolve<T, LOGQ, NTQ>(
-        qb, tw, twlen / NQ, ltid, [&](int u) { return u < jq ? mul(in(4 * u + s), ch[u]) : mk<T>(T(0), T(0)); },
+        qb, tw, ltid, [&](int u) { return u < jq ? mul(in(4 * u + s), ch[u]) : mk<T>(T(0), T(0)); },
         [&](int u) { return bh[u]; },
         [&](int u, cplx<T> v) {
             if (u < jq) qb[ip::slot(u)] = mul(v, ch[u]);
