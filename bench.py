@@ -36,8 +36,8 @@ MEASURED = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # still in L2 when a kernel ends are not counted, so a ratio can fall below 1.
 TRAFFIC_OVER_ALGORITHMIC = {
     "fused_fsht": (1.4479 + 0.1249) / 1.4828,                      # fused_tc_ws_kernel, packed b
-    "ring_fft": (0.11342 + 0.08983 + 0.31140 + 0.34239) / 0.94031,  # ring_ct_kernel + ring_fft_kernel
-    "lat_fft": (0.53804 + 0.24894) / 0.80688,                      # lat_fft_pair_ct_kernel, packed b
+    "ring_fft": (0.11342 + 0.08983 + 0.31140 + 0.34239) / 0.94031,  # ring stage
+    "lat_fft": (0.53804 + 0.24894) / 0.80688,                      # grid FFT, packed b
     "spread": (0.54846 + 0.49414) / 1.07532,                       # spread_rb_kernel
 }
 # forms of the FP32 run-time sweep kernel (hpx_plan_tuning)
