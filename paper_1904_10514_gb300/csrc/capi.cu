@@ -528,7 +528,7 @@ void tune_shapes(hpx_plan_s* P, const void* maps, void* alm, cudaEvent_t e0, cud
     g_tune_cache[key] = {P->ringE, P->latE, P->rotForm, P->packSep, P->ringForm};
 }
 
-// HPX_FLAG_AUTOTUNE: choose the launch shapes of the FFT stages (tune_shapes),
+// HPX_FLAG_AUTOTUNE: choose the forms of the stages (tune_shapes),
 // then time the operator path and the run-time sweeps on scratch buffers (3
 // analyses each after one warm-up) and keep the faster.
 int autotune(hpx_plan_s* P) {

@@ -248,7 +248,7 @@ int prepare_fused_tc(hpx_plan_s* P);
 // the launch (bvec -> beta, like launch_dense)
 int prepare_dense_tc(hpx_plan_s* P);
 // the synthesis operators on the tensor cores (from synM; 0 on success) and the
-// launch (alm -> bvec, like launch_synth_apply)
+// launch (alm -> bvec, like launch_operator_cols)
 int prepare_synth_tc(hpx_plan_s* P);
 void launch_synth_tc(const hpx_plan_s* P, const float* alm, cudaStream_t s);
 void launch_dense_tc(const hpx_plan_s* P, cudaStream_t s);
