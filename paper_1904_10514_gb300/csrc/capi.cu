@@ -14,6 +14,7 @@
 #include "../../include/hpx.h"
 #include "plan.h"
 #include "plan_math.h"
+#include "release_operators.h"
 
 namespace {
 
@@ -570,25 +571,7 @@ int autotune(hpx_plan_s* P) {
     if (cudaGetLastError() != cudaSuccess) return HPX_ERR_CUDA;
     P->tuned_ms[0] = ms[0] / 3;
     P->tuned_ms[1] = ms[1] / 3;
-    if (ms[1] < ms[0]) {   // keep the sweeps: release the operators
-        void* ptrs[] = {P->fusedM, P->synM ? nullptr : P->fusedOff, P->fusedTiles, P->tcOff, P->tcFirst,
-                        P->tcRinv, P->bscale, P->adjScale, P->bpk};
-        for (void* q : ptrs)
-            if (q) cudaFree(q);
-        P->fusedM = nullptr;
-        if (!P->synM) P->fusedOff = nullptr;
-        P->fusedTiles = nullptr;
-        P->tcOff = nullptr;
-        P->tcFirst = nullptr;
-        P->tcRinv = nullptr;
-        P->bscale = nullptr;
-        P->adjScale = nullptr;
-        P->bpk = nullptr;
-        P->bytes -= P->fused_bytes;
-        P->fused_bytes = 0;
-        P->use_tc = false;
-        P->flags |= HPX_FLAG_SWEEPS;
-    }
+    if (ms[1] < ms[0]) hpx::release_operators(P, [](void* q) { cudaFree(q); });   // keep the sweeps
     return HPX_OK;
 }
 
