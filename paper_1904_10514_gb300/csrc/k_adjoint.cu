@@ -583,7 +583,7 @@ void launch_ring_back(const hpx_plan_s* P, T* maps, cudaStream_t s) {
         if (c.N < kRingCtMin) {
             auto kern = ring_back_short_kernel<T, SYN>;
             const size_t smem = (size_t)std::max(ip::slots(c.N), c.N + c.N / 16) * sizeof(cplx<T>);
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_shared(kern);
             kern<<<grid, 128, smem, s>>>(Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.pow2, t.logn, t.logL,
                                          t.shOff, t.chOff, t.bhOff, shift, (const cplx<T>*)t.chirp,
                                          (const cplx<T>*)t.bhat, tw, (const cplx<T>*)t.twc, g.Lmax, g.p, g.L, g.Q, g.npix,
@@ -644,7 +644,7 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
         int logM = 0;
         while ((1 << logM) < g.M) ++logM;
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
-        cudaFuncSetAttribute(nufft_adj_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_shared(nufft_adj_kernel<T>);
         dim3 grid(g.L + 1, g.B);
         if (!launch_nufft2<T>(P, s))
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,
@@ -705,7 +705,7 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
         int logM = 0;
         while ((1 << logM) < g.M) ++logM;
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
-        cudaFuncSetAttribute(nufft_adj_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_shared(nufft_adj_kernel<T>);
         dim3 grid(g.L + 1, g.B);
         if (!launch_nufft2<T>(P, s))
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,

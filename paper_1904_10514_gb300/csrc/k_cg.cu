@@ -110,7 +110,7 @@ void launch_cg(const hpx_plan_s* P, cudaStream_t s) {
     for (int k = 0; k < 4; ++k) nmax = std::max(nmax, t.cgn[k]);
     const size_t smem = (size_t)(t.cgN + t.cgN / 16 + 4 * nmax) * sizeof(cplx<T>);
     auto kern = t.cgN > 16 * 512 ? cg_kernel<T, 32> : cg_kernel<T, 16>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(kern);
     const double tol = sizeof(T) == 4 ? 1e-7 : 1e-14;
     dim3 grid(g.L + 1, g.B);
     kern<<<grid, 512, smem, s>>>((cplx<T>*)P->bvec, (const cplx<T>*)t.cgH,

@@ -593,7 +593,7 @@ void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Mrows
         if (!Mrows) {
             auto run = [&](auto kern, int NB) {   // each operator read once: all maps in one block
                 const size_t smem = (size_t)2 * NB * ldm * sizeof(float);
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                allow_shared(kern);
                 kern<<<P->fused_ntiles, 128, smem, s>>>(M, P->fusedOff, P->fusedTiles, (const cplx<float>*)P->bvec,
                                                         (cplx<float>*)alm, g.P2, ldm, g.p, g.L, g.B, g.nalm);
             };
@@ -612,7 +612,7 @@ void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Mrows
     auto run = [&](auto kern, int NB) {
         constexpr int CH = 32 * 16 / sizeof(T);
         const size_t smem = (size_t)2 * NB * ((g.P2 - 1 + CH - 1) / CH * CH + 1) * sizeof(T);
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_shared(kern);
         dim3 grid(P->fused_ntiles, (g.B + NB - 1) / NB, per);
         kern<<<grid, 256, smem, s>>>(M, P->fusedOff, P->fusedTiles, (const cplx<T>*)P->bvec, alm, g.P2, ldm, g.p,
                                      g.L, g.B, g.nalm);

@@ -335,7 +335,7 @@ void launch_spread(const hpx_plan_s* P, cudaStream_t s) {
             const int nrw = t.spreadRows - t.spreadH + EW + DM;
             const size_t smem = (size_t)(32 * kZS + NS * 32 * nrw) * sizeof(cplx<float>);
             auto kern = spread_rb_kernel<EW, DM, NS>;
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_shared(kern);
             dim3 grid((H + 32) / 32, g.B);
             kern<<<grid, 256, smem, s>>>((const cplx<float>*)P->Y, (cplx<float>*)P->U, t.hstart, (const float*)t.hwts,
                                          t.spreadH, H, g.p, g.Q, g.L, nrw, rho);
@@ -343,7 +343,7 @@ void launch_spread(const hpx_plan_s* P, cudaStream_t s) {
         }
     }
     const size_t smem = (size_t)(32 * kZS + 32 * t.spreadRows) * sizeof(cplx<T>);
-    cudaFuncSetAttribute(spread_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(spread_kernel<T>);
     dim3 grid((H + 32) / 32, (g.L + 32) / 32, g.B);
     spread_kernel<T><<<grid, 256, smem, s>>>((const cplx<T>*)P->Y, (cplx<T>*)P->U, t.hstart, (const T*)t.hwts,
                                              t.spreadH, H, g.p, g.Q, g.L, rho);
@@ -601,7 +601,7 @@ void launch_nufft(const hpx_plan_s* P, cudaStream_t s) {
     while ((1 << logM) < g.M) ++logM;
     const size_t smem = (size_t)(g.M + g.M / 16 + g.Q) * sizeof(cplx<T>);
     auto kern = g.M > 16 * 512 ? nufft_kernel<T, 32> : nufft_kernel<T, 16>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(kern);
     dim3 grid(g.L + 1, g.B);
     kern<<<grid, 512, smem, s>>>((const cplx<T>*)P->Y, (cplx<T>*)P->bvec, t.nstart, (const T*)t.swts, t.spreadE,
                                  (const T*)t.dec, (const cplx<T>*)t.twid, g.Lmax, g.M, logM, g.p, g.Q, g.P2);

@@ -239,7 +239,7 @@ bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
             const int nrw = (t.interpRows - t.interpE + EW + DM) | 1;   // first window start .. last window end
             const size_t smem2 = (size_t)(32 * 33 + NS * 32 * nrw) * sizeof(cplx<float>);
             auto kern2 = interp_rb_kernel<EW, DM, NS>;
-            cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+            allow_shared(kern2);
             dim3 grid2((g.Q + 31) / 32, g.B);
             kern2<<<grid2, 256, smem2, s>>>((const cplx<float>*)P->U, (cplx<float>*)P->Y, t.tstart,
                                             (const float*)t.hwn, t.interpE, g.M / 2, g.p, g.Q, g.L, P->ldu, nrw);
@@ -248,7 +248,7 @@ bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
     }
     const int nrw = t.interpRows | 1;
     const size_t smem2 = (size_t)(32 * 33 + 32 * nrw) * sizeof(cplx<T>);
-    cudaFuncSetAttribute(interp_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+    allow_shared(interp_kernel<T>);
     dim3 grid2((g.Q + 31) / 32, (g.L + 32) / 32, g.B);
     interp_kernel<T><<<grid2, 256, smem2, s>>>((const cplx<T>*)P->U, (cplx<T>*)P->Y, t.tstart, (const T*)t.hwn,
                                                t.interpE, g.M / 2, g.p, g.Q, g.L, P->ldu, nrw);

@@ -424,7 +424,7 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
         const size_t smem = (size_t)(brief ? ring_short_slots(N) : N + N / 16) * sizeof(cplx<T>);
         auto kern = brief ? ring_fft_kernel<T, 16, kRingShortThreads>
                           : big ? ring_fft_kernel<T, 32, 0> : ring_fft_kernel<T, 16, 0>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_shared(kern);
         dim3 grid(g.B, nrings);
         kern<<<grid, threads, smem, s>>>(
             maps, (cplx<T>*)P->Y, t.nphi, t.startN, t.startS, t.pow2, t.logn, t.fftL, t.logL, t.shOff,

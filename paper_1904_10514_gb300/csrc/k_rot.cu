@@ -336,7 +336,7 @@ void launch_rot(const hpx_plan_s* P, T* alm, cudaStream_t s) {
     const int nmax = g.L / 2 + 1;
     constexpr int G = 1;
     const size_t smem = (size_t)2 * nmax * 2 * G * sizeof(T);
-    cudaFuncSetAttribute(rot_stage_kernel<T, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_shared(rot_stage_kernel<T, G>);
     dim3 grid(g.L + 1, g.B);
     rot_stage_kernel<T, G><<<grid, 64, smem, s>>>((const cplx<T>*)P->beta, (cplx<T>*)alm, P->t.angOff,
                                                   (const cplx<T>*)P->t.ang, g.p, g.P2, g.L, g.B, g.nalm, nmax);

@@ -205,6 +205,16 @@ template <class T>
 void launch_ring_list(const RingJob<T>* jobs, const int4* items, int nitems, int nlong, const T* maps_base,
                       cudaStream_t s);
 
+// Lets a kernel ask for more than 48 KB of dynamic shared memory.  The limit belongs to the
+// kernel and not to the launch, so a kernel whose size depends on the plan gets one
+// value from every launch, above what any plan needs: with the plan's own
+// size, a thread that launches for a smaller plan would lower it under another one.
+constexpr int kSharedLimit = 220 * 1024;   // 227 KB less room for static shared memory
+template <class K>
+void allow_shared(K kern) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSharedLimit);
+}
+
 // ring transforms of this many points or more run in launches of one length and
 // one kind (plain or Bluestein) with the compile-time FFT of fft_ct.cuh
 constexpr int kRingCtMin = 4096;
