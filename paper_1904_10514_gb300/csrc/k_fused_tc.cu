@@ -1177,24 +1177,6 @@ void launch_adjoint_tc(const hpx_plan_s* P, const float* alm, cudaStream_t s, fl
 #endif
 }
 
-// S^T of the synthesis on the tensor cores: bvec -> alm, times outScale (k_healpix.cu)
-void launch_sh_adjoint_tc(const hpx_plan_s* P, float* alm, cudaStream_t s, float outScale) {
-#if HPX_TC_F16
-    const auto& g = P->g;
-    pack_x_kernel<false><<<dim3(g.B, g.L + 1), 256, 0, s>>>(
-        (const cplx<float>*)P->bvec, (const float*)P->synRinv, nullptr, nullptr, P->synRowBase,
-        (unsigned char*)P->synBpk, (float*)P->synScale, g.L, g.p, g.P2, g.nalm, 1.f);
-    const int nt = (g.L / 2 + 1 + TM - 1) / TM;   // of the longest chain
-    const size_t smem_h = NSH * (TILE_A + TILE_BP);
-    cudaFuncSetAttribute(fused_tc_t_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_h);
-    fused_tc_t_kernel<false><<<dim3((g.L + 1) * 2 * nt, (g.B + 31) / 32), NTW, smem_h, s>>>(
-        (const unsigned char*)P->synT, P->synOff, nullptr, (const unsigned char*)P->synBpk, (const float*)P->synScale,
-        (cplx<float>*)alm, g.P2, g.p, g.L, g.B, g.nalm, nt, outScale, P->d_status);
-#else
-    (void)P; (void)alm; (void)s; (void)outScale;
-#endif
-}
-
 int prepare_synth_tc(hpx_plan_s* P) {
 #if HPX_TC_F16
     const auto& g = P->g;

@@ -17,10 +17,10 @@
 //   NUFFT          the transpose of the synthesis' type-2 NUFFT: the analysis'
 //                  type-1 NUFFT (spreading + grid FFT);
 //   Legendre       the transpose of the synthesis' order-m -> latitude-Fourier
-//                  conversion: its operators R_{m,c} Es applied row-wise (FP32 plans
-//                  of more than 8 maps: on the tensor cores, from the tiles of S^T;
-//                  else the per-order operator kernel on synM), or Es applied by the
-//                  dense kernel followed by the forward Givens sweeps.
+//                  conversion: its operators R_{m,c} Es applied row-wise (the
+//                  per-order operator kernels on synM: FP32 products, also where the
+//                  synthesis itself takes FP16 pairs, from 9 maps on), or Es applied
+//                  by the dense kernel followed by the forward Givens sweeps.
 #include "plan.h"
 
 namespace hpx {
@@ -57,13 +57,6 @@ void launch_sh_adjoint(const hpx_plan_s* P, const T* maps, T* alm, cudaStream_t 
     zero_pole_rows_kernel<T><<<g.B, 256, 0, s>>>((cplx<T>*)P->Y, g.p, g.Q);
     launch_spread<T>(P, s);
     launch_lat_fft<T>(P, s);
-    bool done = false;
-    if constexpr (sizeof(T) == 4)
-        if (P->synT) {   // on the tensor cores, from the synthesis' own tiles
-            launch_sh_adjoint_tc(P, (float*)alm, s, 1.f);
-            done = true;
-        }
-    if (done) return;
     if (P->synM) {
         launch_fused<T>(P, alm, s, P->synM);
     } else {

@@ -274,7 +274,6 @@ int build_fused(hpx_plan_s* P, const double* D64, const cplx<double>* skew64, cu
 template <class T>
 void launch_operator_cols(const hpx_plan_s* P, const void* M, bool quad, const T* alm, cudaStream_t s, T wpos, bool dropim);
 void launch_adjoint_tc(const hpx_plan_s* P, const float* alm, cudaStream_t s, float wpos);
-void launch_sh_adjoint_tc(const hpx_plan_s* P, float* alm, cudaStream_t s, float outScale);
 // float offset of element (row r of a tile with rp rows, column k) in the
 // tensor-core layout of M, relative to the tile's first chunk
 __host__ __device__ inline int64_t tc_elem(int rp, int r, int k) {
