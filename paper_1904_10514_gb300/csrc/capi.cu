@@ -74,7 +74,7 @@ void free_plan(hpx_plan_s* P) {
                     t.bhOff, t.pw, t.shift, t.chirp, t.bhat, t.twid, t.twc, t.ch4Off, t.bh4Off, t.chirp4, t.bhat4, t.poleN,
                     t.poleS, t.polew, t.rowptr,
                     t.ent, t.entw, t.dec, t.D, t.tstart, t.hwn, t.angOff, t.ang, t.skOff, t.skew, t.skewT, t.nrowptr, t.nent, t.nentw, t.nstart, t.swts, t.hstart, t.hwts, t.Es, t.shifted, t.C, t.cgH, P->Y, P->U, P->bvec,
-                    P->fusedM, P->fusedOff, P->fusedTiles, P->tcOff, P->tcFirst, P->tcRinv, P->bscale, P->adjScale, P->d_status, P->synM, P->ringList,
+                    P->fusedM, P->fusedOff, P->fusedTiles, P->tcOff, P->tcFirst, P->tcRinv, P->bscale, P->d_status, P->synM, P->ringList,
                     P->jres, P->jalm, P->dTC, P->dRinv, P->dTiles, P->dTcOff, P->mapIdx, P->bpk, P->synT,
                     P->synRinv, P->synTiles, P->synNch, P->synOff, P->synRowBase, P->synScale, P->synBpk};
     for (void* q : ptrs)

@@ -613,14 +613,9 @@ template <class T>
 void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, T wpos) {
     const auto& g = P->g;
     const auto& t = P->t;
-    if (P->fusedM) {   // the plan's operators, transposed
-        if constexpr (sizeof(T) == 4) {
-            if (P->use_tc) launch_adjoint_tc(P, (const float*)alm, s, (float)wpos);
-            else launch_operator_cols<T>(P, P->fusedM, g.B <= 8, alm, s, wpos, true);
-        } else {
-            launch_operator_cols<T>(P, P->fusedM, false, alm, s, wpos, true);
-        }
-    } else {
+    if (P->fusedM && !P->use_tc) {   // the plan's operators, transposed
+        launch_operator_cols<T>(P, P->fusedM, sizeof(T) == 4 && g.B <= 8, alm, s, wpos, true);
+    } else {   // (operators stored as FP16 pairs hold 22 bits: the sweeps keep FP32 throughout)
         const int ngroups = (2 * g.B + 31) / 32;
         const int nitems = (g.L + 1) * 2 * ngroups;
         const int G = sweep_orders_per_warp(g.B), sitems = (g.L / 2 / G + 1) * 4 * ngroups;

@@ -650,201 +650,6 @@ __global__ void __launch_bounds__(NTW, 2) fused_tc_ws_kernel(
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(dtmem), "r"(NACC * TN) : "memory");
 }
 
-// The transposed contraction with the same stored operators: out[o] = sum_i
-// O[i][o] x[i], where the stored tiles (row tiles of 128 of i, K-chunks of 32 of o)
-// have the reduction along their rows.  A stored core matrix (8 rows x 8 halves) is,
-// read the other way, an MN-major core matrix (8 consecutive o per 16 bytes, 8
-// consecutive i), so the tensor cores take the tiles as they are (A transposed in
-// the instruction descriptor) and no second copy of the operators is needed.
-// CTA tile: (m, c, 128 outputs) x 32 maps; reduction in chunks of 32 rows: the copy
-// warp gathers, one 512-byte bulk copy per lane, the 4 groups of 8 rows x 4 K-chunks
-// x (hi, lo) of a chunk and places group ig of K-chunk j at 2048 ig + 512 j, so that
-// core matrices are 128 bytes apart along o and 2048 along i; the rest of the
-// pipeline is fused_tc_ws_kernel's.  Row groups past the tile's last (at most 3)
-// repeat its last one: x is zero there.  Outputs past the operators' K-chunks are
-// other rows of D, which nothing reads.
-// ADJ: O = M (tcOff, tcFirst, chunks of all P2 modes), x = the weighted coefficients,
-// out = bvec[map][m][par][o], o < P2.  !ADJ: O = S^T (synT: rows = modes, chunks =
-// the chain's degrees), x = the right-hand sides, out = a_{m+c+2o}^m times outScale:
-// the transposed synthesis.  The row scales of O are folded into x when it is packed.
-// Bound by the stream of the operators.  16 maps, Nside 256: the
-// transposed synthesis 339 us on the FP32 pipes, now 75 us and 43 us for packing x; the
-// adjoint 336 + 239 us as sweeps and table.
-constexpr uint32_t kIdescHT = kIdescH | (1u << 15);   // A is MN-major
-
-__device__ __forceinline__ void mma_f16_t(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        :
-        : "r"(dtmem), "l"(adesc), "l"(bdesc), "r"(kIdescHT), "r"(acc));
-}
-
-template <bool ADJ>
-__global__ void __launch_bounds__(NTW, 2) fused_tc_t_kernel(
-    const unsigned char* __restrict__ Mh, const int64_t* __restrict__ tileOff, const int* __restrict__ tileFirst,
-    const unsigned char* __restrict__ bpk, const float* __restrict__ xscale, cplx<float>* __restrict__ out, int P2,
-    int p, int L, int B, int64_t nalm, int not_, float outScale, int* __restrict__ status) {
-    extern __shared__ __align__(1024) unsigned char smem_w[];
-    unsigned char* const sA = smem_w;                  // NSH x TILE_A: 32 rows x 128 outputs (hi, then lo)
-    unsigned char* const sB = smem_w + NSH * TILE_A;   // NSH x TILE_BP: packed x chunks (hi, lo)
-    __shared__ __align__(8) uint64_t fullA[NSH], emptyA[NSH], accFull[NACC], accEmpty[NACC];
-    __shared__ uint32_t tmem_base;
-    __shared__ int abort_, issuedA, seenA, committed;
-    __shared__ float tinv[TN / 2];
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ot = blockIdx.x % not_, mc = blockIdx.x / not_;
-    const int m = mc >> 1, c = mc & 1, o0 = ot * TM;
-    const int par = ((m & 1) + c) & 1;
-    const int nchain = chain_len(m, c, L);
-    const int nout = ADJ ? P2 : nchain, nred = ADJ ? nchain : P2;
-    if (o0 >= nout) return;                                    // (the grid covers the longest chain)
-    const int b0 = blockIdx.y * (TN / 2);
-    const int nchB = (P2 + KC - 1) / KC;                       // K-chunks of a packed half
-    const int nchO = (nout + KC - 1) / KC;                     // stored K-chunks of the operator
-    const int nj = min(4, nchO - o0 / KC);                     // of this CTA's outputs
-    const int nchunks = (nred + KC - 1) / KC;
-    const int first = ADJ ? tileFirst[m * 2 + c] : mc * ((P2 + TM - 1) / TM);
-    volatile int* abort = &abort_;
-
-    if (warp == 0) {   // NACC x 64 accumulator columns
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(NACC * TN)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (tid == 0) {
-        for (int q = 0; q < NSH; ++q) {
-            mbar_init(smem_u32(&fullA[q]), 1);
-            mbar_init(smem_u32(&emptyA[q]), 1);
-        }
-        for (int q = 0; q < NACC; ++q) {
-            mbar_init(smem_u32(&accFull[q]), 1);
-            mbar_init(smem_u32(&accEmpty[q]), NW);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        abort_ = 0;
-        issuedA = 0;
-        seenA = 0;
-        committed = 0;
-    }
-    if (tid < TN / 2) {
-        const int bm = b0 + tid;
-        tinv[tid] = bm < B ? outScale / pow2_scale(xscale[((int64_t)bm * (L + 1) + m) * 2 + c], 13) : 0.f;
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t dtmem = tmem_base;
-
-    if (warp == 4) {
-        // ---------------------------------------------------------- copies (one lane each)
-        const unsigned char* Bt = bpk + (((int64_t)blockIdx.y * (L + 1) + m) * 2 + c) * nchB * TILE_BP;
-        const int j = lane & 3, ig = (lane >> 2) & 3, lo = lane >> 4;   // K-chunk, row group, part
-        for (int ch = 0; ch < nchunks; ++ch) {
-            const int s = ch % NSH;
-            const bool go = ch < NSH || ws_wait(smem_u32(&emptyA[s]), (uint32_t)((ch / NSH + 1) & 1), abort);
-            if (!__all_sync(0xffffffffu, go)) break;
-            const uint32_t fb = smem_u32(&fullA[s]);
-            if (lane == 0) {
-                mbar_expect_tx(fb, (uint32_t)nj * 4096u + TILE_BP);
-                issuedA = ch + 1;
-                bulk_g2s_keep(smem_u32(sB + s * TILE_BP), Bt + (int64_t)ch * TILE_BP, TILE_BP, fb);
-            }
-            __syncwarp();
-            if (j < nj) {
-                const int t = ch >> 2;   // row tile; its stored rows, a multiple of 8
-                const int rp = (min(TM, nred - t * TM) + 7) & ~7;
-                const int rg = min((ch & 3) * 4 + ig, (rp >> 3) - 1);
-                const unsigned char* src = Mh + tileOff[first + t] * 4 + (int64_t)(o0 / KC + j) * rp * 128 +
-                                           (lo ? rp * 64 : 0) + rg * 512;
-                bulk_g2s(smem_u32(sA + s * TILE_A + lo * 8192 + ig * 2048 + j * 512), src, 512u, fb);
-            }
-        }
-    } else if (warp == 5) {
-        // ---------------------------------------------------------- MMAs
-        if (lane == 0) {
-            for (int ch = 0; ch < nchunks; ++ch) {
-                const int s = ch % NSH, a = ch % NACC;
-                if (!ws_wait(smem_u32(&fullA[s]), (uint32_t)((ch / NSH) & 1), abort)) break;
-                seenA = ch + 1;
-                if (ch >= NACC && !ws_wait(smem_u32(&accEmpty[a]), (uint32_t)((ch / NACC + 1) & 1), abort)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t aH = smem_u32(sA + s * TILE_A), aL = aH + 8192;
-                const uint32_t bH = smem_u32(sB + s * TILE_BP), bL = bH + TILE_H;
-                const uint32_t d = dtmem + (uint32_t)(a * TN);
-#pragma unroll
-                for (int ks = 0; ks < KC / 16; ++ks) {   // 16 rows: two row groups of A
-                    const uint32_t oa = ks * 4096, ob = ks * 256;
-                    mma_f16_t(d, make_desc(aH + oa, 2048, 128), make_desc(bL + ob, 128, 512), ks > 0 ? 1u : 0u);
-                    mma_f16_t(d, make_desc(aL + oa, 2048, 128), make_desc(bH + ob, 128, 512), 1u);
-                }
-#pragma unroll
-                for (int ks = 0; ks < KC / 16; ++ks) {
-                    const uint32_t oa = ks * 4096, ob = ks * 256;
-                    mma_f16_t(d, make_desc(aH + oa, 2048, 128), make_desc(bH + ob, 128, 512), 1u);
-                }
-                mma_commit(smem_u32(&emptyA[s]));
-                mma_commit(smem_u32(&accFull[a]));
-                committed = ch + 1;
-            }
-        }
-    } else {
-        // ---------------------------------------------------------- workers
-        float acc[64];
-#pragma unroll
-        for (int q = 0; q < 64; ++q) acc[q] = 0.f;
-        const uint32_t trow = dtmem + ((uint32_t)(32 * warp) << 16);
-        bool ok = true;
-        for (int ch = 0; ch < nchunks && ok; ++ch) {
-            const int a = ch % NACC;
-            if (!ws_wait(smem_u32(&accFull[a]), (uint32_t)((ch / NACC) & 1), abort)) {
-                ok = false;
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                uint32_t v[16];
-                tmem_ld16(trow + (uint32_t)(a * TN + 16 * h), v);
-#pragma unroll
-                for (int q = 0; q < 16; ++q) acc[16 * h + q] += __uint_as_float(v[q]);
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            mbar_arrive(smem_u32(&accEmpty[a]));
-        }
-        const int o = o0 + 32 * warp + lane;
-        if (ok && o < nout) {
-            const int64_t base = (int64_t)m * (2 * L + 1 - m) / 2 + m + c + 2 * (int64_t)o;
-#pragma unroll
-            for (int q = 0; q < 32; ++q)
-                if (b0 + q < B) {
-                    const cplx<float> v = mk<float>(acc[q] * tinv[q], acc[32 + q] * tinv[q]);
-                    if constexpr (ADJ) out[(((int64_t)(b0 + q) * (p + 1) + m) * 2 + par) * P2 + o] = v;
-                    else out[(int64_t)(b0 + q) * nalm + base] = v;
-                }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (abort_) {
-        if (tid == 0) {
-            atomicExch(status, HPX_ERR_TIMEOUT);
-            // copies issued but not seen by the MMA warp, and the last MMAs
-            for (int q = seenA; q < issuedA; ++q)
-                mbar_wait(smem_u32(&fullA[q % NSH]), (uint32_t)((q / NSH) & 1));
-            if (committed > 0)
-                mbar_wait(smem_u32(&accFull[(committed - 1) % NACC]), (uint32_t)(((committed - 1) / NACC) & 1));
-        }
-        __syncthreads();
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(dtmem), "r"(NACC * TN) : "memory");
-}
-
 // Plan time, FP32 tiles -> FP16 form in place (one block of 128 threads per
 // tile, thread r = row r): the row's largest magnitude gives its scale s_r,
 // 1 / s_r goes to rinv, and every chunk (all of it read before any of it is
@@ -928,11 +733,11 @@ int prepare_fused_tc(hpx_plan_s* P) {
     const size_t rb = (size_t)rows * sizeof(float), bb = (size_t)g.B * (g.L + 1) * sizeof(float);
     const size_t pb = bpk_bytes(g.B, g.L, g.P2);
     if (cudaMalloc(&P->tcRinv, rb) != cudaSuccess || cudaMalloc(&P->bscale, bb) != cudaSuccess ||
-        cudaMalloc(&P->adjScale, 2 * bb) != cudaSuccess || cudaMalloc(&P->bpk, pb) != cudaSuccess)
+        cudaMalloc(&P->bpk, pb) != cudaSuccess)
         return -1;
     cudaMemset(P->bpk, 0, pb);   // columns of maps past the batch stay zero
-    P->bytes += (int64_t)(rb + 3 * bb + pb);
-    P->fused_bytes += (int64_t)(rb + 3 * bb + pb);
+    P->bytes += (int64_t)(rb + bb + pb);
+    P->fused_bytes += (int64_t)(rb + bb + pb);
     tc_to_f16_kernel<<<P->fused_ntiles, TM>>>((float*)P->fusedM, P->tcOff, P->fusedTiles, g.P2, g.L, P->tcRinv, 0,
                                               nullptr, nullptr);
     return cudaDeviceSynchronize() == cudaSuccess ? 0 : -1;
@@ -1111,70 +916,6 @@ __global__ void __launch_bounds__(256) pack_alm_kernel(const cplx<float>* __rest
               [&](int i) { return i < n0 ? a[2 * i] : mk<float>(0.f, 0.f); }, threadIdx.x, blockDim.x);
     pack_half(bpk, b, m, 1, L, nch, pow2_scale(mx.y, 13),
               [&](int i) { return i < n1 ? a[2 * i + 1] : mk<float>(0.f, 0.f); }, threadIdx.x, blockDim.x);
-}
-
-// x of the transposed contractions in the packed B layout, each half with its own
-// scale.  One block per (map, order), maps fastest.
-// ADJ: half c = the weighted coefficients of chain c times the row scales of M.
-// !ADJ: half c = the right-hand sides of the chain's parity times the row scales of
-// S_{m,c}^T (rowBase of its first row tile; its tiles store ldr rows in a row).
-template <bool ADJ>
-__global__ void __launch_bounds__(256) pack_x_kernel(const cplx<float>* __restrict__ x, const float* __restrict__ rinv,
-                                                     const int64_t* __restrict__ tileOff,
-                                                     const int* __restrict__ tileFirst,
-                                                     const int64_t* __restrict__ rowBase,
-                                                     unsigned char* __restrict__ bpk, float* __restrict__ xscale, int L,
-                                                     int p, int P2, int64_t nalm, float wpos) {
-    __shared__ float2 red32[32];
-    const int b = blockIdx.x, m = blockIdx.y;
-    const int nch = (P2 + KC - 1) / KC;
-    const cplx<float>* a = ADJ ? x + (int64_t)b * nalm + (int64_t)m * (2 * L + 1 - m) / 2 + m
-                               : x + ((int64_t)b * (p + 1) + m) * 2 * P2;
-    const float w = m == 0 ? 1.f : wpos;
-    const bool drop = m == 0 || m == p;
-    const int len[2] = {ADJ ? chain_len(m, 0, L) : P2, ADJ ? chain_len(m, 1, L) : P2};
-    int64_t r0[2];   // first row scale of the half (row tiles are stored consecutively)
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-        r0[c] = ADJ ? (len[c] > 0 ? tileOff[tileFirst[m * 2 + c]] / (32 * nch) : 0)
-                    : rowBase[(int64_t)(m * 2 + c) * ((P2 + TM - 1) / TM)];
-    auto val = [&](int c, int i) {   // zero past the half
-        if (i >= len[c]) return mk<float>(0.f, 0.f);
-        const float r = rinv[r0[c] + i];
-        if constexpr (ADJ) {
-            const cplx<float> v = a[2 * i + c];
-            return mk<float>(w * v.r * r, drop ? 0.f : w * v.i * r);
-        } else {
-            return scale(a[(((m & 1) + c) & 1) * P2 + i], r);
-        }
-    };
-    float mx[2] = {0.f, 0.f};
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-        for (int i = threadIdx.x; i < len[c]; i += 256) {
-            const cplx<float> v = val(c, i);
-            mx[c] = fmaxf(mx[c], fmaxf(fabsf(v.r), fabsf(v.i)));
-        }
-    const float2 mm = block_max2(make_float2(mx[0], mx[1]), red32);
-    if (threadIdx.x < 2) xscale[((int64_t)b * (L + 1) + m) * 2 + threadIdx.x] = threadIdx.x ? mm.y : mm.x;
-    pack_half(bpk, b, m, 0, L, nch, pow2_scale(mm.x, 13), [&](int i) { return val(0, i); }, threadIdx.x, 256);
-    pack_half(bpk, b, m, 1, L, nch, pow2_scale(mm.y, 13), [&](int i) { return val(1, i); }, threadIdx.x, 256);
-}
-
-void launch_adjoint_tc(const hpx_plan_s* P, const float* alm, cudaStream_t s, float wpos) {
-#if HPX_TC_F16
-    const auto& g = P->g;
-    pack_x_kernel<true><<<dim3(g.B, g.L + 1), 256, 0, s>>>((const cplx<float>*)alm, P->tcRinv, P->tcOff, P->tcFirst,
-                                                           nullptr, P->bpk, P->adjScale, g.L, g.p, g.P2, g.nalm, wpos);
-    const int nt = (g.P2 + TM - 1) / TM;
-    const size_t smem_h = NSH * (TILE_A + TILE_BP);
-    cudaFuncSetAttribute(fused_tc_t_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_h);
-    fused_tc_t_kernel<true><<<dim3((g.L + 1) * 2 * nt, (g.B + 31) / 32), NTW, smem_h, s>>>(
-        (const unsigned char*)P->fusedM, P->tcOff, P->tcFirst, P->bpk, P->adjScale, (cplx<float>*)P->bvec, g.P2, g.p,
-        g.L, g.B, g.nalm, nt, 1.f, P->d_status);
-#else
-    (void)P; (void)alm; (void)s; (void)wpos;
-#endif
 }
 
 int prepare_synth_tc(hpx_plan_s* P) {

@@ -104,7 +104,6 @@ struct hpx_plan_s {
     int* tcFirst = nullptr;        // first tile of (m, c)
     float* tcRinv = nullptr;       // FP16 form: 1 / row scale, per stored row of the tiles
     float* bscale = nullptr;       // FP16 form: [B][L+1] largest magnitude of each b column
-    float* adjScale = nullptr;     // [B][L+1][2] largest magnitude of each packed half of the adjoint's coefficients
     unsigned char* bpk = nullptr;  // FP16 form: b as scaled FP16 pairs in the MMA layout (fp16pair.cuh)
     int* d_status = nullptr;       // device status word (timed-out waits, non-finite inputs)
     int64_t fused_bytes = 0;       // bytes of M
@@ -269,11 +268,9 @@ void launch_finite_check(const void* x, int64_t n, bool fp64, int* status, cudaS
 template <class T>
 int build_fused(hpx_plan_s* P, const double* D64, const cplx<double>* skew64, cudaStream_t s, void* out, int form);
 // the transposed contraction of operators of the layout M (quad: that of
-// fused_quad_kernel) with the weighted coefficients: alm -> bvec (k_fused.cu), and on
-// the tensor cores with M in the tiles of launch_fused_tc (k_fused_tc.cu)
+// fused_quad_kernel) with the weighted coefficients: alm -> bvec (k_fused.cu)
 template <class T>
 void launch_operator_cols(const hpx_plan_s* P, const void* M, bool quad, const T* alm, cudaStream_t s, T wpos, bool dropim);
-void launch_adjoint_tc(const hpx_plan_s* P, const float* alm, cudaStream_t s, float wpos);
 // float offset of element (row r of a tile with rp rows, column k) in the
 // tensor-core layout of M, relative to the tile's first chunk
 __host__ __device__ inline int64_t tc_elem(int rp, int r, int k) {

@@ -22,7 +22,6 @@ void release_operators(hpx_plan_s* P, F release) {
     give(P->tcFirst);
     give(P->tcRinv);
     give(P->bscale);
-    give(P->adjScale);
     give(P->bpk);
     P->bytes -= P->fused_bytes;
     P->fused_bytes = 0;

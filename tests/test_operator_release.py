@@ -17,7 +17,7 @@ static hpx_plan_s* make(bool syn) {
     char* at = nullptr;
     auto fake = [&](auto*& q) { at += 256; q = (std::remove_reference_t<decltype(q)>)at; };
     fake(P->fusedM); fake(P->fusedOff); fake(P->fusedTiles); fake(P->tcOff); fake(P->tcFirst);
-    fake(P->tcRinv); fake(P->bscale); fake(P->adjScale); fake(P->bpk);
+    fake(P->tcRinv); fake(P->bscale); fake(P->bpk);
     if (syn) fake(P->synM);
     P->bytes = 100; P->fused_bytes = 60; P->use_tc = true;
     return P;
@@ -44,5 +44,5 @@ def test_synthesis_keeps_offsets_and_tiles(tmp_path):
     assert r.returncode == 0, r.stderr
     out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.split("\n")
     # without synthesis operators everything goes, with them the offsets and the tiles stay
-    assert out[0] == "9 1 1 0 0 0 1 1 40 1"
-    assert out[1] == "7 0 0 0 1 1 1 1 40 1"
+    assert out[0] == "8 1 1 0 0 0 1 1 40 1"
+    assert out[1] == "6 0 0 0 1 1 1 1 40 1"
