@@ -71,7 +71,7 @@ void free_plan(hpx_plan_s* P) {
     if (P->cap) cudaStreamDestroy(P->cap);
     auto& t = P->t;
     void* ptrs[] = {t.nphi, t.startN, t.startS, t.pow2, t.logn, t.fftL, t.logL, t.shOff, t.chOff,
-                    t.bhOff, t.pw, t.shift, t.chirp, t.bhat, t.twid, t.twc, t.ch4Off, t.bh4Off, t.chirp4, t.bhat4, t.poleN,
+                    t.bhOff, t.pw, t.shift, t.chirp, t.bhat, t.twid, t.twc, t.twx, t.ch4Off, t.bh4Off, t.chirp4, t.bhat4, t.poleN,
                     t.poleS, t.polew, t.rowptr,
                     t.ent, t.entw, t.dec, t.D, t.tstart, t.hwn, t.angOff, t.ang, t.skOff, t.skew, t.skewT, t.nrowptr, t.nent, t.nentw, t.nstart, t.swts, t.hstart, t.hwts, t.Es, t.shifted, t.C, t.cgH, P->Y, P->U, P->bvec,
                     P->fusedM, P->fusedOff, P->fusedTiles, P->tcOff, P->tcFirst, P->tcRinv, P->bscale, P->d_status, P->synM, P->ringList,
@@ -234,6 +234,7 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
     t.ch4Off = up.vec(tb.ch4Off); t.bh4Off = up.vec(tb.bh4Off);
     t.chirp4 = up.real(tb.chirp4, fp64); t.bhat4 = up.real(tb.bhat4, fp64);
     t.twid = up.real(tb.twid, fp64); t.twc = up.real(tb.twc, fp64);
+    t.twx = up.real(tb.twx, fp64);
     t.poleN = up.vec(tb.poleN); t.poleS = up.vec(tb.poleS); t.polew = up.vec(tb.polew);
     t.npole = (int)tb.polew.size();
     {   // ring pairs grouped by transform length (longest first), and from

@@ -69,22 +69,23 @@ __device__ __forceinline__ void first_pass(cplx<T>* a, int tid, LD ld) {
 
 // Pass I of span S = 16^I and radix R over the whole transform, in place, after a
 // barrier; the first group's twiddles are read ahead of it.
-template <class T, int LOGN, int I, int NT, bool INV>
+template <class T, int LOGN, int I, int NT, bool INV, bool EX>
 __device__ __forceinline__ void inner_pass(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid) {
     constexpr int N = 1 << LOGN, R = radix(LOGN, I), S = 1 << (4 * I), NG = N / R, G = (NG + NT - 1) / NT;
-    Twiddles<T> t = load_twiddles_c<T, R, S, INV>(tid & (S - 1), tw);
+    PassTwiddles<T, R, S, INV, EX> t;
+    t.fetch(tid & (S - 1), tw);
     __syncthreads();
 #pragma unroll
     for (int gg = 0; gg < G; ++gg) {
         const int k = tid + gg * NT;
         if (NG % NT != 0 && k >= NG) break;
         const int j = k & (S - 1);
-        if (gg > 0 && NT % S != 0) t = load_twiddles_c<T, R, S, INV>(j, tw);
+        if (gg > 0 && NT % S != 0) t.fetch(j, tw);
         cplx<T>* e = a + slot((k / S) * (S * R) + j);
         cplx<T> x[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r] = e[slot(r * S)];
-        twiddle_by<T, R>(x, t);
+        t.apply(x);
         reg_dft<T, R, INV>(x);
 #pragma unroll
         for (int q = 0; q < R; ++q) e[slot(q * S)] = x[q];
@@ -92,11 +93,11 @@ __device__ __forceinline__ void inner_pass(cplx<T>* a, const cplx<T>* __restrict
 }
 
 // The passes between the first and the last.
-template <class T, int LOGN, int NT, bool INV, int I = 1>
+template <class T, int LOGN, int NT, bool INV, bool EX, int I = 1>
 __device__ __forceinline__ void inner_passes(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid) {
     if constexpr (I < npass(LOGN) - 1) {
-        inner_pass<T, LOGN, I, NT, INV>(a, tw, tid);
-        inner_passes<T, LOGN, NT, INV, I + 1>(a, tw, tid);
+        inner_pass<T, LOGN, I, NT, INV, EX>(a, tw, tid);
+        inner_passes<T, LOGN, NT, INV, EX, I + 1>(a, tw, tid);
     }
 }
 
@@ -107,23 +108,23 @@ __host__ __device__ constexpr int out_radix(int logn, int nt) { return logn == 1
 // Last pass, after a barrier: outputs j + q S (S = N / R, group j = tid + gg NT) to
 // st(index, q, gg, value) for q < LO or q >= HI.  PRE: the first group's twiddles are
 // read ahead of the barrier.
-template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE, class ST>
+template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE, bool EX, class ST>
 __device__ __forceinline__ void last_pass(const cplx<T>* a, const cplx<T>* __restrict__ tw, int tid,
                                           ST st) {
     constexpr int N = 1 << LOGN, R = last_radix(LOGN), S = N / R, G = (S + NT - 1) / NT;
-    Twiddles<T> t;
-    if constexpr (PRE) t = load_twiddles_c<T, R, S, INV>(min(tid, S - 1), tw);
+    PassTwiddles<T, R, S, INV, EX> t;
+    if constexpr (PRE) t.fetch(min(tid, S - 1), tw);
     __syncthreads();
 #pragma unroll
     for (int gg = 0; gg < G; ++gg) {
         const int j = tid + gg * NT;
         if (S % NT != 0 && j >= S) break;
-        if (!PRE || gg > 0) t = load_twiddles_c<T, R, S, INV>(j, tw);
+        if (!PRE || gg > 0) t.fetch(j, tw);
         const cplx<T>* e = a + slot(j);
         cplx<T> x[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) x[r] = e[slot(r * S)];
-        twiddle_by<T, R>(x, t);
+        t.apply(x);
         reg_dft<T, R, INV>(x);
 #pragma unroll
         for (int q = 0; q < R; ++q)
@@ -135,12 +136,13 @@ __device__ __forceinline__ void last_pass(const cplx<T>* a, const cplx<T>* __res
 // elements j + 256 r of thread j < 256, in registers, after a barrier and with another
 // one behind the reads (st may store anywhere in a): outputs j + 256 q, q < LO or
 // q >= HI, to st(index, q, 0, value).
-template <class T, int NT, bool INV, int LO, int HI, class ST>
+template <class T, int NT, bool INV, int LO, int HI, bool EX, class ST>
 __device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>* __restrict__ tw,
                                                  int tid, ST st) {
     static_assert(NT == 256, "one thread per j");
     const cplx<T>* e = a + slot(tid);
-    const Twiddles<T> t = load_twiddles_c<T, 16, 256, INV>(tid, tw);
+    PassTwiddles<T, 16, 256, INV, EX> t;
+    t.fetch(tid, tw);
     __syncthreads();
     cplx<T> x[16], y[16];
 #pragma unroll
@@ -148,15 +150,17 @@ __device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>
 #pragma unroll
     for (int r = 0; r < 16; ++r) y[r] = e[slot(4096 + 256 * r)];
     __syncthreads();
-    twiddle_by<T, 16>(x, t);
+    t.apply(x);
     reg_dft<T, 16, INV>(x);
-    twiddle_by<T, 16>(y, t);
+    t.apply(y);
     reg_dft<T, 16, INV>(y);
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
         const int k = tid + 256 * q;
         cplx<T> z[2] = {x[q], y[q]};
-        twiddle_by<T, 2>(z, load_twiddles_c<T, 2, 4096, INV>(k, tw));
+        PassTwiddles<T, 2, 4096, INV, EX> t2;
+        t2.fetch(k, tw);
+        t2.apply(z);
         reg_dft<T, 2, INV>(z);
         if (q < LO || q >= HI) st(k, q, 0, z[0]);
         if (q + 16 < LO || q + 16 >= HI) st(k + 4096, q + 16, 0, z[1]);
@@ -166,30 +170,31 @@ __device__ __forceinline__ void last_passes_8192(const cplx<T>* a, const cplx<T>
 // The whole transform: ld(i, r) as first_pass, st(index, q, gg, value) as last_pass.
 // st may store to the positions of a (natural order): a thread only produces
 // positions that it alone has read.  Ends without a barrier.
-template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE = true, class LD, class ST>
+// EX: twiddles from the rows of all powers (tw = twx, else twc).
+template <class T, int LOGN, int NT, bool INV, int LO, int HI, bool PRE, bool EX, class LD, class ST>
 __device__ __forceinline__ void transform(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid, LD ld,
                                           ST st) {
     first_pass<T, LOGN, NT, INV, false>(a, tid, ld);
     if constexpr (LOGN == 13 && NT == 256) {
-        inner_pass<T, LOGN, 1, NT, INV>(a, tw, tid);
-        last_passes_8192<T, NT, INV, LO, HI>(a, tw, tid, st);
+        inner_pass<T, LOGN, 1, NT, INV, EX>(a, tw, tid);
+        last_passes_8192<T, NT, INV, LO, HI, EX>(a, tw, tid, st);
     } else {
-        inner_passes<T, LOGN, NT, INV>(a, tw, tid);
-        last_pass<T, LOGN, NT, INV, LO, HI, PRE>(a, tw, tid, st);
+        inner_passes<T, LOGN, NT, INV, EX>(a, tw, tid);
+        last_pass<T, LOGN, NT, INV, LO, HI, PRE, EX>(a, tw, tid, st);
     }
 }
 
 // Cyclic convolution of N = 2^LOGN points by NT >= N/16 threads: input ld(i), zero for
 // i >= N/2 (not read there), transformed kernel ker(i); st(i, value) receives the
 // outputs i < N/2.  The barriers are the block's: side-by-side convolutions run
-// their passes in step.  Ends without one.
-template <class T, int LOGN, int NT, class LD, class KER, class ST>
+// their passes in step.  Ends without one.  EX as transform().
+template <class T, int LOGN, int NT, bool EX, class LD, class KER, class ST>
 __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__ tw, int tid, LD ld,
                                          KER ker, ST st) {
     constexpr int N = 1 << LOGN, R = radix(LOGN, npass(LOGN) - 1), NG = N / 16, D = 16 / R;
     static_assert(NT >= NG, "the turn keeps one group per thread");
     first_pass<T, LOGN, NT, false, true>(a, tid, [&](int i, int) { return ld(i); });
-    inner_passes<T, LOGN, NT, false>(a, tw, tid);
+    inner_passes<T, LOGN, NT, false, EX>(a, tw, tid);
     const bool on = NG == NT || tid < NG;
     __syncthreads();
     cplx<T> y[16];
@@ -200,7 +205,9 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
             cplx<T> x[R];
 #pragma unroll
             for (int q = 0; q < R; ++q) x[q] = e[slot((i + q * D) * NG)];
-            twiddle_by<T, R>(x, load_twiddles_c<T, R, N / R, false>(tid + i * NG, tw));
+            PassTwiddles<T, R, N / R, false, EX> t;
+            t.fetch(tid + i * NG, tw);
+            t.apply(x);
             reg_dft<T, R, false>(x);
 #pragma unroll
             for (int q = 0; q < R; ++q) {
@@ -216,8 +223,8 @@ __device__ __forceinline__ void convolve(cplx<T>* a, const cplx<T>* __restrict__
 #pragma unroll
         for (int r = 0; r < 16; ++r) to[r] = y[r];
     }
-    inner_passes<T, LOGN, NT, true>(a, tw, tid);
-    last_pass<T, LOGN, NT, true, R / 2, R, false>(a, tw, tid, [&](int i, int, int, cplx<T> v) { st(i, v); });
+    inner_passes<T, LOGN, NT, true, EX>(a, tw, tid);
+    last_pass<T, LOGN, NT, true, R / 2, R, false, EX>(a, tw, tid, [&](int i, int, int, cplx<T> v) { st(i, v); });
 }
 
 }  // namespace ip

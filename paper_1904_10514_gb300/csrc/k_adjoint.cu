@@ -451,7 +451,7 @@ template <class T, int LOGQ, int NTQ, class V>
 __device__ __forceinline__ void ring_back_quarters(cplx<T>* buf, T* f, int sN, int sS, int n,
                                                    const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
                                                    const cplx<T>* __restrict__ tw, V in) {
-    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ>(buf, n, ch, bh, tw, in);
+    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ, true>(buf, n, ch, bh, tw, in);
     const int jq = n >> 2;
     for (int q = threadIdx.x; q < jq; q += 4 * NTQ) {
         cplx<T> z[4];
@@ -468,7 +468,7 @@ template <class T, int LOGN, int NT, class V>
 __device__ __forceinline__ void ring_back_whole(cplx<T>* buf, T* f, int sN, int sS, int n,
                                                 const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
                                                 const cplx<T>* __restrict__ tw, V in) {
-    ip::convolve<T, LOGN, NT>(
+    ip::convolve<T, LOGN, NT, true>(
         buf, tw, threadIdx.x, [&](int k) { return k < n ? mul(in(k), ch[k]) : mk<T>(T(0), T(0)); },
         [&](int k) { return bh[k]; },
         [&](int k, cplx<T> v) {
@@ -485,7 +485,7 @@ template <class T, int LOGN, int NT, class V>
 __device__ __forceinline__ void ring_back_plain(cplx<T>* buf, T* f, int sN, int sS, const cplx<T>* __restrict__ tw,
                                                 V in) {
     constexpr int R = ip::out_radix(LOGN, NT);
-    ip::transform<T, LOGN, NT, false, R, R>(
+    ip::transform<T, LOGN, NT, false, R, R, true, true>(
         buf, tw, threadIdx.x, [&](int k, int) { return in(k); },
         [&](int k, int, int, cplx<T> v) {
             f[sN + k] = v.r;
@@ -516,7 +516,9 @@ __global__ void __launch_bounds__(KIND ? 4 * NT : NT, MINB) ring_back_kernel(
 }
 
 // Every transform of at most 2048 points in one launch of 128 threads per ring
-// pair; below 512 points the run-time length FFT.
+// pair; below 512 points radix-2 passes of run-time length, which keep more of the threads
+// busy than radix-16 ones (Nside 16, 1 map: 12.7 us with radix 16, now 10.7, FP64 28.1 and
+// 19.3; Nside 64 and more: the same).
 template <class T, bool SYN>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3) ring_back_short_kernel(
     const cplx<T>* __restrict__ Y, T* __restrict__ maps, const int* __restrict__ nphi_t,
@@ -524,7 +526,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3) ring_back_short_k
     const int* __restrict__ pow2_t, const int* __restrict__ logn_t, const int* __restrict__ logL_t,
     const int64_t* __restrict__ shOff_t, const int64_t* __restrict__ chOff_t, const int64_t* __restrict__ bhOff_t,
     const cplx<T>* __restrict__ shift, const cplx<T>* __restrict__ chirp, const cplx<T>* __restrict__ bhat,
-    const cplx<T>* __restrict__ tw, const cplx<T>* __restrict__ twc, int twlen, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
+    const cplx<T>* __restrict__ tw, const cplx<T>* __restrict__ twx, int twlen, int p, int L, int Q, int64_t npix, const int* __restrict__ ringlist) {
     extern __shared__ unsigned char smem_raw[];
     cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
     const int i = ringlist[blockIdx.y], b = blockIdx.x;
@@ -535,37 +537,37 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 3) ring_back_short_k
     const cplx<T>*ch = chirp + chOff_t[i], *bh = bhat + bhOff_t[i];
     if (pow2_t[i]) {
         switch (logn_t[i]) {
-            case 11: ring_back_plain<T, 11, 128>(buf, f, sN, sS, twc, in); return;
-            case 10: ring_back_plain<T, 10, 128>(buf, f, sN, sS, twc, in); return;
-            case 9: ring_back_plain<T, 9, 128>(buf, f, sN, sS, twc, in); return;
+            case 11: ring_back_plain<T, 11, 128>(buf, f, sN, sS, twx, in); return;
+            case 10: ring_back_plain<T, 10, 128>(buf, f, sN, sS, twx, in); return;
+            case 9: ring_back_plain<T, 9, 128>(buf, f, sN, sS, twx, in); return;
             default: break;
         }
     } else {
         switch (logL_t[i]) {
-            case 11: ring_back_whole<T, 11, 128>(buf, f, sN, sS, n, ch, bh, twc, in); return;
-            case 10: ring_back_whole<T, 10, 128>(buf, f, sN, sS, n, ch, bh, twc, in); return;
-            case 9: ring_back_whole<T, 9, 128>(buf, f, sN, sS, n, ch, bh, twc, in); return;
+            case 11: ring_back_whole<T, 11, 128>(buf, f, sN, sS, n, ch, bh, twx, in); return;
+            case 10: ring_back_whole<T, 10, 128>(buf, f, sN, sS, n, ch, bh, twx, in); return;
+            case 9: ring_back_whole<T, 9, 128>(buf, f, sN, sS, n, ch, bh, twx, in); return;
             default: break;
         }
     }
     const int tid = threadIdx.x;
     if (pow2_t[i]) {
-        for (int k = tid; k < n; k += 128) buf[pad(k)] = in(k);
+        for (int k = tid; k < n; k += 128) buf[k] = in(k);
         __syncthreads();
-        block_fft_pad<T, 16>(buf, logn_t[i], tw, twlen, false);
+        block_fft(buf, n, logn_t[i], tw, twlen, false);
     } else {
         const int N = 1 << logL_t[i];
-        for (int k = tid; k < N; k += 128) buf[pad(k)] = k < n ? mul(in(k), ch[k]) : mk<T>(T(0), T(0));
+        for (int k = tid; k < N; k += 128) buf[k] = k < n ? mul(in(k), ch[k]) : mk<T>(T(0), T(0));
         __syncthreads();
-        block_fft_pad<T, 16>(buf, logL_t[i], tw, twlen, false);
-        for (int k = tid; k < N; k += 128) buf[pad(k)] = mul(buf[pad(k)], bh[k]);
+        block_fft(buf, N, logL_t[i], tw, twlen, false);
+        for (int k = tid; k < N; k += 128) buf[k] = mul(buf[k], bh[k]);
         __syncthreads();
-        block_fft_pad<T, 16>(buf, logL_t[i], tw, twlen, true);
-        for (int k = tid; k < n; k += 128) buf[pad(k)] = mul(buf[pad(k)], ch[k]);
+        block_fft(buf, N, logL_t[i], tw, twlen, true);
+        for (int k = tid; k < n; k += 128) buf[k] = mul(buf[k], ch[k]);
         __syncthreads();
     }
     for (int k = tid; k < n; k += 128) {
-        const cplx<T> v = buf[pad(k)];
+        const cplx<T> v = buf[k];
         f[sN + k] = v.r;
         if (sN != sS) f[sS + k] = -v.i;
     }
@@ -582,11 +584,11 @@ void launch_ring_back(const hpx_plan_s* P, T* maps, cudaStream_t s) {
         constexpr bool F = sizeof(T) == 4;
         if (c.N < kRingCtMin) {
             auto kern = ring_back_short_kernel<T, SYN>;
-            const size_t smem = (size_t)std::max(ip::slots(c.N), c.N + c.N / 16) * sizeof(cplx<T>);
+            const size_t smem = (size_t)ip::slots(c.N) * sizeof(cplx<T>);
             allow_shared(kern);
             kern<<<grid, 128, smem, s>>>(Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.pow2, t.logn, t.logL,
                                          t.shOff, t.chOff, t.bhOff, shift, (const cplx<T>*)t.chirp,
-                                         (const cplx<T>*)t.bhat, tw, (const cplx<T>*)t.twc, g.Lmax, g.p, g.L, g.Q, g.npix,
+                                         (const cplx<T>*)t.bhat, tw, (const cplx<T>*)t.twx, g.Lmax, g.p, g.L, g.Q, g.npix,
                                          list);
             continue;
         }
@@ -595,7 +597,7 @@ void launch_ring_back(const hpx_plan_s* P, T* maps, cudaStream_t s) {
             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             kern<<<grid, threads, smem, s>>>(Y, maps, t.nphi, t.startN, t.startS, t.shifted, t.shOff, t.ch4Off,
                                              t.bh4Off, shift, (const cplx<T>*)t.chirp4, (const cplx<T>*)t.bhat4,
-                                             (const cplx<T>*)t.twc, g.p, g.L, g.Q, g.npix, list);
+                                             (const cplx<T>*)t.twx, g.p, g.L, g.Q, g.npix, list);
         };
         if (c.N == 4096) {
             if (c.blue) run(ring_back_kernel<T, SYN, 10, 64, F ? 4 : 2, 2>, 256);

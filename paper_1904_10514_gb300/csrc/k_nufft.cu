@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(NT, MINB) lat_fft_pair_kernel(
         }
         return v;
     };
-    ip::transform<T, LOGM, NT, false, LO, HI>(
+    ip::transform<T, LOGM, NT, false, LO, HI, true, false>(
         u, tw, tid, [&](int t, int r) { return src[r < 8 || (r == 8 && t == M / 2) ? t : M + M / 2 - t]; },
         [&](int j, int q, int gg, cplx<T> v) {
             // (the ranges of gg and q are known at compile time)

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(NT, MINB) ifft_pair_kernel(const cplx<T>* __re
         if (j >= M - p) return both(M - j, T(-1));
         return mk<T>(T(0), T(0));
     };
-    ip::transform<T, LOGM, NT, true, R, R>(
+    ip::transform<T, LOGM, NT, true, R, R, true, true>(
         buf, tw, tid, ld, [&](int k, int, int, cplx<T> v) { buf[ip::slot(k)] = v; });
     __syncthreads();
     cplx<T>* out0 = U + ((int64_t)b * (L + 1) + m0) * ldu;
@@ -221,7 +221,7 @@ bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
     auto run1 = [&](auto kern, int threads) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
         kern<<<grid1, threads, smem1, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->U, (const T*)t.dec,
-                                           (const cplx<T>*)t.twc, g.p, g.L, g.P2, P->ldu);
+                                           (const cplx<T>*)t.twx, g.p, g.L, g.P2, P->ldu);
     };
     // the shapes of the analysis' grid FFT (k_nufft.cu)
     if (logM == 5) run1(ifft_pair_kernel<T, 5, 32, 1>, 32);

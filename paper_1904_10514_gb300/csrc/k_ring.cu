@@ -84,7 +84,7 @@ __device__ __forceinline__ void ring_plain(cplx<T>* buf, const T* __restrict__ f
                                            int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
     constexpr int N = 1 << LOGN, R = ip::out_radix(LOGN, NT);
     const bool equator = sN == sS;
-    ip::transform<T, LOGN, NT, false, R, R, false>(
+    ip::transform<T, LOGN, NT, false, R, R, false, false>(
         buf, tw, threadIdx.x,
         [&](int k, int) { return mk<T>(f[sN + k], equator ? T(0) : f[sS + k]); },
         [&](int k, int, int, cplx<T> v) { buf[ip::slot(k)] = v; });
@@ -97,7 +97,7 @@ __device__ __forceinline__ void ring_whole(cplx<T>* buf, const T* __restrict__ f
                                            const cplx<T>* __restrict__ ch, const cplx<T>* __restrict__ bh,
                                            const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw,
                                            int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
-    ip::convolve<T, LOGN, NT>(
+    ip::convolve<T, LOGN, NT, false>(
         buf, tw, threadIdx.x,
         [&](int k) { return k < n ? mul(mk<T>(f[sN + k], f[sS + k]), ch[k]) : mk<T>(T(0), T(0)); },
         [&](int k) { return bh[k]; },
@@ -113,7 +113,7 @@ __device__ __forceinline__ void ring_quarters(cplx<T>* buf, const T* __restrict_
                                               const cplx<T>* __restrict__ ph, const cplx<T>* __restrict__ tw,
                                               int p, int L, T ew, bool sh, cplx<T>* rowN, cplx<T>* rowS) {
     constexpr int NT = 4 * NTQ;
-    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ>(
+    const RingQuarters<T> R = quarter_transforms<T, LOGQ, NTQ, false>(
         buf, n, ch, bh, tw, [&](int k) { return mk<T>(f[sN + k], f[sS + k]); });
     R.natural(n, threadIdx.x, NT);
     ring_rows_out<T>([&](int k) { return R.at(k, n); }, n, p, L, ph, sh, ew, rowN, rowS, false, threadIdx.x, NT);

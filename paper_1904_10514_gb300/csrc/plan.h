@@ -19,6 +19,7 @@ struct DevTables {
     int64_t *shOff = nullptr, *chOff = nullptr, *bhOff = nullptr;
     void *shift = nullptr, *chirp = nullptr, *bhat = nullptr, *twid = nullptr;   // cplx<T>
     void* twc = nullptr;                            // cplx<T>: compact twiddle tables (twc_offset, common.cuh)
+    void* twx = nullptr;                            // cplx<T>: twiddle rows of the backward directions (twx_offset)
     int64_t *ch4Off = nullptr, *bh4Off = nullptr;   // quarter-length Bluestein tables (ring form 1)
     void *chirp4 = nullptr, *bhat4 = nullptr;       // cplx<T>
     int *poleN = nullptr, *poleS = nullptr;

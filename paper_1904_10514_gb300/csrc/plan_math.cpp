@@ -257,16 +257,23 @@ std::string build_tables(int nside, int lmax, bool fp64, PlanTables& t) {
         t.twid[2 * k + 1] = std::sin(ang);
     }
 
-    // the same values in rows per span S, radix R and power r = 1, 2, 4, 8 < R (twc_offset)
+    // the same values in rows per span S, radix R and power r: r = 1, 2, 4, 8 below R
+    // (twc_offset), and every r from 1 to R - 1 (twx_offset)
     t.twc.clear();
+    t.twx.clear();
     for (int S : {16, 256, 4096})
         for (int R : {2, 4, 8, 16}) {
             if (S == 4096 && R > 4) continue;
-            for (int r = 1; r < R; r <<= 1)
+            for (int r = 1; r < R; ++r)
                 for (int j = 0; j < S; ++j) {
                     const double ang = -2.0 * kPi * (double)(r * j) / (double)(S * R);
-                    t.twc.push_back(std::cos(ang));
-                    t.twc.push_back(std::sin(ang));
+                    const double c = std::cos(ang), sn = std::sin(ang);
+                    t.twx.push_back(c);
+                    t.twx.push_back(sn);
+                    if ((r & (r - 1)) == 0) {
+                        t.twc.push_back(c);
+                        t.twc.push_back(sn);
+                    }
                 }
         }
 

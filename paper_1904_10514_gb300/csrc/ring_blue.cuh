@@ -56,9 +56,9 @@ struct RingQuarters {
     }
 };
 
-// The quarter transforms of the sequence in(k), k < n, by 4 NTQ threads.  Ends with a
-// barrier.
-template <class T, int LOGQ, int NTQ, class IN>
+// The quarter transforms of the sequence in(k), k < n, by 4 NTQ threads (EX: as
+// ip::transform).  Ends with a barrier.
+template <class T, int LOGQ, int NTQ, bool EX, class IN>
 __device__ __forceinline__ RingQuarters<T> quarter_transforms(cplx<T>* buf, int n, const cplx<T>* __restrict__ ch,
                                                               const cplx<T>* __restrict__ bh,
                                                               const cplx<T>* __restrict__ tw, IN in) {
@@ -66,7 +66,7 @@ __device__ __forceinline__ RingQuarters<T> quarter_transforms(cplx<T>* buf, int 
     const int jq = n >> 2;
     const int s = threadIdx.x / NTQ, ltid = threadIdx.x - s * NTQ;
     cplx<T>* qb = buf + s * QS;
-    ip::convolve<T, LOGQ, NTQ>(
+    ip::convolve<T, LOGQ, NTQ, EX>(
         qb, tw, ltid, [&](int u) { return u < jq ? mul(in(4 * u + s), ch[u]) : mk<T>(T(0), T(0)); },
         [&](int u) { return bh[u]; },
         [&](int u, cplx<T> v) {
