@@ -219,6 +219,7 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
     if (!P) { set_err(HPX_ERR_OOM); return nullptr; }
     P->precision = d->precision;
     cudaGetDevice(&P->device);
+    cudaDeviceGetAttribute(&P->sms, cudaDevAttrMultiProcessorCount, P->device);
     P->stream = nullptr;
     auto& g = P->g;
     g.ns = ns; g.p = tb.p; g.L = L; g.Q = tb.Q; g.npairs = tb.npairs; g.M = tb.M; g.P2 = tb.P2;

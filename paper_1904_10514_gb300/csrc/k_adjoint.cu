@@ -619,18 +619,17 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
         launch_operator_cols<T>(P, P->fusedM, sizeof(T) == 4 && g.B <= 8, alm, s, wpos, true);
     } else {   // (operators stored as FP16 pairs hold 22 bits: the sweeps keep FP32 throughout)
         const int ngroups = (2 * g.B + 31) / 32;
-        const int nitems = (g.L + 1) * 2 * ngroups;
-        const int G = sweep_orders_per_warp(g.B), sitems = (g.L / 2 / G + 1) * 4 * ngroups;
-        (void)G; (void)sitems; (void)nitems;
-        const int blocks = (nitems * 32 + 127) / 128;
         constexpr int KMAX = sizeof(T) == 4 ? 32 : 16;
-        if constexpr (sizeof(T) == 4)   // angle rows and inputs staged ahead of use
+        if constexpr (sizeof(T) == 4) {   // angle rows and inputs staged ahead of use
+            const int G = sweep_orders_per_warp(g.B, g.L, P->sms), sitems = (g.L / 2 / G + 1) * 4 * ngroups;
             rot_adj_staged_kernel<32><<<(sitems * 32 + 63) / 64, 64, 0, s>>>(
                 (const float*)alm, (float*)P->beta, t.skOff, (const cplx<float>*)t.skewT, t.nq, g.P2, g.L, g.p, g.B,
                 g.nalm, G, ngroups, sitems, (float)wpos, true);
-        else
+        } else {
+            const int nitems = (g.L + 1) * 2 * ngroups, blocks = (nitems * 32 + 127) / 128;
             rot_adj_kernel<T, KMAX><<<blocks, 128, 0, s>>>(alm, (T*)P->beta, t.skOff, (const cplx<T>*)t.skewT, t.nq,
                                                            g.P2, g.L, g.p, g.B, g.nalm, ngroups, nitems, wpos, true);
+        }
         const int nmp = g.L / 2 + 1;
         dim3 grid((nmp * g.B + AC - 1) / AC, (g.P2 + AK - 1) / AK, 4);
         if (sizeof(T) == 8 || !launch_dense_adj_big(P, s, t.D))
@@ -679,18 +678,17 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
         launch_operator_cols<T>(P, P->synM, false, alm, s, T(1), false);   // the sweeps and Es composed per (m, c)
     } else {
         const int ngroups = (2 * g.B + 31) / 32;
-        const int nitems = (g.L + 1) * 2 * ngroups;
-        const int G = sweep_orders_per_warp(g.B), sitems = (g.L / 2 / G + 1) * 4 * ngroups;
-        (void)G; (void)sitems; (void)nitems;
-        const int blocks = (nitems * 32 + 127) / 128;
         constexpr int KMAX = sizeof(T) == 4 ? 32 : 16;
-        if constexpr (sizeof(T) == 4)
+        if constexpr (sizeof(T) == 4) {
+            const int G = sweep_orders_per_warp(g.B, g.L, P->sms), sitems = (g.L / 2 / G + 1) * 4 * ngroups;
             rot_adj_staged_kernel<32><<<(sitems * 32 + 63) / 64, 64, 0, s>>>(
                 (const float*)alm, (float*)P->beta, t.skOff, (const cplx<float>*)t.skewT, t.nq, g.P2, g.L, g.p, g.B,
                 g.nalm, G, ngroups, sitems, 1.f, false);
-        else
+        } else {
+            const int nitems = (g.L + 1) * 2 * ngroups, blocks = (nitems * 32 + 127) / 128;
             rot_adj_kernel<T, KMAX><<<blocks, 128, 0, s>>>(alm, (T*)P->beta, t.skOff, (const cplx<T>*)t.skewT, t.nq,
                                                            g.P2, g.L, g.p, g.B, g.nalm, ngroups, nitems, T(1), false);
+        }
         const int nmp = g.L / 2 + 1;
         dim3 grid((nmp * g.B + AC - 1) / AC, (g.P2 + AK - 1) / AK, 4);
         if (sizeof(T) == 8 || !launch_dense_adj_big(P, s, t.Es))

@@ -313,7 +313,7 @@ void launch_rot(const hpx_plan_s* P, T* alm, cudaStream_t s) {
             // complex column per lane with 32 stages per pass (168 registers, 12 warps
             // per SM) or 16 (twice the passes over the chains, 20 warps per SM)
             if (P->rotForm == 2) {   // one real column per lane
-                const int G = sweep_orders_per_warp(g.B);
+                const int G = sweep_orders_per_warp(g.B, g.L, P->sms);
                 const int rgroups = (2 * g.B + 31) / 32, ritems = (g.L / 2 / G + 1) * 4 * rgroups;
                 rot_staged_real_kernel<32><<<(ritems * 32 + threads - 1) / threads, threads, 0, s>>>(
                     (cplx<float>*)P->beta, (cplx<float>*)alm, P->t.skOff, (const cplx<float>*)P->t.skew, P->t.nq,

@@ -64,6 +64,7 @@ struct hpx_plan_s {
     hpx::Geometry g;
     int precision;
     int device;
+    int sms = 152;          // multiprocessors of the device
     cudaStream_t stream;
     hpx::DevTables t;
     // workspace

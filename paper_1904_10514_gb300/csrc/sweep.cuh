@@ -70,12 +70,19 @@ __device__ __forceinline__ float rot_lo(float c, float s, float carry, float x) 
     return __fmaf_rn(c, x, -__fmul_rn(s, carry));
 }
 
-// Orders that a warp of real lanes sweeps together (k_rot.cu): as many as fit 32
-// lanes with 2B real columns each, rounded up to a power of two.
-inline int sweep_orders_per_warp(int B) {
-    int w = 1;
+// Orders that a warp of real lanes sweeps together (k_rot.cu): at most as many as fit 32
+// lanes with 2B real columns each, rounded up to a power of two, and only as many as
+// leave 3 warps per multiprocessor: below that the sweeps wait for the longest order,
+// and the orders a warp takes beyond the first add their own passes of one sweep to it.
+// Transposed sweeps of one map in us, 1 / 2 / 4 / 8 / 16 orders per warp: Nside 64 52 / 52
+// / 55 / 75 / 149, 256 389 / 303 / 306 / 391 / 771, 512 1930 / 1315 / 1069 / 1337 / 2239,
+// 1024 11070 / 7160 / 5000 / 4880 / 7490 (the rule takes 1, 2, 4 and 8).
+inline int sweep_orders_per_warp(int B, int L, int sms) {
+    int w = 1, G = 1;
     while (w < 2 * B) w <<= 1;
-    return w < 32 ? 32 / w : 1;
+    const int64_t warps = (int64_t)2 * (L + 1) * ((2 * B + 31) / 32);
+    while (2 * G * w <= 32 && warps >= (int64_t)2 * G * 3 * sms) G <<= 1;
+    return G;
 }
 
 template <int RB>

@@ -1,0 +1,45 @@
+"""Both sides of the rules that choose a form by the size of the work: the same maps in a
+batch of one and in batches that take the other form."""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+# two FP32 evaluations with relative errors up to 5e-7 each; FP64 as the adjoint's gate
+TOL = {"fp32": 1e-6, "fp64": 2e-12}
+
+
+def _coefficients(L, B, prec):
+    rng = np.random.default_rng(L + B)
+    n = (L + 1) * (L + 2) // 2
+    a = rng.standard_normal((B, n)) + 1j * rng.standard_normal((B, n))
+    return torch.as_tensor(a, device="cuda").to(torch.complex64 if prec == "fp32" else torch.complex128)
+
+
+@pytest.mark.parametrize("nside,lmax,B", [(256, 512, 8), (256, 511, 4), (512, 1024, 4), (512, 900, 8)])
+def test_orders_per_warp(nside, lmax, B):
+    """Sweeps of 2 and 4 orders per warp (one in the small plans of the other tests): the analysis has
+    the bits of the complex-lane form, the transposed sweeps agree with those of another batch."""
+    import paper_1904_10514_gb300 as hp
+    x = torch.as_tensor(np.random.default_rng(B).standard_normal((B, 12 * nside * nside)), dtype=torch.float32,
+                        device="cuda")
+    a = _coefficients(lmax, 32, "fp32")
+    plan = hp.Plan(nside, lmax, B, "fp32", sweeps=True, synthesis=True)
+    t = list(plan.tuning)
+    fwd = []
+    for form in (0, 2):
+        t[2] = form
+        plan.tuning = tuple(t)
+        fwd.append(plan.analyze(x).clone())
+    assert torch.equal(*fwd)
+    many, adj = plan.sh_synthesis(a[:B]).clone(), plan.synthesize(a[:B]).clone()
+    torch.cuda.synchronize()
+    plan.close()
+    plan = hp.Plan(nside, lmax, 32, "fp32", sweeps=True, synthesis=True)   # one order per warp
+    for u, v in ((many, plan.sh_synthesis(a)), (adj, plan.synthesize(a))):
+        d = torch.linalg.vector_norm(u - v[:B]) / torch.linalg.vector_norm(u)
+        assert float(d) <= TOL["fp32"]
+    torch.cuda.synchronize()
+    plan.close()
