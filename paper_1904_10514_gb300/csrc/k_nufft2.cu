@@ -206,7 +206,8 @@ __global__ void __launch_bounds__(256, 2) interp_rb_kernel(const cplx<float>* __
     }
 }
 
-// Returns false at nside 2 (16 grid points); the caller then runs nufft_adj_kernel.
+// Returns false at nside 2 (16 grid points) and for small batches of small grids; the
+// caller then runs nufft_adj_kernel.
 template <class T>
 bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
     const auto& g = P->g;
@@ -215,7 +216,12 @@ bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
     constexpr bool F = sizeof(T) == 4;
     int logM = 0;
     while ((1 << logM) < g.M) ++logM;
-    if (logM < 5) return false;
+    // small grids in few columns: one block per column does all of it (nufft_adj_kernel)
+    // in a wave or so, in 8 to 10 us where the two kernels here, each with its own
+    // latency, take 13 to 20.  FP32: up to 512 points and 600 columns of them (Nside 64,
+    // 1 map: 10 against 20 us; 32 maps, lmax 33: 23 against 19); FP64, bound by its pipe:
+    // up to a fourth of that (Nside 64, 1 map: 25 against 44; Nside 32, 8 maps: 42 / 40)
+    if (logM < 5 || (g.M <= 512 && (int64_t)g.B * (g.L + 1) * g.M <= (F ? 4 : 1) * (int64_t)P->sms * 512)) return false;
     const size_t smem1 = (size_t)ip::slots(g.M) * sizeof(cplx<T>);
     dim3 grid1((g.L + 2) / 2, g.B);
     auto run1 = [&](auto kern, int threads) {

@@ -43,3 +43,21 @@ def test_orders_per_warp(nside, lmax, B):
         assert float(d) <= TOL["fp32"]
     torch.cuda.synchronize()
     plan.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("nside,lmax,B", [(4, 7, 1300), (8, 16, 310), (16, 32, 80), (32, 64, 20), (64, 33, 19),
+                                          (64, 128, 5)])
+def test_backward_grid(nside, lmax, B, prec):
+    """One block per column for small grids in few columns, grid FFT and interpolation else."""
+    import paper_1904_10514_gb300 as hp
+    a = _coefficients(lmax, B, prec)
+    out = []
+    for b in (B, 1):
+        plan = hp.Plan(nside, lmax, b, prec, sweeps=True, synthesis=True)
+        out.append((plan.sh_synthesis(a[:b]).clone(), plan.synthesize(a[:b]).clone()))
+        torch.cuda.synchronize()
+        plan.close()
+    for many, one in zip(*out):
+        d = torch.linalg.vector_norm(many[0] - one[0]) / torch.linalg.vector_norm(one[0])
+        assert float(d) <= TOL[prec]
