@@ -418,12 +418,17 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
     const auto& g = P->g;
     const auto& t = P->t;
     auto launch = [&](int N, int nrings, const int* list) {
-        // E elements per thread: blocks of N / E threads (at least one warp)
-        const bool big = N > 16 * kRingThreads, brief = N <= 16 * kRingShortThreads;
-        const int threads = brief ? kRingShortThreads : std::max(32, N / (big ? 32 : 16));
-        const size_t smem = (size_t)(brief ? ring_short_slots(N) : N + N / 16) * sizeof(cplx<T>);
-        auto kern = brief ? ring_fft_kernel<T, 16, kRingShortThreads>
-                          : big ? ring_fft_kernel<T, 32, 0> : ring_fft_kernel<T, 16, 0>;
+        // 128 threads per ring pair, or one warp of 16 elements per thread and pass for
+        // transforms of at most 512 points: the same roundings, fewer idle threads, more
+        // ring pairs per SM.  The warps win where the ring pairs are more than twice what
+        // fits at once (Nside 64, 32 maps: 20 against 28 us FP32, 200 against 234 FP64; 4
+        // maps FP64: 8 us slower, 8 maps: 4 us faster; FP32 8 maps: 2 us slower, 16 maps:
+        // 2 us faster), and at Nside 2 and 4 (6.9 against 8.1 us)
+        const int fit = P->sms * (sizeof(T) == 4 ? 6 : 3);
+        const bool warps = N <= 32 || (N <= 512 && (int64_t)g.B * nrings > 2 * fit);
+        const int threads = warps ? 32 : kRingShortThreads;
+        const size_t smem = (size_t)(warps ? N + N / 16 : ring_short_slots(N)) * sizeof(cplx<T>);
+        auto kern = warps ? ring_fft_kernel<T, 16, 0> : ring_fft_kernel<T, 16, kRingShortThreads>;
         allow_shared(kern);
         dim3 grid(g.B, nrings);
         kern<<<grid, threads, smem, s>>>(

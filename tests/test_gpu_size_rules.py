@@ -61,3 +61,21 @@ def test_backward_grid(nside, lmax, B, prec):
     for many, one in zip(*out):
         d = torch.linalg.vector_norm(many[0] - one[0]) / torch.linalg.vector_norm(one[0])
         assert float(d) <= TOL[prec]
+
+
+@pytest.mark.parametrize("prec,nside,lmax,B", [("fp32", 4, 8, 2), ("fp32", 16, 32, 70), ("fp32", 64, 33, 17),
+                                               ("fp64", 4, 8, 2), ("fp64", 16, 9, 33), ("fp64", 64, 33, 9)])
+def test_short_rings(prec, nside, lmax, B):
+    """One warp per ring pair in large batches of short rings (and at Nside 4), four in the plan
+    of one map: the same bits."""
+    import paper_1904_10514_gb300 as hp
+    x = torch.as_tensor(np.random.default_rng(nside).standard_normal((B, 12 * nside * nside)), device="cuda")
+    x = x.to(torch.float32 if prec == "fp32" else torch.float64)
+    # (FP32 sweeps and FP64 operators sum in one order for every batch)
+    out = []
+    for b in (B, 1):
+        plan = hp.Plan(nside, lmax, b, prec, sweeps=prec == "fp32", simt=True)
+        out.append(plan.analyze(x[:b].contiguous()).clone())
+        torch.cuda.synchronize()
+        plan.close()
+    assert torch.equal(out[0][0], out[1][0])
