@@ -369,7 +369,7 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
                                    : hpx::build_fused<float>(P, D64, sk64, nullptr, P->fusedM, form))
                            : -1;
             if (rc == 0 && P->use_tc) rc = hpx::prepare_fused_tc(P);
-            // synthesis operators R_{m,c} Es (row-major), when asked for and room allows
+            // synthesis operators R_{m,c} Es, when asked for and room allows
             const size_t sBytes = (size_t)off.back() * P->fused_ldm * (fp64 ? 8 : 4);
             cudaMemGetInfo(&freeB, &totalB);
             if (rc == 0 && (d->flags & HPX_FLAG_SYNTHESIS) && sBytes + ((size_t)1 << 30) < freeB &&
@@ -377,8 +377,15 @@ hpx_plan_s* hpx_plan_ex(const hpx_plan_desc* d) {
                 P->bytes += (int64_t)sBytes;
                 cudaMemset(P->synM, 0, sBytes);
                 double* Es64 = fp64 ? (double*)t.Es : up.vec(EsHost);
-                rc = up.ok ? (fp64 ? hpx::build_fused<double>(P, Es64, sk64, nullptr, P->synM, 0)
-                                   : hpx::build_fused<float>(P, Es64, sk64, nullptr, P->synM, 0))
+                // 5 to 8 FP32 maps: in groups of 32 rows, which the transposed synthesis
+                // streams faster (Nside 512, 8 maps: 1274 us per call by rows, 758 in
+                // groups; Nside 256 255 and 194), the synthesis as fast; by rows where the
+                // chains leave the groups' blocks half empty (Nside 256, lmax 70: 62 and
+                // 76) and for fewer maps (1 map, Nside 512, synthesis: 334 and 396)
+                P->synQuad = !fp64 && g.B > 4 && g.B <= 8 && L >= 128;
+                const int sform = P->synQuad ? 2 : 0;
+                rc = up.ok ? (fp64 ? hpx::build_fused<double>(P, Es64, sk64, nullptr, P->synM, sform)
+                                   : hpx::build_fused<float>(P, Es64, sk64, nullptr, P->synM, sform))
                            : -1;
                 if (!fp64 && Es64) { cudaFree(Es64); P->bytes -= (int64_t)(EsHost.size() * 8); }
                 // FP32 plans on the tensor cores apply them there too

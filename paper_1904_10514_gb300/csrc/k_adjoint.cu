@@ -675,7 +675,8 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
     if (sizeof(T) == 4 && P->synT) {
         launch_synth_tc(P, (const float*)alm, s);   // the same operators on the tensor cores
     } else if (P->synM) {
-        launch_operator_cols<T>(P, P->synM, false, alm, s, T(1), false);   // the sweeps and Es composed per (m, c)
+        // the sweeps and Es composed per (m, c)
+        launch_operator_cols<T>(P, P->synM, P->synQuad, alm, s, T(1), false);
     } else {
         const int ngroups = (2 * g.B + 31) / 32;
         constexpr int KMAX = sizeof(T) == 4 ? 32 : 16;

@@ -208,7 +208,9 @@ __global__ void __launch_bounds__(TR* TC) fused_apply_kernel(const T* __restrict
 // warps (128 rows) with eight loads in flight per lane.  Before, row-major M went
 // through shared memory in tiles of 512 rows x 2 maps with 64 threads: analysis and
 // C_l of one map at Nside 256 took 297 us, now 98; five at Nside 128 79.9, now 64.9.
-template <int NB>
+// BLOCKED (the transposed synthesis of 5 to 8 maps, launch_fused): each 32 k are summed
+// by themselves and then added, as few roundings as the lanes' sums of fused_rows_kernel.
+template <int NB, bool BLOCKED = false>
 __global__ void __launch_bounds__(128) fused_quad_kernel(const float* __restrict__ M, const int64_t* __restrict__ moff,
                                                          const int* __restrict__ tiles,
                                                          const cplx<float>* __restrict__ bvec,
@@ -252,22 +254,35 @@ __global__ void __launch_bounds__(128) fused_quad_kernel(const float* __restrict
     };
     const int n4 = ldm >> 2;
     int k4 = 0;
+    float sum[BLOCKED ? NC : 1];
+    if constexpr (BLOCKED)
+#pragma unroll
+        for (int q = 0; q < NC; ++q) sum[q] = 0.f;
     for (; k4 + 8 <= n4; k4 += 8) {
         float4 v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) v[u] = __ldg(A + (int64_t)(k4 + u) * cnt);
 #pragma unroll
         for (int u = 0; u < 8; ++u) step(v[u], k4 + u);
+        if constexpr (BLOCKED)
+#pragma unroll
+            for (int q = 0; q < NC; ++q) {
+                sum[q] += acc[q];
+                acc[q] = 0.f;
+            }
     }
     for (; k4 < n4; ++k4) step(__ldg(A + (int64_t)k4 * cnt), k4);
+    if constexpr (BLOCKED)
+#pragma unroll
+        for (int q = 0; q < NC; ++q) acc[q] += sum[q];
     const int64_t at = (int64_t)m * (2 * L + 1 - m) / 2 + m + c + 2 * (int64_t)(g0 + lane);
 #pragma unroll
     for (int q = 0; q < NB; ++q)
         if (b0 + q < B) alm[(int64_t)(b0 + q) * nalm + at] = mk<float>(acc[2 * q], acc[2 * q + 1]);
 }
 
-// FP64 batches (and the FP32 equal-weight analysis of at most 8 maps, on row-major
-// operators): a matrix-vector form.  A block takes 64 rows of one (m, c) and NB
+// FP64 batches (and the FP32 equal-weight analysis of small batches whose synthesis
+// operators are row-major): a matrix-vector form.  A block takes 64 rows of one (m, c) and NB
 // maps; a warp takes R rows at a time, its lanes split the k of a row (one 16-byte
 // load per lane and row: 512 contiguous bytes of the operator per warp load, R loads
 // in flight per lane), b sits in shared memory as 2 NB real columns, and the R x 2 NB
@@ -576,10 +591,10 @@ template void launch_operator_cols<double>(const hpx_plan_s*, const void*, bool,
 int fused_tile_rows(bool fp64) { return fp64 ? kFusedRows : 128; }
 
 template <class T>
-void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Mrows) {
+void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Msyn) {
     const auto& g = P->g;
     const int ldm = P->fused_ldm;
-    const T* M = (const T*)(Mrows ? Mrows : P->fusedM);
+    const T* M = (const T*)(Msyn ? Msyn : P->fusedM);
     if constexpr (sizeof(T) == 4) {
         if (g.B > 8) {
             dim3 grid(P->fused_ntiles, (g.B + 31) / 32);
@@ -590,14 +605,15 @@ void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Mrows
         }
     }
     if constexpr (sizeof(T) == 4) {
-        if (!Mrows) {
+        if (!Msyn || P->synQuad) {
             auto run = [&](auto kern, int NB) {   // each operator read once: all maps in one block
                 const size_t smem = (size_t)2 * NB * ldm * sizeof(float);
                 allow_shared(kern);
                 kern<<<P->fused_ntiles, 128, smem, s>>>(M, P->fusedOff, P->fusedTiles, (const cplx<float>*)P->bvec,
                                                         (cplx<float>*)alm, g.P2, ldm, g.p, g.L, g.B, g.nalm);
             };
-            if (g.B == 1) run(fused_quad_kernel<1>, 1);
+            if (Msyn) run(fused_quad_kernel<8, true>, 8);
+            else if (g.B == 1) run(fused_quad_kernel<1>, 1);
             else if (g.B == 2) run(fused_quad_kernel<2>, 2);
             else if (g.B <= 4) run(fused_quad_kernel<4>, 4);
             else run(fused_quad_kernel<8>, 8);

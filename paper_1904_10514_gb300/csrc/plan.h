@@ -109,7 +109,8 @@ struct hpx_plan_s {
     unsigned char* bpk = nullptr;  // FP16 form: b as scaled FP16 pairs in the MMA layout (fp16pair.cuh)
     int* d_status = nullptr;       // device status word (timed-out waits, non-finite inputs)
     int64_t fused_bytes = 0;       // bytes of M
-    void* synM = nullptr;          // T, n_alm x ldm row-major: synthesis operators R_{m,c} Es (HPX_FLAG_SYNTHESIS)
+    void* synM = nullptr;          // T, n_alm x ldm: synthesis operators R_{m,c} Es (HPX_FLAG_SYNTHESIS), row-major, or
+    bool synQuad = false;          // in the groups of fused_quad_kernel
     // FP32 plans on the tensor cores: the synthesis operators transposed into
     // tiles of 128 latitude modes x the chain's degrees (FP16 pairs, K-chunks of
     // 32), their row scales, the tile table (m, c, k0), each tile's K-chunk count,
@@ -244,9 +245,9 @@ bool launch_dense_adj_big(const hpx_plan_s* P, cudaStream_t s, const void* Dmat)
 template <class T> void launch_cg(const hpx_plan_s* P, cudaStream_t s);
 template <class T> void launch_rot(const hpx_plan_s* P, T* alm, cudaStream_t s);
 int fused_tile_rows(bool fp64);
-// per-order operators on the FP32 pipes; Mrows: row-major operators of the
-// layout of fusedM's SIMT form (NULL = fusedM), e.g. the synthesis operators synM
-template <class T> void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Mrows = nullptr);
+// per-order operators on the FP32 or FP64 pipes; Msyn: the synthesis operators synM
+// (NULL: fusedM)
+template <class T> void launch_fused(const hpx_plan_s* P, T* alm, cudaStream_t s, const void* Msyn = nullptr);
 // S^T of the spherical-harmonic synthesis times `scale` (maps -> alm) and the
 // Jacobi-refined equal-weight analysis of the HEALPix software (k_healpix.cu)
 template <class T> void launch_sh_adjoint(const hpx_plan_s* P, const T* maps, T* alm, cudaStream_t s, T scale);

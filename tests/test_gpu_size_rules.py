@@ -79,3 +79,20 @@ def test_short_rings(prec, nside, lmax, B):
         torch.cuda.synchronize()
         plan.close()
     assert torch.equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("nside,lmax,B", [(64, 128, 5), (128, 255, 8), (256, 300, 7), (64, 127, 8)])
+def test_synthesis_operators_of_5_to_8_maps(nside, lmax, B):
+    """Stored in groups of rows from lmax 128 on, by rows below: both directions against FP64."""
+    import paper_1904_10514_gb300 as hp
+    a = _coefficients(lmax, B, "fp64")
+    out = {}
+    for prec in ("fp32", "fp64"):
+        plan = hp.Plan(nside, lmax, B, prec, synthesis=True)
+        f = plan.sh_synthesis(a.to(plan.cdtype)).clone()
+        x = f if prec == "fp32" else out["fp32"][0].double()
+        out[prec] = (f, plan.sh_synthesis_adjoint(x).clone())
+        torch.cuda.synchronize()
+        plan.close()
+    for u, v in zip(out["fp32"], out["fp64"]):
+        assert float(torch.linalg.vector_norm(u - v) / torch.linalg.vector_norm(v)) <= 5e-7
