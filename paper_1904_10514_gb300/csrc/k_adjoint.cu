@@ -640,12 +640,13 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
         int logM = 0;
         while ((1 << logM) < g.M) ++logM;
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
-        allow_shared(nufft_adj_kernel<T>);
         dim3 grid(g.L + 1, g.B);
-        if (!launch_nufft2<T>(P, s))
+        if (!launch_nufft2<T>(P, s)) {
+            allow_shared(nufft_adj_kernel<T>);
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,
                                                     (const T*)t.nentw, (const T*)t.dec, (const cplx<T>*)t.twid,
                                                     g.Lmax, g.M, logM, g.p, g.Q, g.P2);
+        }
     }
     {
         launch_ring_back<T, false>(P, maps, s);
@@ -701,12 +702,13 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
         int logM = 0;
         while ((1 << logM) < g.M) ++logM;
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
-        allow_shared(nufft_adj_kernel<T>);
         dim3 grid(g.L + 1, g.B);
-        if (!launch_nufft2<T>(P, s))
+        if (!launch_nufft2<T>(P, s)) {
+            allow_shared(nufft_adj_kernel<T>);
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,
                                                         (const T*)t.nentw, (const T*)t.dec, (const cplx<T>*)t.twid,
                                                         g.Lmax, g.M, logM, g.p, g.Q, g.P2);
+        }
     }
     if (ev) cudaEventRecord(ev[2], s);
     launch_ring_back<T, true>(P, maps, s);

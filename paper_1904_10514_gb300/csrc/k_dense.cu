@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(256, 2) dense_big_kernel(const float* __restri
 static bool dense_big(const hpx_plan_s* P, dim3& grid) {
     const auto& g = P->g;
     grid = dim3(((g.L / 2 + 1) * g.B + DC - 1) / DC, (g.P2 + DR - 1) / DR, 4);
-    return (int64_t)grid.x * grid.y * 4 >= 2 * 152;
+    return (int64_t)grid.x * grid.y * 4 >= 2 * P->sms;
 }
 
 bool launch_dense_adj_big(const hpx_plan_s* P, cudaStream_t s, const void* Dmat) {

@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(TR* TC) fused_apply_kernel(const T* __restrict
 // bound is the operator's stream, 4 (nside + 1) n_alm bytes per call: blocks of four
 // warps (128 rows) with eight loads in flight per lane.  Before, row-major M went
 // through shared memory in tiles of 512 rows x 2 maps with 64 threads: analysis and
-// C_l of one map at Nside 256 took 297 us, now 98; five at Nside 128 79.9, now 64.9.
+// C_l of one map at Nside 256 took 297 us, now 92; five at Nside 128 79.9, now 64.5.
 // BLOCKED (the transposed synthesis of 5 to 8 maps, launch_fused): each 32 k are summed
 // by themselves and then added, as few roundings as the lanes' sums of fused_rows_kernel.
 template <int NB, bool BLOCKED = false>
@@ -292,8 +292,8 @@ __global__ void __launch_bounds__(128) fused_quad_kernel(const float* __restrict
 // lane distance 16, 8, 4, 2, 1, then the last term k = nside.
 // The bound is the FP64 pipe (2 FMA per SM and clock on this GPU), so no lane
 // computes for a map or row that is not there beyond the tail of a group.  One map,
-// Nside 512: analysis and C_l 5.11 -> 1.87 ms (this kernel about 4.2 -> 1.0, FMA floor
-// 0.87); Nside 16: 107 -> 80 us.
+// Nside 512: analysis and C_l 5.11 -> 1.84 ms (this kernel about 4.2 -> 1.0, FMA floor
+// 0.87); Nside 16: 107 -> 78 us.
 // Tiles of 512 rows x 2 maps, always computed in full, before.
 template <class T, int NB, int R>
 __global__ void __launch_bounds__(256) fused_rows_kernel(const T* __restrict__ M, const int64_t* __restrict__ moff,

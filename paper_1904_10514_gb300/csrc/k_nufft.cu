@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(32) lat_fft_small_kernel(const cplx<T>* __rest
 // there and forms both right-hand sides.  PW: pw[j] = (a, b), 1 / (1 - rho e^{-2 pi i j
 // / M}) = a - i b (prewhiten_kernel).
 // What bounds it is the shared-memory and L1 pipe (64% at 8192 points) at 40% issue, not
-// DRAM (25%).  32 maps: Nside 1024 2.10 -> 1.52 ms, of which the packing of b 0.43;
+// DRAM (25%).  32 maps: Nside 1024 2.10 -> 1.32 ms, of which the packing of b 0.43;
 // Nside 512 x 64 maps 0.88 -> 0.61 ms (before: four loads and the combination of two
 // half grids per element, two barriers per pass, sine, cosine and quotient per mode).
 template <class T, int LOGM, int NT, int MINB, bool PW>

@@ -300,8 +300,9 @@ __device__ __forceinline__ void ring_pair(
                      rowS, equator, tid, nt);
 }
 
-// Every ring pair of transforms up to 2048 points (NT = 128 threads), one launch:
-// alone, each of the short classes' launches is bound by its latency.
+// Every ring pair of transforms up to 2048 points (NT = 128 threads), or up to 512 points
+// with a warp per ring pair (NT = 0), one launch: alone, each of the short classes'
+// launches is bound by its latency.
 template <class T, int E, int NT>
 __global__ void __launch_bounds__(NT > 0 ? NT : kRingThreads, NT > 0 ? (sizeof(T) == 4 ? 6 : 3) : (E <= 16 ? 2 : 1)) ring_fft_kernel(
     const T* __restrict__ maps, cplx<T>* __restrict__ Y, const int* __restrict__ nphi_t,

@@ -28,7 +28,7 @@ struct PlanTables {
     std::vector<double> chirp4;  // complex: e^{-i pi u^2 / j}, u < j
     std::vector<double> bhat4;   // complex: FFT_{L/4} of the conjugate chirp, divided by L / 4
     int Lmax = 0;                // twiddle table covers FFT lengths up to Lmax
-    std::vector<double> twid;    // complex: e^{-2 pi i k / Lmax}, k < Lmax/2
+    std::vector<double> twid;    // complex: e^{-2 pi i k / Lmax}, k < Lmax
     std::vector<double> twc, twx;   // complex: twiddle rows of the compile-time FFTs (twc_offset, twx_offset)
     int smem_ring = 0;           // largest in-CTA FFT length of step 1
 
