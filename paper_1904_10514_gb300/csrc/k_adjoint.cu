@@ -641,7 +641,7 @@ void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, 
         while ((1 << logM) < g.M) ++logM;
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
         dim3 grid(g.L + 1, g.B);
-        if (!launch_nufft2<T>(P, s)) {
+        if (!launch_nufft2<T>(P, s, T(1))) {
             allow_shared(nufft_adj_kernel<T>);
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,
                                                     (const T*)t.nentw, (const T*)t.dec, (const cplx<T>*)t.twid,
@@ -703,7 +703,7 @@ void launch_sh_synthesis(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_
         while ((1 << logM) < g.M) ++logM;
         const size_t smem = (size_t)g.M * sizeof(cplx<T>);
         dim3 grid(g.L + 1, g.B);
-        if (!launch_nufft2<T>(P, s)) {
+        if (!launch_nufft2<T>(P, s, T(0.5))) {
             allow_shared(nufft_adj_kernel<T>);
             nufft_adj_kernel<T><<<grid, 512, smem, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->Y, t.nrowptr, t.nent,
                                                         (const T*)t.nentw, (const T*)t.dec, (const cplx<T>*)t.twid,

@@ -22,6 +22,9 @@
 //       is symmetric and the odd order's antisymmetric, so one inverse FFT of
 //       the sum of the two spectra gives both: v_m = (z(t) + z(M - t))/2,
 //       v_{m+1} = (z(t) - z(M - t))/2.  Output: U[b][m][t], t = 0..M/2.
+//       The FFT's rounding errors are those of the sum and fall on both orders alike, so
+//       the even order enters times `even`, a power of two (1/2 in the synthesis, whose
+//       even orders carry the rings' weight 2; halfInv = 1 / (2 even) takes it out).
 //   interp_rb_kernel  the transpose of the half-grid spreading: node r takes the
 //       grid points tstart[r] .. tstart[r] + E - 1 with the spreading weights of
 //       (grid point, node) (table hwn, one per parity of m).  A block takes 32
@@ -37,7 +40,7 @@ namespace hpx {
 template <class T, int LOGM, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) ifft_pair_kernel(const cplx<T>* __restrict__ bvec, cplx<T>* __restrict__ U,
                                                              const T* __restrict__ dec, const cplx<T>* __restrict__ tw,
-                                                             int p, int L, int P2, int ldu) {
+                                                             int p, int L, int P2, int ldu, T even, T halfInv) {
     constexpr int M = 1 << LOGM, R = ip::out_radix(LOGM, NT);
     constexpr int H = M >> 1;
     extern __shared__ unsigned char smem_raw[];
@@ -48,11 +51,11 @@ __global__ void __launch_bounds__(NT, MINB) ifft_pair_kernel(const cplx<T>* __re
     const bool has1 = m1 <= L;
     const cplx<T>* in0 = bvec + ((int64_t)b * (p + 1) + m0) * 2 * P2;
     const cplx<T>* in1 = in0 + 2 * P2;
-    // c0_j + c1_j (lower half) or c0_j - c1_j (upper half), c1 = conj(i/2) v deconvolved
+    // even c0_j + c1_j (lower half) or even c0_j - c1_j (upper half), c1 = conj(i/2) v deconvolved
     auto both = [&](int j, T sg) {
         const int o = (j & 1) * P2 + (j >> 1);
         const T d = dec[j];
-        cplx<T> v = scale(in0[o], d);
+        cplx<T> v = scale(in0[o], even * d);
         if (has1) {
             const cplx<T> w = in1[o];
             const T hd = sg * T(0.5) * d;
@@ -63,7 +66,7 @@ __global__ void __launch_bounds__(NT, MINB) ifft_pair_kernel(const cplx<T>* __re
     // j = t + r M/16, t < M/16: r <= 4 can hold j <= p = M/4, r >= 12 j >= M - p
     auto ld = [&](int j, int r) {
         if (r > 4 && r < 12) return mk<T>(T(0), T(0));
-        if (j == 0) return scale(in0[0], T(2) * dec[0]);
+        if (j == 0) return scale(in0[0], T(2) * even * dec[0]);
         if (j <= p) return both(j, T(1));
         if (j >= M - p) return both(M - j, T(-1));
         return mk<T>(T(0), T(0));
@@ -75,7 +78,7 @@ __global__ void __launch_bounds__(NT, MINB) ifft_pair_kernel(const cplx<T>* __re
     cplx<T>* out1 = out0 + ldu;
     for (int t = tid; t <= H; t += NT) {
         const cplx<T> z = buf[ip::slot(t)], zr = buf[ip::slot((M - t) & (M - 1))];
-        cplx<T> v0 = scale(add(z, zr), T(0.5));
+        cplx<T> v0 = scale(add(z, zr), halfInv);
         if (t == 0 || t == H) v0 = scale(v0, T(0.5));
         out0[t] = v0;
         if (has1) out1[t] = scale(sub(z, zr), T(0.5));
@@ -209,7 +212,7 @@ __global__ void __launch_bounds__(256, 2) interp_rb_kernel(const cplx<float>* __
 // Returns false at nside 2 (16 grid points) and for small batches of small grids; the
 // caller then runs nufft_adj_kernel.
 template <class T>
-bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
+bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s, T even) {
     const auto& g = P->g;
     const auto& t = P->t;
     constexpr int EW = 12, DM = 4, NS = 3;
@@ -227,7 +230,7 @@ bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
     auto run1 = [&](auto kern, int threads) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
         kern<<<grid1, threads, smem1, s>>>((const cplx<T>*)P->bvec, (cplx<T>*)P->U, (const T*)t.dec,
-                                           (const cplx<T>*)t.twx, g.p, g.L, g.P2, P->ldu);
+                                           (const cplx<T>*)t.twx, g.p, g.L, g.P2, P->ldu, even, T(0.5) / even);
     };
     // the shapes of the analysis' grid FFT (k_nufft.cu)
     if (logM == 5) run1(ifft_pair_kernel<T, 5, 32, 1>, 32);
@@ -261,7 +264,7 @@ bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s) {
     return true;
 }
 
-template bool launch_nufft2<float>(const hpx_plan_s*, cudaStream_t);
-template bool launch_nufft2<double>(const hpx_plan_s*, cudaStream_t);
+template bool launch_nufft2<float>(const hpx_plan_s*, cudaStream_t, float);
+template bool launch_nufft2<double>(const hpx_plan_s*, cudaStream_t, double);
 
 }  // namespace hpx

@@ -283,7 +283,8 @@ __host__ __device__ inline int64_t tc_elem(int rp, int r, int k) {
 // adjoint under the real-map inner product, 1: under the plain Euclidean one)
 // type-2 latitude NUFFT of the adjoint and the synthesis in two kernels
 // (k_nufft2.cu); false where they do not apply (then nufft_adj_kernel runs)
-template <class T> bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s);
+// even: power of two that brings the coefficients of the even orders to the size of the odd ones'
+template <class T> bool launch_nufft2(const hpx_plan_s* P, cudaStream_t s, T even);
 template <class T> void launch_adjoint(const hpx_plan_s* P, const T* alm, T* maps, cudaStream_t s, T wpos = T(2));
 // ev: NULL, or kStages + 1 events recorded around its stages (profiling)
 template <class T>
