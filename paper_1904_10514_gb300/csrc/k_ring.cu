@@ -424,9 +424,10 @@ void launch_ring_fft(const hpx_plan_s* P, const T* maps, cudaStream_t s, T ew, i
         // ring pairs per SM.  The warps win where the ring pairs are more than twice what
         // fits at once (Nside 64, 32 maps: 20 against 28 us FP32, 200 against 234 FP64; 4
         // maps FP64: 8 us slower, 8 maps: 4 us faster; FP32 8 maps: 2 us slower, 16 maps:
-        // 2 us faster), and at Nside 2 and 4 (6.9 against 8.1 us)
+        // 2 us faster), and at Nside 2 and 4 in
+        // FP32 (6.9 against 8.1 us; FP64 9.9 against 9.6)
         const int fit = P->sms * (sizeof(T) == 4 ? 6 : 3);
-        const bool warps = N <= 32 || (N <= 512 && (int64_t)g.B * nrings > 2 * fit);
+        const bool warps = (sizeof(T) == 4 && N <= 32) || (N <= 512 && (int64_t)g.B * nrings > 2 * fit);
         const int threads = warps ? 32 : kRingShortThreads;
         const size_t smem = (size_t)(warps ? N + N / 16 : ring_short_slots(N)) * sizeof(cplx<T>);
         auto kern = warps ? ring_fft_kernel<T, 16, 0> : ring_fft_kernel<T, 16, kRingShortThreads>;
