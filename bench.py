@@ -32,13 +32,13 @@ NSIDE, LMAX, BATCH = 1024, 2048, 32
 WORKLOAD = "bench_nside1024x32"
 MEASURED = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # measured DRAM traffic (read + written, GB) / algorithmic bytes of each stage at Nside 512, 32 maps
-# (ncu --set full captures of the stage's launches; the summaries are in profiles/).  Dirty lines
-# still in L2 when a kernel ends are not counted, so a ratio can fall below 1.
+# (one ncu capture, profiles/ncu_stages_nside512x32.md).  Dirty lines still in L2 when a kernel ends
+# are not counted, so a ratio can fall below 1.
 TRAFFIC_OVER_ALGORITHMIC = {
-    "fused_fsht": (1.4479 + 0.1249) / 1.4828,                      # fused_tc_ws_kernel, packed b
-    "ring_fft": (0.11342 + 0.08983 + 0.31140 + 0.34239) / 0.94031,  # ring stage
-    "lat_fft": (0.53804 + 0.24894) / 0.80688,                      # grid FFT, packed b
-    "spread": (0.54846 + 0.49414) / 1.07532,                       # spread_rb_kernel
+    "fused_fsht": (1.44789 + 0.12533) / 1.4828,                     # fused_tc_ws_kernel<0>, packed b
+    "ring_fft": (0.11341 + 0.09417 + 0.31128 + 0.34558) / 0.94031,  # ring_ip_kernel + ring_fft_kernel
+    "lat_fft": (0.53804 + 0.24934) / 0.80688,                       # lat_fft_pair_kernel, packed b
+    "spread": (0.54809 + 0.49525) / 1.07532,                        # spread_rb_kernel
 }
 # forms of the FP32 run-time sweep kernel (hpx_plan_tuning)
 SWEEP_FORMS = ["complex lanes, 32 stages per pass", "complex lanes, 16 stages per pass",

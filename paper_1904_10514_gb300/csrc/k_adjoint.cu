@@ -389,7 +389,7 @@ __global__ void pole_adj_kernel(const cplx<T>* __restrict__ Y, T* __restrict__ m
 //     m = k - q n, so a rotation is made once per k; phi0 = 0: none.
 // Bound by the shared-memory passes and, in the synthesis, the reads of the aliased
 // orders.  Synthesis of 32 maps at Nside 512: 1266 us (plain and short rings, radix-2
-// passes) + 321 us (Bluestein rings, whole convolutions) before, 487 + 257 us now.
+// passes) + 321 us (Bluestein rings, whole convolutions) before, 728 us now.
 template <class T, bool SYN>
 struct BackInput {
     const cplx<T>*rowN, *rowS, *ph;

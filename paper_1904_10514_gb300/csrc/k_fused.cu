@@ -428,7 +428,7 @@ __device__ __forceinline__ cplx<T> weighted(cplx<T> v, int m, int p, CoefWeights
 // on: the last blocks of the grid take that k, a warp each, instead of a tile of one.
 // FP32 is bound by the latency of the tiles' loads, FP64 by the FP64 pipe.  6 maps,
 // Nside 256, lmax 400 (synthesis): 96 us as matrix-matrix tiles, 65 us with a tile for
-// the last k, now 54 us.
+// the last k, now 48 us (in groups of 32 rows).
 template <class T, int NB, bool QUAD>
 __global__ void __launch_bounds__(128) operator_cols_kernel(const T* __restrict__ M, const int64_t* __restrict__ moff,
                                                             const cplx<T>* __restrict__ alm,

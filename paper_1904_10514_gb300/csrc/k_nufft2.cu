@@ -12,7 +12,7 @@
 //
 // Two kernels, the transposes of lat_fft_pair and spread_rb.  6 maps, Nside 256, lmax
 // 400: 163 us as one radix-2 FFT and one strided column per block (the form left for
-// Nside 2), now 12 + 25 us.
+// small grids in few columns), now 12 + 25 us.
 //   ifft_pair_kernel  one block per pair of orders (m even, m + 1) and map:
 //       the transposed truncation puts the deconvolved coefficients c_j on j = 0..p;
 //       the transposed symmetric extension of the half grid folds them into the
